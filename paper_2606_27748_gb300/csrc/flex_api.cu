@@ -139,7 +139,7 @@ int flex_linattn_fwd(const flex_shape* shape, const void* q, const void* k, cons
         return count(3, flex::launch_tc_nc(p, q, k, v, W1, W2, kw, out, den,
                                            (char*)ws + header_bytes(), status, s));
     }
-    if (flex::simt_pick_chunk_fwd(p) == 0) return FLEX_EUNSUPPORTED;
+    if (!flex::simt_fwd_supported(p)) return FLEX_EUNSUPPORTED;
     return count(1, flex::launch_simt_fwd(p, q, k, v, W1, W2, tau, out, den, s));
 }
 
@@ -169,7 +169,7 @@ int flex_linattn_bwd(const flex_shape* shape, const void* q, const void* k, cons
                      flex::launch_tc_bwd(p, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv,
                                          dW1, dW2, dtau, scratch, &((flex::WsHeader*)ws)->status,
                                          s));
-    if (flex::simt_pick_chunk_bwd(p) == 0) return FLEX_EUNSUPPORTED;
+    if (!flex::simt_bwd_supported(p)) return FLEX_EUNSUPPORTED;
     return count(2, flex::launch_simt_bwd(p, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv,
                                           dW1, dW2, dtau, scratch, s));
 }

@@ -38,10 +38,8 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 void add_launches(int n);
 
 // ---- SIMT path (fp32 arithmetic; any supported dtype) --------------------------------
-size_t simt_fwd_smem_bytes(const Problem& p, int chunk);
-size_t simt_bwd_smem_bytes(const Problem& p, int chunk);
-int simt_pick_chunk_fwd(const Problem& p);   // 0 if nothing fits
-int simt_pick_chunk_bwd(const Problem& p);
+bool simt_fwd_supported(const Problem& p);  // sizes the fp32 kernels take
+bool simt_bwd_supported(const Problem& p);
 size_t simt_bwd_ws_bytes(const Problem& p);
 
 cudaError_t launch_featmap(const Problem& p, const void* x, const float* W1, const float* W2,

@@ -105,7 +105,7 @@ extern "C" int flex_linattn_bwd_noalloc(const flex_shape* shape, const void* q, 
     p.bf16 = shape->dtype == FLEX_BF16;
     p.nonstat = W2 != nullptr;
     p.causal = causal ? 1 : 0;
-    if (flex::simt_pick_chunk_bwd(p) == 0) return FLEX_EUNSUPPORTED;
+    if (!flex::simt_bwd_supported(p)) return FLEX_EUNSUPPORTED;
     // The fixed scratch must hold every partial; larger problems are refused.
     if (flex::simt_bwd_ws_bytes(p) > kNoallocScratchFloats * sizeof(float))
         return FLEX_EWORKSPACE;

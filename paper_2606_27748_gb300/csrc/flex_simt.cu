@@ -1,11 +1,11 @@
-// SIMT kernels: fp32 arithmetic on the CUDA cores, one CTA per (b, h) sequence.
+// SIMT kernels: fp32 arithmetic on the CUDA cores.
 //
 // These kernels serve the fp32 storage type, whose tolerance (relative L2 <= 1e-4)
-// excludes bf16/tf32 tensor-core operands, and the feature-map entry point.  They run the
-// chunked form of Eq. (linear att): inside a chunk of C tokens the masked C x C kernel
-// matrix phi(Q) phi(K)^T is applied directly, across chunks the running state
-// S = sum phi(k) v^T and z = sum phi(k) carries the prefix.  z rides in S as column d
-// (v is extended with a constant 1), so numerator and denominator share every product.
+// excludes bf16/tf32 tensor-core operands, bf16 shapes off the tensor-core path, the
+// feature-map entry point and the workspace-free backward.  They run the chunked form of
+// Eq. (linear att): inside a chunk of T tokens the masked T x T kernel matrix
+// phi(Q) phi(K)^T is applied directly, across chunks the running state
+// S = sum phi(k) v^T, z = sum phi(k) carries the prefix.
 //
 // Inside the attention kernels the features are unscaled, phi' = [cos, sin] (times cos w
 // for the nonstationary map): the global factor M^{-1/2} of Eq. phi_n / phi_non cancels in
@@ -22,11 +22,16 @@
 
 #include <algorithm>
 
+#include "tc_common.cuh"
+#include "tc_util.cuh"
+
 namespace flex {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMaxDwPerThread = 64;  // Mc * d <= kThreads * 64
+constexpr int kMaxCluster = 8;   // CTAs that share one sequence
+constexpr int kMaxT = 64;        // tokens per chunk
+constexpr int kMaxMG = 32;       // frequencies per group (64 features)
 
 __device__ __forceinline__ float load_act(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ float load_act(const __nv_bfloat16* p, size_t i)
@@ -38,60 +43,26 @@ __device__ __forceinline__ void store_act(__nv_bfloat16* p, size_t i, float x)
 {
     p[i] = __float2bfloat16_rn(x);
 }
-
-// Projection rows of one head into shared memory, row stride d + 1:
-// stationary: W1 (M rows); nonstationary: U = (W1+W2)/2 then V = (W1-W2)/2 (2M rows).
-__device__ void load_projection(const Problem& p, const float* W1, const float* W2, int h,
-                                float* W)
+// Four consecutive elements (d % 4 == 0 and 16-byte aligned tensors: aligned accesses).
+__device__ __forceinline__ float4 load_act4(const float* p, size_t i)
 {
-    const int d = p.d, M = p.M;
-    const float* w1 = W1 + (size_t)h * M * d;
-    const float* w2 = p.nonstat ? W2 + (size_t)h * M * d : nullptr;
-    for (int idx = threadIdx.x; idx < M * d; idx += blockDim.x) {
-        int m = idx / d, i = idx % d;
-        if (!p.nonstat) {
-            W[m * (d + 1) + i] = w1[idx];
-        } else {
-            W[m * (d + 1) + i] = 0.5f * (w1[idx] + w2[idx]);
-            W[(M + m) * (d + 1) + i] = 0.5f * (w1[idx] - w2[idx]);
-        }
-    }
+    return *reinterpret_cast<const float4*>(p + i);
 }
-
-template <typename T>
-__device__ void load_rows(const T* src, size_t base, int rows, int d, float* dst, int stride)
+__device__ __forceinline__ float4 load_act4(const __nv_bfloat16* p, size_t i)
 {
-    for (int idx = threadIdx.x; idx < rows * d; idx += blockDim.x) {
-        int t = idx / d, i = idx % d;
-        dst[t * stride + i] = load_act(src, base + (size_t)t * d + i);
-    }
+    const uint2 u = *reinterpret_cast<const uint2*>(p + i);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
 }
-
-// Unscaled features of `rows` vectors X[t][0..d) into P[t][0..2M), row stride pstride.
-__device__ void features(const Problem& p, const float* X, int rows, const float* W, float* P,
-                         int pstride)
+__device__ __forceinline__ void store_act4(float* p, size_t i, float4 x)
 {
-    const int d = p.d, M = p.M;
-    for (int idx = threadIdx.x; idx < rows * M; idx += blockDim.x) {
-        int t = idx / M, m = idx % M;
-        const float* x = X + t * d;
-        const float* wa = W + m * (d + 1);
-        float a = 0.f;
-        for (int i = 0; i < d; ++i) a = fmaf(x[i], wa[i], a);
-        float sa, ca;
-        sincosf(a, &sa, &ca);
-        if (!p.nonstat) {
-            P[t * pstride + m] = ca;
-            P[t * pstride + M + m] = sa;
-        } else {
-            const float* wb = W + (M + m) * (d + 1);
-            float w = 0.f;
-            for (int i = 0; i < d; ++i) w = fmaf(x[i], wb[i], w);
-            float cw = cosf(w);
-            P[t * pstride + m] = ca * cw;
-            P[t * pstride + M + m] = sa * cw;
-        }
-    }
+    *reinterpret_cast<float4*>(p + i) = x;
+}
+__device__ __forceinline__ void store_act4(__nv_bfloat16* p, size_t i, float4 x)
+{
+    const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
+    *reinterpret_cast<uint2*>(p + i) = make_uint2(*reinterpret_cast<const uint32_t*>(&a),
+                                                  *reinterpret_cast<const uint32_t*>(&b));
 }
 
 // ------------------------------------------------------------------------------------
@@ -129,252 +100,594 @@ __global__ void featmap_kernel(Problem p, const T* x, const float* W1, const flo
 }
 
 // ------------------------------------------------------------------------------------
-// Forward.
+// Attention: plan, tile products, features.
 // ------------------------------------------------------------------------------------
-// [v_j | 1] -> [w_j v_j | w_j] for the key rows of a chunk, w_j = exp(|k_j|^2 itau).
-__device__ void weight_keys(const float* Xk, int rows, int d, float itau, float* Vx)
-{
-    for (int j = threadIdx.x; j < rows; j += blockDim.x) {
-        float n2 = 0.f;
-        for (int e = 0; e < d; ++e) n2 = fmaf(Xk[j * d + e], Xk[j * d + e], n2);
-        const float w = expf(n2 * itau);
-        for (int e = 0; e < d; ++e) Vx[j * (d + 1) + e] *= w;
-        Vx[j * (d + 1) + d] = w;
-    }
-}
-
-struct FwdLayout {
-    size_t W, S, Xq, Xk, Vx, Pq, Pk, A, O, total;  // offsets in floats
+// One cluster of CL CTAs per (b, h) sequence; CTA r owns a contiguous range of chunks of
+// T tokens.  When the sequence is split (or not causal) each CTA first sums its own range's
+// state; the cluster then turns those into what each range starts from (the total, or the
+// exclusive prefix or suffix) through distributed shared memory, so no workspace and no
+// second launch is needed.  Frequencies are taken MG at a time: a group has F = 2 MG
+// features, feature columns 4x..4x+3 being cos, sin of frequency 2x and cos, sin of 2x + 1,
+// so the thread that projects two frequencies writes (and later differentiates) its own
+// four features.  All products run as 4 x 4 register tiles over shared-memory operands: per
+// four k 8 float4 loads feed 64 fmas, so the fma pipe and not the shared-memory port is the
+// limit (one output per thread took two loads per fma), and a short sequence spreads over
+// up to 8 SMs instead of one.  Measured on GB300 against one CTA per sequence with
+// one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 23 us, bf16 n B32 H4
+// N1024 d32 M16 477 -> 104 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
+// 8.58 -> 0.51 ms (6.7 of the 78 TFLOP/s fp32 peak: per chunk the products run between
+// barriers with one backward CTA per SM, so load latency and the barriers bound it).
+struct Plan {
+    int T;              // tokens per chunk (a multiple of 8, at most kMaxT)
+    int ng, MG;         // frequency groups; frequencies per group (a multiple of 4)
+    int CT;             // feature column tiles of a group, MG / 2
+    int F;              // features of a group, 2 MG
+    int KP;             // projection rows of a group: MG (s), 2 MG (n: u and w)
+    int pd, pp, pa;     // pitches (floats) of rows of d, of features, of T x T blocks
+    int wres;           // every group's projection rows stay in shared memory
+    int CL;             // CTAs per sequence
+    int S, W, dW, Xq, Xk, V, G, Pq, Pk, A, red, total;  // offsets (floats)
 };
 
-__host__ __device__ inline FwdLayout fwd_layout(const Problem& p, int C)
+// Row of column tile x, column c in arrays whose rows are read four at a time by
+// neighbouring x (projection rows, state rows): c CT + x, so that 16 lanes with
+// consecutive x read consecutive rows (pitch 4 mod 32: no bank conflicts).
+__device__ __forceinline__ int prow(const Plan& L, int feature)
 {
-    const int d = p.d, D = 2 * p.M, Mc = p.nonstat ? 2 * p.M : p.M;
-    FwdLayout L;
-    size_t o = 0;
-    L.W = o;  o += (size_t)Mc * (d + 1);
-    L.S = o;  o += (size_t)D * (d + 1);
-    L.Xq = o; o += (size_t)C * d;
-    L.Xk = o; o += (size_t)C * d;
-    L.Vx = o; o += (size_t)C * (d + 1);
-    L.Pq = o; o += (size_t)C * (D + 1);
-    L.Pk = o; o += (size_t)C * (D + 1);
-    L.A = o;  o += (size_t)C * C;
-    L.O = o;  o += (size_t)C * (d + 1);
-    L.total = o;
-    return L;
+    return (feature & 3) * L.CT + (feature >> 2);
 }
 
-// S[f][e] += sum_{j < rows} Pk[j][f] * Vx[j][e]
-__device__ void state_update(const float* Pk, const float* Vx, int rows, int D, int d,
-                             float* S)
+// acc[r][c] += sum_k a[r pa + k] b[c pb + k], K a multiple of 4.
+template <int NC>
+__device__ __forceinline__ void mm_nt(const float* a, int pa, const float* b, int pb, int K,
+                                      float (&acc)[4][NC])
 {
-    for (int idx = threadIdx.x; idx < D * (d + 1); idx += blockDim.x) {
-        int f = idx / (d + 1), e = idx % (d + 1);
-        float acc = S[idx];
-        for (int j = 0; j < rows; ++j) acc = fmaf(Pk[j * (D + 1) + f], Vx[j * (d + 1) + e], acc);
-        S[idx] = acc;
+    for (int k = 0; k < K; k += 4) {
+        float4 x[4], y[NC];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(a + r * pa + k);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) y[c] = *reinterpret_cast<const float4*>(b + c * pb + k);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                acc[r][c] = fmaf(x[r].x, y[c].x, acc[r][c]);
+                acc[r][c] = fmaf(x[r].y, y[c].y, acc[r][c]);
+                acc[r][c] = fmaf(x[r].z, y[c].z, acc[r][c]);
+                acc[r][c] = fmaf(x[r].w, y[c].w, acc[r][c]);
+            }
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) simt_fwd_kernel(Problem p, int C, const T* q,
-                                                            const T* k, const T* v,
-                                                            const float* W1, const float* W2,
-                                                            const float* tau, T* out,
-                                                            float* den)
+// acc[r][c] += sum_k a[r pa + k] b[row(k)][c]; the rows of k..k+3 lie at o0..o3 from b,
+// which advances by `step` every four (plain rows or the permuted rows of prow).
+__device__ __forceinline__ void mm_nn(const float* a, int pa, const float* b, int o1, int o2,
+                                      int o3, int step, int K, float (&acc)[4][4])
 {
-    extern __shared__ float sm[];
-    const int d = p.d, D = 2 * p.M, N = p.N;
-    const int bh = blockIdx.x, h = bh % p.H;
-    const size_t base = (size_t)bh * N * d;
-    const FwdLayout L = fwd_layout(p, C);
-    float *W = sm + L.W, *S = sm + L.S, *Xq = sm + L.Xq, *Xk = sm + L.Xk, *Vx = sm + L.Vx;
-    float *Pq = sm + L.Pq, *Pk = sm + L.Pk, *A = sm + L.A, *O = sm + L.O;
-    const float inv_m = 1.0f / (float)p.M;
-    const float itau = tau ? expf(-tau[h]) : 0.f;
+    for (int k = 0; k < K; k += 4, b += step) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(a + r * pa + k);
+        y[0] = *reinterpret_cast<const float4*>(b);
+        y[1] = *reinterpret_cast<const float4*>(b + o1);
+        y[2] = *reinterpret_cast<const float4*>(b + o2);
+        y[3] = *reinterpret_cast<const float4*>(b + o3);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float xr[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                acc[r][0] = fmaf(xr[kk], y[kk].x, acc[r][0]);
+                acc[r][1] = fmaf(xr[kk], y[kk].y, acc[r][1]);
+                acc[r][2] = fmaf(xr[kk], y[kk].z, acc[r][2]);
+                acc[r][3] = fmaf(xr[kk], y[kk].w, acc[r][3]);
+            }
+        }
+    }
+}
 
-    load_projection(p, W1, W2, h, W);
-    for (int idx = threadIdx.x; idx < D * (d + 1); idx += blockDim.x) S[idx] = 0.f;
-    for (int idx = threadIdx.x; idx < C; idx += blockDim.x) Vx[idx * (d + 1) + d] = 1.f;
+// acc[r][c] += sum_k a[k pa + r] b[k pb + c], K a multiple of 4.
+__device__ __forceinline__ void mm_tn(const float* a, int pa, const float* b, int pb, int K,
+                                      float (&acc)[4][4])
+{
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        const float4 x = *reinterpret_cast<const float4*>(a + k * pa);
+        const float4 y = *reinterpret_cast<const float4*>(b + k * pb);
+        const float xr[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            acc[r][0] = fmaf(xr[r], y.x, acc[r][0]);
+            acc[r][1] = fmaf(xr[r], y.y, acc[r][1]);
+            acc[r][2] = fmaf(xr[r], y.z, acc[r][2]);
+            acc[r][3] = fmaf(xr[r], y.w, acc[r][3]);
+        }
+    }
+}
+
+template <int R, int C>
+__device__ __forceinline__ void zero(float (&acc)[R][C])
+{
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[r][c] = 0.f;
+}
+
+// Projection rows of group g of one head.  s: column c (0, 1) of tile x is frequency
+// 2x + c; n: columns 0..3 are u, w of frequency 2x, then u, w of 2x + 1, with
+// U = (W1+W2)/2, V = (W1-W2)/2.  Rows past M are zero.
+template <bool NS>
+__device__ void stage_projection(const Problem& p, const Plan& L, const float* W1,
+                                 const float* W2, int h, int g, float* W)
+{
+    const int d = p.d, dq = d / 4;
+    for (int idx = threadIdx.x; idx < L.KP * dq; idx += kThreads) {
+        const int row = idx / dq, e = 4 * (idx % dq), c = row / L.CT, x = row % L.CT;
+        const int f = g * L.MG + 2 * x + (NS ? c >> 1 : c);
+        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (f < p.M) {
+            const size_t o = ((size_t)h * p.M + f) * d + e;
+            w = *reinterpret_cast<const float4*>(W1 + o);
+            if (NS) {
+                const float4 w2 = *reinterpret_cast<const float4*>(W2 + o);
+                const float s = (c & 1) ? -1.f : 1.f;
+                w = make_float4(0.5f * (w.x + s * w2.x), 0.5f * (w.y + s * w2.y),
+                                0.5f * (w.z + s * w2.z), 0.5f * (w.w + s * w2.w));
+            }
+        }
+        *reinterpret_cast<float4*>(W + row * L.pd + e) = w;
+    }
+}
+
+// Rows of a chunk, zero from row CL on.
+template <typename T>
+__device__ void load_rows(const T* src, size_t base, int rows, int d, float* dst, int pitch,
+                          int nrows)
+{
+    const int dq = d / 4;
+    for (int idx = threadIdx.x; idx < nrows * dq; idx += kThreads) {
+        const int t = idx / dq, e = 4 * (idx % dq);
+        *reinterpret_cast<float4*>(dst + t * pitch + e) =
+            t < rows ? load_act4(src, base + (size_t)t * d + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// Column d of the value rows: 1 for the chunk's keys, 0 past its end.
+__device__ __forceinline__ void unit_weights(const Plan& L, int d, int rows, float* V)
+{
+    if (threadIdx.x < L.T) V[threadIdx.x * L.pd + d] = threadIdx.x < rows ? 1.f : 0.f;
+}
+
+// Prefactor: [v_j | 1] -> [w_j v_j | w_j], w_j = exp(|k_j|^2 itau); |k_j|^2 to kn2.  Four
+// lanes per row.
+__device__ __forceinline__ void weight_keys(const Plan& L, const float* Xk, int rows, int d,
+                                            float itau, float* V, float* kn2)
+{
+    if (threadIdx.x >= 4 * L.T) return;
+    const int j = threadIdx.x >> 2, part = threadIdx.x & 3;
+    float n2 = 0.f;
+    for (int e = 4 * part; e < d; e += 16) {
+        const float4 x = *reinterpret_cast<const float4*>(Xk + j * L.pd + e);
+        n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, n2))));
+    }
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+    const float w = j < rows ? expf(n2 * itau) : 0.f;
+    for (int e = 4 * part; e < d; e += 16) {
+        float4* v = reinterpret_cast<float4*>(V + j * L.pd + e);
+        if (j < rows) *v = make_float4(w * v->x, w * v->y, w * v->z, w * v->w);
+    }
+    if (part == 0) {
+        V[j * L.pd + d] = w;
+        kn2[j] = n2;
+    }
+}
+
+// This thread's place in the feature tile of a chunk: rows 4y..4y+3, column tile x.
+struct Place {
+    int y, x;
+    bool on;
+};
+
+// Unscaled features of this thread's 4 rows x 2 frequencies: pf = (cos, sin) of each (times
+// cos w), zero for rows from `rows` on and frequencies past M.  With CHAIN also
+// qf = (cos u sin w, sin u sin w) (n), for the derivative with respect to w.
+template <bool NS, bool CHAIN>
+__device__ __forceinline__ void features(const Problem& p, const Plan& L, const Place& f,
+                                         const float* X, int rows, const float* W, int g,
+                                         float (&pf)[4][4], float (&qf)[4][4])
+{
+    constexpr int NC = NS ? 4 : 2;
+    float a[4][NC];
+    zero(a);
+    mm_nt<NC>(X + 4 * f.y * L.pd, L.pd, W + f.x * L.pd, L.CT * L.pd, p.d, a);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const bool ok = 4 * f.y + r < rows && g * L.MG + 2 * f.x + i < p.M;
+            float s, c, sw = 0.f, cw = 1.f;
+            sincosf(a[r][NS ? 2 * i : i], &s, &c);
+            if (NS) {
+                if (CHAIN)
+                    sincosf(a[r][NC / 2 * i + (NS ? 1 : 0)], &sw, &cw);
+                else
+                    cw = cosf(a[r][NC / 2 * i + (NS ? 1 : 0)]);
+            }
+            pf[r][2 * i] = ok ? (NS ? c * cw : c) : 0.f;
+            pf[r][2 * i + 1] = ok ? (NS ? s * cw : s) : 0.f;
+            if (NS && CHAIN) {
+                qf[r][2 * i] = ok ? c * sw : 0.f;
+                qf[r][2 * i + 1] = ok ? s * sw : 0.f;
+            }
+        }
+}
+__device__ __forceinline__ void store_tile(float* P, int pitch, const Place& f, const float (&v)[4][4])
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        *reinterpret_cast<float4*>(P + (4 * f.y + r) * pitch + 4 * f.x) =
+            make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+}
+
+// State of one group: S[prow(f)][e] += sum_j P[j][f] Y[j][e] and, in column d, the sum
+// weighted by Y[j][d] (z, or r from G = [g | c]).
+__device__ __forceinline__ void state_update(const Plan& L, int d, const float* P, const float* Y,
+                                             float* S)
+{
+    const int dq = d / 4;
+    for (int id = threadIdx.x; id < L.CT * dq; id += kThreads) {
+        const int x = id / dq, e = 4 * (id % dq);
+        float acc[4][4];
+        zero(acc);
+        mm_tn(P + 4 * x, L.pp, Y + e, L.pd, L.T, acc);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float4* s = reinterpret_cast<float4*>(S + (r * L.CT + x) * L.pd + e);
+            *s = make_float4(s->x + acc[r][0], s->y + acc[r][1], s->z + acc[r][2],
+                             s->w + acc[r][3]);
+        }
+    }
+    if (threadIdx.x < 4 * L.F) {  // four lanes per feature (4 F is a multiple of 32)
+        const int f = threadIdx.x >> 2;
+        float z = 0.f;
+        for (int j = threadIdx.x & 3; j < L.T; j += 4) z = fmaf(P[j * L.pp + f], Y[j * L.pd + d], z);
+        z += __shfl_xor_sync(0xffffffffu, z, 1);
+        z += __shfl_xor_sync(0xffffffffu, z, 2);
+        if ((threadIdx.x & 3) == 0) S[prow(L, f) * L.pd + d] += z;
+    }
+}
+
+// The ranges' states, summed over the cluster in rank order: every CTA's S becomes the
+// total, or the sum over the lower (prefix) or higher (suffix) ranks.  Each CTA owns a slice
+// of the state: it alone reads and rewrites that slice in all CTAs, so it works in place.
+enum { kTotal, kPrefix, kSuffix };
+__device__ void exchange_state(float* S, int n, int CL, int mode)
+{
+    tc::cluster_sync();
+    const uint32_t base = tc::smem_u32(S);
+    const int rank = (int)tc::cluster_rank();
+    for (int i = rank * kThreads + threadIdx.x; i < n / 4; i += CL * kThreads) {
+        float4 v[kMaxCluster];
+#pragma unroll
+        for (int r = 0; r < kMaxCluster; ++r)
+            if (r < CL) v[r] = tc::ld_cluster_v4(tc::mapa(base + 16 * i, r));
+        float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto add = [&](const float4& x) {
+            run = make_float4(run.x + x.x, run.y + x.y, run.z + x.z, run.w + x.w);
+        };
+        if (mode == kTotal)
+#pragma unroll
+            for (int r = 0; r < kMaxCluster; ++r)
+                if (r < CL) add(v[r]);
+#pragma unroll
+        for (int o = 0; o < kMaxCluster; ++o) {
+            const int r = mode == kSuffix ? kMaxCluster - 1 - o : o;
+            if (r < CL) {
+                tc::st_cluster_v4(tc::mapa(base + 16 * i, r), run.x, run.y, run.z, run.w);
+                if (mode != kTotal) {
+                    float4 x = v[0];
+#pragma unroll
+                    for (int s = 1; s < kMaxCluster; ++s)
+                        if (s == r) x = v[s];
+                    add(x);
+                }
+            }
+        }
+    }
+    tc::cluster_sync();
+}
+
+// Chunks [cb, ce) of this CTA.
+__device__ __forceinline__ void chunk_range(const Plan& L, int N, int rank, int* cb, int* ce)
+{
+    const int nch = (N + L.T - 1) / L.T, per = (nch + L.CL - 1) / L.CL;
+    *cb = min(nch, rank * per);
+    *ce = min(nch, *cb + per);
+}
+
+// ------------------------------------------------------------------------------------
+// Forward.
+// ------------------------------------------------------------------------------------
+template <typename T, bool NS, int ND>
+__global__ void __launch_bounds__(kThreads, 2)
+    simt_fwd_kernel(Problem p, Plan L, const T* q, const T* k, const T* v, const float* W1,
+                    const float* W2, const float* tau, T* out, float* den)
+{
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
+    const int tid = threadIdx.x, d = p.d, N = p.N, dq = d / 4;
+    const int rank = L.CL > 1 ? (int)tc::cluster_rank() : 0;
+    const int bh = blockIdx.x / L.CL, h = bh % p.H;
+    const size_t base = (size_t)bh * N * d;
+    float *S = sm + L.S, *Xq = sm + L.Xq, *Xk = sm + L.Xk, *V = sm + L.V;
+    float *Pq = sm + L.Pq, *Pk = sm + L.Pk, *A = sm + L.A, *red = sm + L.red;
+    const float inv_m = 1.0f / (float)p.M, itau = tau ? expf(-tau[h]) : 0.f;
+    const int gS = L.F * L.pd, gW = L.wres ? L.KP * L.pd : 0;  // strides of a group
+    const Place f = {tid / L.CT, tid % L.CT, tid / L.CT < L.T / 4};
+    const int TT = L.T / 4, ay = tid / TT, ax = tid % TT;  // T x T tile: rows 4 ay + r, cols ax + TT c
+    const bool a_on = ay < TT;
+    int cb, ce;
+    chunk_range(L, N, rank, &cb, &ce);
+
+    if (L.wres)
+        for (int g = 0; g < L.ng; ++g)
+            stage_projection<NS>(p, L, W1, W2, h, g, sm + L.W + g * gW);
+    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
+
+    if (!p.causal || L.CL > 1) {  // this range's sums
+        for (int c = cb; c < ce; ++c) {
+            const int t0 = c * L.T, rows = min(L.T, N - t0);
+            load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
+            load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+            unit_weights(L, d, rows, V);
+            __syncthreads();
+            if (tau) weight_keys(L, Xk, rows, d, itau, V, red);
+            for (int g = 0; g < L.ng; ++g) {
+                float* W = sm + L.W + g * gW;
+                if (!L.wres) {
+                    stage_projection<NS>(p, L, W1, W2, h, g, W);
+                    __syncthreads();
+                }
+                if (f.on) {
+                    float pf[4][4], qf[4][4];
+                    features<NS, false>(p, L, f, Xk, rows, W, g, pf, qf);
+                    store_tile(Pk, L.pp, f, pf);
+                }
+                __syncthreads();
+                state_update(L, d, Pk, V, S + g * gS);
+                __syncthreads();
+            }
+        }
+        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
+    }
     __syncthreads();
 
-    if (!p.causal) {  // totals S, z over the whole sequence first
-        for (int t0 = 0; t0 < N; t0 += C) {
-            const int CL = min(C, N - t0);
-            load_rows(k, base + (size_t)t0 * d, CL, d, Xk, d);
-            load_rows(v, base + (size_t)t0 * d, CL, d, Vx, d + 1);
-            __syncthreads();
-            if (tau) weight_keys(Xk, CL, d, itau, Vx);
-            features(p, Xk, CL, W, Pk, D + 1);
-            __syncthreads();
-            state_update(Pk, Vx, CL, D, d, S);
-            __syncthreads();
-        }
-    }
-    for (int t0 = 0; t0 < N; t0 += C) {
-        const int CL = min(C, N - t0);
-        load_rows(q, base + (size_t)t0 * d, CL, d, Xq, d);
+    for (int c = cb; c < ce; ++c) {
+        const int t0 = c * L.T, rows = min(L.T, N - t0);
+        load_rows(q, base + (size_t)t0 * d, rows, d, Xq, L.pd, L.T);
         if (p.causal) {
-            load_rows(k, base + (size_t)t0 * d, CL, d, Xk, d);
-            load_rows(v, base + (size_t)t0 * d, CL, d, Vx, d + 1);
+            load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
+            load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+            unit_weights(L, d, rows, V);
         }
         __syncthreads();
-        if (tau && p.causal) weight_keys(Xk, CL, d, itau, Vx);
-        features(p, Xq, CL, W, Pq, D + 1);
-        if (p.causal) features(p, Xk, CL, W, Pk, D + 1);
-        __syncthreads();
-        if (p.causal) {
-            for (int idx = threadIdx.x; idx < CL * CL; idx += blockDim.x) {
-                int i = idx / CL, j = idx % CL;
-                float a = 0.f;
-                if (j <= i)
-                    for (int f = 0; f < D; ++f) a = fmaf(Pq[i * (D + 1) + f], Pk[j * (D + 1) + f], a);
-                A[i * C + j] = a;
+        if (tau && p.causal) weight_keys(L, Xk, rows, d, itau, V, red);
+        float aa[4][4], num[ND][4][4], dsum = 0.f;
+        zero(aa);
+#pragma unroll
+        for (int n = 0; n < ND; ++n) zero(num[n]);
+        for (int g = 0; g < L.ng; ++g) {
+            float* W = sm + L.W + g * gW;
+            float* Sg = S + g * gS;
+            if (!L.wres) {
+                stage_projection<NS>(p, L, W1, W2, h, g, W);
+                __syncthreads();
+            }
+            if (f.on) {
+                float pf[4][4], qf[4][4];
+                features<NS, false>(p, L, f, Xq, rows, W, g, pf, qf);
+                store_tile(Pq, L.pp, f, pf);
+                if (p.causal) {
+                    features<NS, false>(p, L, f, Xk, rows, W, g, pf, qf);
+                    store_tile(Pk, L.pp, f, pf);
+                }
             }
             __syncthreads();
+            if (p.causal && a_on)
+                mm_nt<4>(Pq + 4 * ay * L.pp, L.pp, Pk + ax * L.pp, TT * L.pp, L.F, aa);
+#pragma unroll
+            for (int n = 0; n < ND; ++n) {
+                const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
+                if (y < TT)
+                    mm_nn(Pq + 4 * y * L.pp, L.pp, Sg + e, L.CT * L.pd, 2 * L.CT * L.pd,
+                          3 * L.CT * L.pd, L.pd, L.F, num[n]);
+            }
+            if (tid < 4 * L.T)  // denominator: four lanes per row
+                for (int i = tid & 3; i < L.CT; i += 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(Pq + (tid >> 2) * L.pp + 4 * i);
+                    const float* z = Sg + i * L.pd + d;
+                    dsum = fmaf(x.x, z[0], dsum);
+                    dsum = fmaf(x.y, z[L.CT * L.pd], dsum);
+                    dsum = fmaf(x.z, z[2 * L.CT * L.pd], dsum);
+                    dsum = fmaf(x.w, z[3 * L.CT * L.pd], dsum);
+                }
+            __syncthreads();
+            if (p.causal) {
+                state_update(L, d, Pk, V, Sg);
+                if (g + 1 < L.ng) __syncthreads();
+            }
         }
-        // numerator (columns < d) and denominator (column d) of every row of the chunk
-        for (int idx = threadIdx.x; idx < CL * (d + 1); idx += blockDim.x) {
-            int i = idx / (d + 1), e = idx % (d + 1);
-            float acc = 0.f;
-            if (p.causal)
-                for (int j = 0; j <= i; ++j) acc = fmaf(A[i * C + j], Vx[j * (d + 1) + e], acc);
-            for (int f = 0; f < D; ++f) acc = fmaf(Pq[i * (D + 1) + f], S[f * (d + 1) + e], acc);
-            O[i * (d + 1) + e] = acc;
+        if (p.causal) {
+            if (a_on)
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        const int i = 4 * ay + r, j = ax + TT * cc;
+                        A[i * L.pa + j] = j <= i ? aa[r][cc] : 0.f;
+                    }
+            __syncthreads();
+#pragma unroll
+            for (int n = 0; n < ND; ++n) {
+                const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
+                if (y < TT)
+                    mm_nn(A + 4 * y * L.pa, L.pa, V + e, L.pd, 2 * L.pd, 3 * L.pd, 4 * L.pd, L.T,
+                          num[n]);
+            }
+            if (tid < 4 * L.T)
+                for (int j = tid & 3; j < L.T; j += 4)
+                    dsum = fmaf(A[(tid >> 2) * L.pa + j], V[j * L.pd + d], dsum);
+        }
+        if (tid < 4 * L.T) {
+            dsum += __shfl_xor_sync(0xffffffffu, dsum, 1);
+            dsum += __shfl_xor_sync(0xffffffffu, dsum, 2);
+            const int i = tid >> 2;
+            if ((tid & 3) == 0) {
+                red[kMaxT + i] = dsum;
+                if (den && i < rows) den[(size_t)bh * N + t0 + i] = dsum * inv_m;
+            }
         }
         __syncthreads();
-        for (int idx = threadIdx.x; idx < CL * d; idx += blockDim.x) {
-            int i = idx / d, e = idx % d;
-            store_act(out, base + (size_t)(t0 + i) * d + e, O[i * (d + 1) + e] / O[i * (d + 1) + d]);
+#pragma unroll
+        for (int n = 0; n < ND; ++n) {
+            const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
+            if (y < TT)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int i = 4 * y + r;
+                    if (i >= rows) break;
+                    const float dn = red[kMaxT + i];
+                    store_act4(out, base + (size_t)(t0 + i) * d + e,
+                               make_float4(num[n][r][0] / dn, num[n][r][1] / dn,
+                                           num[n][r][2] / dn, num[n][r][3] / dn));
+                }
         }
-        if (den)
-            for (int i = threadIdx.x; i < CL; i += blockDim.x)
-                den[(size_t)bh * N + t0 + i] = O[i * (d + 1) + d] * inv_m;
-        if (p.causal) state_update(Pk, Vx, CL, D, d, S);
-        __syncthreads();
     }
+    if (L.CL > 1) tc::cluster_sync();  // no CTA leaves while another may read its state
 }
 
 // ------------------------------------------------------------------------------------
 // Backward.
 // ------------------------------------------------------------------------------------
-struct BwdLayout {
-    size_t W, S, Xq, Xk, Vx, Gx, Pq, Pk, dP, A, dA, dAct, Kc, total;
-};
-
-__host__ __device__ inline BwdLayout bwd_layout(const Problem& p, int C)
-{
-    const int d = p.d, D = 2 * p.M, Mc = p.nonstat ? 2 * p.M : p.M;
-    BwdLayout L;
-    size_t o = 0;
-    L.W = o;    o += (size_t)Mc * (d + 1);
-    L.S = o;    o += (size_t)D * (d + 1);
-    L.Xq = o;   o += (size_t)C * d;
-    L.Xk = o;   o += (size_t)C * d;
-    L.Vx = o;   o += (size_t)C * (d + 1);
-    L.Gx = o;   o += (size_t)C * (d + 1);
-    L.Pq = o;   o += (size_t)C * (D + 1);
-    L.Pk = o;   o += (size_t)C * (D + 1);
-    L.dP = o;   o += (size_t)C * (D + 1);
-    L.A = o;    o += (size_t)C * C;
-    L.dA = o;   o += (size_t)C * C;
-    L.dAct = o; o += (size_t)C * (Mc + 1);
-    L.Kc = o;   o += (size_t)C;
-    L.total = o;
-    return L;
-}
-
-// Gx[t] = [dout_t / den'_t, -(dout_t . out_t) / den'_t] with den' = M * den.
+// G[t] = [dout_t / den'_t | -(dout_t . out_t) / den'_t] with den' = M den; zero past `rows`.
+// Four lanes per row.
 template <typename T>
-__device__ void load_upstream(const Problem& p, const T* dout, const T* out, const float* den,
-                              size_t base, size_t den_base, int rows, float* Gx)
+__device__ __forceinline__ void load_upstream(const Problem& p, const Plan& L, const T* dout,
+                                              const T* out, const float* den, size_t base,
+                                              size_t den_base, int rows, float* G)
 {
-    const int d = p.d;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, nwarps = blockDim.x / 32;
-    for (int t = warp; t < rows; t += nwarps) {
-        const float dn = den[den_base + t] * (float)p.M;
-        float s = 0.f;
-        for (int e = lane; e < d; e += 32) {
-            float g = load_act(dout, base + (size_t)t * d + e);
-            s = fmaf(g, load_act(out, base + (size_t)t * d + e), s);
-            Gx[t * (d + 1) + e] = g / dn;
+    if (threadIdx.x >= 4 * L.T) return;
+    const int d = p.d, t = threadIdx.x >> 2, part = threadIdx.x & 3;
+    const bool ok = t < rows;
+    const float dn = ok ? den[den_base + t] * (float)p.M : 1.f;
+    float s = 0.f;
+    for (int e = 4 * part; e < d; e += 16) {
+        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ok) {
+            g = load_act4(dout, base + (size_t)t * d + e);
+            const float4 o = load_act4(out, base + (size_t)t * d + e);
+            s = fmaf(g.x, o.x, fmaf(g.y, o.y, fmaf(g.z, o.z, fmaf(g.w, o.w, s))));
+            g = make_float4(g.x / dn, g.y / dn, g.z / dn, g.w / dn);
         }
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) Gx[t * (d + 1) + d] = -s / dn;
+        *reinterpret_cast<float4*>(G + t * L.pd + e) = g;
     }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (part == 0) G[t * L.pd + d] = -s / dn;
 }
 
-// Chain rule through the feature map: dAct[t][m] = d/da (stationary) or (du, dw).
-__device__ void feature_backward(const Problem& p, const float* X, const float* P,
-                                 const float* dP, int rows, const float* W, float* dAct)
+// Chain rule through the features: dP = (dL/dcos, dL/dsin) of two frequencies a row ->
+// dL/da (s), or dL/du, dL/dw of each (n), stored as projection columns.
+template <bool NS>
+__device__ __forceinline__ void store_chain(const Plan& L, const Place& f, const float (&dp)[4][4],
+                                            const float (&pf)[4][4], const float (&qf)[4][4],
+                                            float* D)
 {
-    const int d = p.d, M = p.M, D = 2 * M, Mc = p.nonstat ? 2 * M : M;
-    for (int idx = threadIdx.x; idx < rows * M; idx += blockDim.x) {
-        int t = idx / M, m = idx % M;
-        const float dc = dP[t * (D + 1) + m], ds = dP[t * (D + 1) + M + m];
-        if (!p.nonstat) {
-            const float c = P[t * (D + 1) + m], s = P[t * (D + 1) + M + m];
-            dAct[t * (Mc + 1) + m] = -s * dc + c * ds;
-        } else {
-            const float* x = X + t * d;
-            const float *wa = W + m * (d + 1), *wb = W + (M + m) * (d + 1);
-            float u = 0.f, w = 0.f;
-            for (int i = 0; i < d; ++i) {
-                u = fmaf(x[i], wa[i], u);
-                w = fmaf(x[i], wb[i], w);
-            }
-            float su, cu, sw, cw;
-            sincosf(u, &su, &cu);
-            sincosf(w, &sw, &cw);
-            dAct[t * (Mc + 1) + m] = cw * (-su * dc + cu * ds);
-            dAct[t * (Mc + 1) + M + m] = -sw * (cu * dc + su * ds);
-        }
-    }
-}
-
-// dx[t][i] = sum_m dAct[t][m] W[m][i] (+ xcoef[t] X[t][i], the key prefactor's term);
-// dW[m][i] += sum_t dAct[t][m] X[t][i].
-template <typename T>
-__device__ void project_back(const Problem& p, const float* X, const float* dAct, int rows,
-                             const float* W, T* dx, size_t base, float* dw_acc,
-                             const float* xcoef)
-{
-    const int d = p.d, Mc = p.nonstat ? 2 * p.M : p.M;
-    for (int idx = threadIdx.x; idx < rows * d; idx += blockDim.x) {
-        int t = idx / d, i = idx % d;
-        float acc = 0.f;
-        for (int m = 0; m < Mc; ++m) acc = fmaf(dAct[t * (Mc + 1) + m], W[m * (d + 1) + i], acc);
-        if (xcoef) acc = fmaf(xcoef[t], X[t * d + i], acc);
-        store_act(dx, base + (size_t)t * d + i, acc);
-    }
 #pragma unroll
-    for (int r = 0; r < kMaxDwPerThread; ++r) {
-        int e = r * kThreads + threadIdx.x;
-        if (e < Mc * d) {
-            int m = e / d, i = e % d;
-            float acc = dw_acc[r];
-            for (int t = 0; t < rows; ++t) acc = fmaf(dAct[t * (Mc + 1) + m], X[t * d + i], acc);
-            dw_acc[r] = acc;
+    for (int r = 0; r < 4; ++r) {
+        const float a0 = fmaf(-pf[r][1], dp[r][0], pf[r][0] * dp[r][1]);
+        const float a1 = fmaf(-pf[r][3], dp[r][2], pf[r][2] * dp[r][3]);
+        float* row = D + (4 * f.y + r) * L.pp;
+        if (NS) {
+            const float b0 = -fmaf(qf[r][0], dp[r][0], qf[r][1] * dp[r][1]);
+            const float b1 = -fmaf(qf[r][2], dp[r][2], qf[r][3] * dp[r][3]);
+            *reinterpret_cast<float4*>(row + 4 * f.x) = make_float4(a0, b0, a1, b1);
+        } else {
+            *reinterpret_cast<float2*>(row + 2 * f.x) = make_float2(a0, a1);
         }
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) simt_bwd_kernel(
-    Problem p, int C, const T* q, const T* k, const T* v, const float* W1, const float* W2,
-    const float* tau, const T* out, const float* den, const T* dout, T* dq, T* dk, T* dv,
-    float* dw_part, float* dtau_part)
+// dx tiles += da W and dW += da^T X of one group.
+template <bool NS, int ND>
+__device__ __forceinline__ void project_back(const Plan& L, int d, const float* D, const float* W,
+                                             const float* X, float* dW, float (&dx)[ND][4][4])
 {
-    extern __shared__ float sm[];
-    const int d = p.d, D = 2 * p.M, N = p.N, Mc = p.nonstat ? 2 * p.M : p.M;
-    const int bh = blockIdx.x, h = bh % p.H;
+    const int dq = d / 4, TT = L.T / 4, o = L.CT * L.pd;
+#pragma unroll
+    for (int n = 0; n < ND; ++n) {
+        const int id = threadIdx.x + n * kThreads, y = id / dq, e = 4 * (id % dq);
+        if (y < TT) {
+            if (NS)
+                mm_nn(D + 4 * y * L.pp, L.pp, W + e, o, 2 * o, 3 * o, L.pd, L.KP, dx[n]);
+            else
+                mm_nn(D + 4 * y * L.pp, L.pp, W + e, o, L.pd, o + L.pd, 2 * L.pd, L.KP, dx[n]);
+        }
+    }
+    for (int id = threadIdx.x; id < L.KP / 4 * dq; id += kThreads) {
+        const int x = id / dq, e = 4 * (id % dq);
+        float acc[4][4];
+        zero(acc);
+        mm_tn(D + 4 * x, L.pp, X + e, L.pd, L.T, acc);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float4* w = reinterpret_cast<float4*>(dW + (4 * x + r) * d + e);
+            *w = make_float4(w->x + acc[r][0], w->y + acc[r][1], w->z + acc[r][2],
+                             w->w + acc[r][3]);
+        }
+    }
+}
+
+template <typename T, int ND>
+__device__ __forceinline__ void store_rows(const Plan& L, int d, const float (&x)[ND][4][4],
+                                           T* dst, size_t base, int rows)
+{
+    const int dq = d / 4;
+#pragma unroll
+    for (int n = 0; n < ND; ++n) {
+        const int id = threadIdx.x + n * kThreads, y = id / dq, e = 4 * (id % dq);
+        if (y < L.T / 4)
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (4 * y + r < rows)
+                    store_act4(dst, base + (size_t)(4 * y + r) * d + e,
+                               make_float4(x[n][r][0], x[n][r][1], x[n][r][2], x[n][r][3]));
+    }
+}
+
+template <typename T, bool NS, int ND>
+__global__ void __launch_bounds__(kThreads, 1)
+    simt_bwd_kernel(Problem p, Plan L, const T* q, const T* k, const T* v, const float* W1,
+                    const float* W2, const float* tau, const T* out, const float* den,
+                    const T* dout, T* dq, T* dk, T* dv, float* dw_part, float* dtau_part)
+{
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
+    const int tid = threadIdx.x, d = p.d, N = p.N, d4 = d / 4;
+    const int rank = L.CL > 1 ? (int)tc::cluster_rank() : 0;
+    const int bh = blockIdx.x / L.CL, h = bh % p.H;
     const size_t base = (size_t)bh * N * d, den_base = (size_t)bh * N;
-    const BwdLayout L = bwd_layout(p, C);
-    float *W = sm + L.W, *S = sm + L.S, *Xq = sm + L.Xq, *Xk = sm + L.Xk, *Vx = sm + L.Vx;
-    float *Gx = sm + L.Gx, *Pq = sm + L.Pq, *Pk = sm + L.Pk, *dP = sm + L.dP;
-    float *A = sm + L.A, *dA = sm + L.dA, *dAct = sm + L.dAct, *Kc = sm + L.Kc;
+    float *S = sm + L.S, *Xq = sm + L.Xq, *Xk = sm + L.Xk, *V = sm + L.V, *G = sm + L.G;
+    float *Pq = sm + L.Pq, *Pk = sm + L.Pk, *dA = sm + L.A, *dW = sm + L.dW, *red = sm + L.red;
+    float* A = Pq;  // masked phi(Q) phi(K)^T, once the features are no longer needed
     const float itau = tau ? expf(-tau[h]) : 0.f;
+    const int gS = L.F * L.pd, gW = L.wres ? L.KP * L.pd : 0, gD = L.KP * d;
+    const Place f = {tid / L.CT, tid % L.CT, tid / L.CT < L.T / 4};
+    const int TT = L.T / 4, ay = tid / TT, ax = tid % TT;
+    const bool a_on = ay < TT;
     float dtau_acc = 0.f;
     // |k_0|^2 of the sequence: dtau = -exp(-tau) sum_j (|k_j|^2 - |k_0|^2) s_j (the s_j of a
     // sequence sum to zero, as every output row is invariant to a common key-weight scale)
@@ -384,168 +697,283 @@ __global__ void __launch_bounds__(kThreads) simt_bwd_kernel(
             const float x = load_act(k, base + e);
             n20 = fmaf(x, x, n20);
         }
+    int cb, ce;
+    chunk_range(L, N, rank, &cb, &ce);
 
-    float dw_acc[kMaxDwPerThread];
+    if (L.wres)
+        for (int g = 0; g < L.ng; ++g)
+            stage_projection<NS>(p, L, W1, W2, h, g, sm + L.W + g * gW);
+    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
+    for (int i = tid; i < L.ng * gD; i += kThreads) dW[i] = 0.f;
+
+    auto load_kv = [&](int t0, int rows) {
+        load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
+        load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+        unit_weights(L, d, rows, V);
+    };
+    auto load_qg = [&](int t0, int rows) {
+        load_rows(q, base + (size_t)t0 * d, rows, d, Xq, L.pd, L.T);
+        load_upstream(p, L, dout, out, den, base + (size_t)t0 * d, den_base + t0, rows, G);
+    };
+    auto group_W = [&](int g) {  // the group's projection rows, staged now unless resident
+        float* W = sm + L.W + g * gW;
+        if (!L.wres) {
+            stage_projection<NS>(p, L, W1, W2, h, g, W);
+            __syncthreads();
+        }
+        return W;
+    };
+    // dA_ij = g_i . v_j + c_i (weighted keys), j <= i
+    auto build_dA = [&]() {
+        if (!a_on) return;
+        float acc[4][4];
+        zero(acc);
+        mm_nt<4>(G + 4 * ay * L.pd, L.pd, V + ax * L.pd, TT * L.pd, d, acc);
 #pragma unroll
-    for (int r = 0; r < kMaxDwPerThread; ++r) dw_acc[r] = 0.f;
-
-    load_projection(p, W1, W2, h, W);
-    for (int idx = threadIdx.x; idx < D * (d + 1); idx += blockDim.x) S[idx] = 0.f;
-    for (int idx = threadIdx.x; idx < C; idx += blockDim.x) Vx[idx * (d + 1) + d] = 1.f;
-    __syncthreads();
+        for (int r = 0; r < 4; ++r) {
+            const int i = 4 * ay + r;
+            const float ci = G[i * L.pd + d];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int j = ax + TT * c;
+                dA[i * L.pa + j] = j <= i ? fmaf(ci, V[j * L.pd + d], acc[r][c]) : 0.f;
+            }
+        }
+    };
+    // this range's sums of phi(x) [y | y_d], over its chunks, into S (zeroed)
+    auto range_state = [&](bool keys) {
+        for (int c = cb; c < ce; ++c) {
+            const int t0 = c * L.T, rows = min(L.T, N - t0);
+            if (keys)
+                load_kv(t0, rows);
+            else
+                load_qg(t0, rows);
+            __syncthreads();
+            if (keys && tau) weight_keys(L, Xk, rows, d, itau, V, red);
+            for (int g = 0; g < L.ng; ++g) {
+                float* W = group_W(g);
+                if (f.on) {
+                    float pf[4][4], qf[4][4];
+                    features<NS, false>(p, L, f, keys ? Xk : Xq, rows, W, g, pf, qf);
+                    store_tile(keys ? Pk : Pq, L.pp, f, pf);
+                }
+                __syncthreads();
+                state_update(L, d, keys ? Pk : Pq, keys ? V : G, S + g * gS);
+                __syncthreads();
+            }
+        }
+    };
 
     // ---- dq: forward direction with S_i, z_i ----
-    if (!p.causal) {
-        for (int t0 = 0; t0 < N; t0 += C) {
-            const int CL = min(C, N - t0);
-            load_rows(k, base + (size_t)t0 * d, CL, d, Xk, d);
-            load_rows(v, base + (size_t)t0 * d, CL, d, Vx, d + 1);
-            __syncthreads();
-            if (tau) weight_keys(Xk, CL, d, itau, Vx);
-            features(p, Xk, CL, W, Pk, D + 1);
-            __syncthreads();
-            state_update(Pk, Vx, CL, D, d, S);
-            __syncthreads();
-        }
+    if (!p.causal || L.CL > 1) {
+        __syncthreads();
+        range_state(true);
+        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
     }
-    for (int t0 = 0; t0 < N; t0 += C) {
-        const int CL = min(C, N - t0);
-        const size_t off = base + (size_t)t0 * d;
-        load_rows(q, off, CL, d, Xq, d);
-        load_upstream(p, dout, out, den, off, den_base + t0, CL, Gx);
-        if (p.causal) {
-            load_rows(k, off, CL, d, Xk, d);
-            load_rows(v, off, CL, d, Vx, d + 1);
-        }
+    __syncthreads();
+    for (int c = cb; c < ce; ++c) {
+        const int t0 = c * L.T, rows = min(L.T, N - t0);
+        load_qg(t0, rows);
+        if (p.causal) load_kv(t0, rows);
         __syncthreads();
-        if (tau && p.causal) {
-            weight_keys(Xk, CL, d, itau, Vx);
+        if (p.causal) {
+            if (tau) {
+                weight_keys(L, Xk, rows, d, itau, V, red);
+                __syncthreads();
+            }
+            build_dA();
+        }
+        float dx[ND][4][4];
+#pragma unroll
+        for (int n = 0; n < ND; ++n) zero(dx[n]);
+        for (int g = 0; g < L.ng; ++g) {
+            float* W = group_W(g);
+            float* Sg = S + g * gS;
+            float pf[4][4], qf[4][4], dp[4][4];
+            if (f.on) {
+                if (p.causal) {
+                    features<NS, false>(p, L, f, Xk, rows, W, g, pf, qf);
+                    store_tile(Pk, L.pp, f, pf);
+                }
+                features<NS, true>(p, L, f, Xq, rows, W, g, pf, qf);
+            }
+            __syncthreads();
+            if (f.on) {
+                zero(dp);
+                if (p.causal)
+                    mm_nn(dA + 4 * f.y * L.pa, L.pa, Pk + 4 * f.x, L.pp, 2 * L.pp, 3 * L.pp,
+                          4 * L.pp, L.T, dp);
+                mm_nt<4>(G + 4 * f.y * L.pd, L.pd, Sg + f.x * L.pd, L.CT * L.pd, d, dp);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float ci = G[(4 * f.y + r) * L.pd + d];
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc)
+                        dp[r][cc] = fmaf(ci, Sg[(cc * L.CT + f.x) * L.pd + d], dp[r][cc]);
+                }
+            }
+            __syncthreads();
+            if (f.on) store_chain<NS>(L, f, dp, pf, qf, Pq);
+            if (p.causal) state_update(L, d, Pk, V, Sg);
+            __syncthreads();
+            project_back<NS, ND>(L, d, Pq, W, Xq, dW + g * gD, dx);
             __syncthreads();
         }
-        features(p, Xq, CL, W, Pq, D + 1);
-        if (p.causal) features(p, Xk, CL, W, Pk, D + 1);
-        if (p.causal)
-            for (int idx = threadIdx.x; idx < CL * CL; idx += blockDim.x) {
-                int i = idx / CL, j = idx % CL;
-                float a = 0.f;
-                if (j <= i)
-                    for (int e = 0; e <= d; ++e) a = fmaf(Gx[i * (d + 1) + e], Vx[j * (d + 1) + e], a);
-                dA[i * C + j] = a;
-            }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < CL * D; idx += blockDim.x) {
-            int i = idx / D, f = idx % D;
-            float acc = 0.f;
-            if (p.causal)
-                for (int j = 0; j <= i; ++j) acc = fmaf(dA[i * C + j], Pk[j * (D + 1) + f], acc);
-            for (int e = 0; e <= d; ++e) acc = fmaf(S[f * (d + 1) + e], Gx[i * (d + 1) + e], acc);
-            dP[i * (D + 1) + f] = acc;
-        }
-        __syncthreads();
-        if (p.causal) state_update(Pk, Vx, CL, D, d, S);
-        feature_backward(p, Xq, Pq, dP, CL, W, dAct);
-        __syncthreads();
-        project_back(p, Xq, dAct, CL, W, dq, off, dw_acc, nullptr);
-        __syncthreads();
+        store_rows<T, ND>(L, d, dx, dq, base + (size_t)t0 * d, rows);
     }
 
     // ---- dk, dv: reverse direction with R_j, r_j (S's buffer is reused for R) ----
-    for (int idx = threadIdx.x; idx < D * (d + 1); idx += blockDim.x) S[idx] = 0.f;
+    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
     __syncthreads();
-    float* R = S;
-    if (!p.causal) {
-        for (int t0 = 0; t0 < N; t0 += C) {
-            const int CL = min(C, N - t0);
-            const size_t off = base + (size_t)t0 * d;
-            load_rows(q, off, CL, d, Xq, d);
-            load_upstream(p, dout, out, den, off, den_base + t0, CL, Gx);
-            __syncthreads();
-            features(p, Xq, CL, W, Pq, D + 1);
-            __syncthreads();
-            state_update(Pq, Gx, CL, D, d, R);
-            __syncthreads();
-        }
+    if (!p.causal || L.CL > 1) {
+        range_state(false);
+        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kSuffix : kTotal);
+        __syncthreads();
     }
-    const int nchunks = (N + C - 1) / C;
-    for (int c = nchunks - 1; c >= 0; --c) {
-        const int t0 = c * C, CL = min(C, N - t0);
-        const size_t off = base + (size_t)t0 * d;
-        load_rows(k, off, CL, d, Xk, d);
-        load_rows(v, off, CL, d, Vx, d + 1);
-        if (p.causal) {
-            load_rows(q, off, CL, d, Xq, d);
-            load_upstream(p, dout, out, den, off, den_base + t0, CL, Gx);
-        }
+    for (int c = ce - 1; c >= cb; --c) {
+        const int t0 = c * L.T, rows = min(L.T, N - t0);
+        load_kv(t0, rows);
+        if (p.causal) load_qg(t0, rows);
         __syncthreads();
         if (tau) {
-            weight_keys(Xk, CL, d, itau, Vx);
+            weight_keys(L, Xk, rows, d, itau, V, red);
             __syncthreads();
         }
-        features(p, Xk, CL, W, Pk, D + 1);
-        if (p.causal) features(p, Xq, CL, W, Pq, D + 1);
-        __syncthreads();
-        if (p.causal)
-            for (int idx = threadIdx.x; idx < CL * CL; idx += blockDim.x) {
-                int i = idx / CL, j = idx % CL;
-                float a = 0.f, da = 0.f;
-                if (j <= i) {
-                    for (int f = 0; f < D; ++f) a = fmaf(Pq[i * (D + 1) + f], Pk[j * (D + 1) + f], a);
-                    for (int e = 0; e <= d; ++e) da = fmaf(Gx[i * (d + 1) + e], Vx[j * (d + 1) + e], da);
+        if (p.causal) build_dA();
+        float dx[ND][4][4], dvt[ND][4][4], aa[4][4], sdot[4] = {0.f, 0.f, 0.f, 0.f};
+        zero(aa);
+#pragma unroll
+        for (int n = 0; n < ND; ++n) {
+            zero(dx[n]);
+            zero(dvt[n]);
+        }
+        for (int g = 0; g < L.ng; ++g) {
+            float* W = group_W(g);
+            float* Rg = S + g * gS;
+            float pf[4][4], qf[4][4], dp[4][4];
+            if (f.on) {
+                if (p.causal) {
+                    features<NS, false>(p, L, f, Xq, rows, W, g, pf, qf);
+                    store_tile(Pq, L.pp, f, pf);
                 }
-                A[i * C + j] = a;
-                dA[i * C + j] = da;
+                features<NS, true>(p, L, f, Xk, rows, W, g, pf, qf);
+                store_tile(Pk, L.pp, f, pf);
             }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < CL * D; idx += blockDim.x) {
-            int j = idx / D, f = idx % D;
-            float acc = 0.f;
-            if (p.causal)
-                for (int i = j; i < CL; ++i) acc = fmaf(dA[i * C + j], Pq[i * (D + 1) + f], acc);
-            for (int e = 0; e <= d; ++e) acc = fmaf(R[f * (d + 1) + e], Vx[j * (d + 1) + e], acc);
-            dP[j * (D + 1) + f] = acc;
-        }
-        for (int idx = threadIdx.x; idx < CL * d; idx += blockDim.x) {
-            int j = idx / d, e = idx % d;
-            float acc = 0.f;
-            if (p.causal)
-                for (int i = j; i < CL; ++i) acc = fmaf(A[i * C + j], Gx[i * (d + 1) + e], acc);
-            for (int f = 0; f < D; ++f) acc = fmaf(R[f * (d + 1) + e], Pk[j * (D + 1) + f], acc);
-            if (tau) acc *= Vx[j * (d + 1) + d];  // dv_j = w_j R_j^T phi(k_j)
-            store_act(dv, off + (size_t)j * d + e, acc);
-        }
-        __syncthreads();
-        if (tau)  // s_j = phi(k_j) . dphi(k_j): dk_j += 2 itau s_j k_j, dtau -= itau |k_j|^2 s_j
-            for (int j = threadIdx.x; j < CL; j += blockDim.x) {
-                float sj = 0.f, n2 = 0.f;
-                for (int f = 0; f < D; ++f) sj = fmaf(Pk[j * (D + 1) + f], dP[j * (D + 1) + f], sj);
-                for (int e = 0; e < d; ++e) n2 = fmaf(Xk[j * d + e], Xk[j * d + e], n2);
-                Kc[j] = 2.f * itau * sj;
-                dtau_acc = fmaf(-itau * (n2 - n20), sj, dtau_acc);
+            __syncthreads();
+            if (p.causal && a_on)
+                mm_nt<4>(Pq + 4 * ay * L.pp, L.pp, Pk + ax * L.pp, TT * L.pp, L.F, aa);
+#pragma unroll
+            for (int n = 0; n < ND; ++n) {
+                const int id = tid + n * kThreads, y = id / d4, e = 4 * (id % d4);
+                if (y < TT)
+                    mm_nn(Pk + 4 * y * L.pp, L.pp, Rg + e, L.CT * L.pd, 2 * L.CT * L.pd,
+                          3 * L.CT * L.pd, L.pd, L.F, dvt[n]);
             }
-        if (p.causal) state_update(Pq, Gx, CL, D, d, R);
-        feature_backward(p, Xk, Pk, dP, CL, W, dAct);
+            if (f.on) {
+                zero(dp);
+                if (p.causal) mm_tn(dA + 4 * f.y, L.pa, Pq + 4 * f.x, L.pp, L.T, dp);
+                mm_nt<4>(V + 4 * f.y * L.pd, L.pd, Rg + f.x * L.pd, L.CT * L.pd, d, dp);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float wj = V[(4 * f.y + r) * L.pd + d];
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        dp[r][cc] = fmaf(wj, Rg[(cc * L.CT + f.x) * L.pd + d], dp[r][cc]);
+                        sdot[r] = fmaf(pf[r][cc], dp[r][cc], sdot[r]);
+                    }
+                }
+            }
+            __syncthreads();
+            if (f.on) store_chain<NS>(L, f, dp, pf, qf, Pk);
+            if (p.causal) state_update(L, d, Pq, G, Rg);
+            __syncthreads();
+            project_back<NS, ND>(L, d, Pk, W, Xk, dW + g * gD, dx);
+            __syncthreads();
+        }
+        if (p.causal && a_on)
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int cc = 0; cc < 4; ++cc) {
+                    const int i = 4 * ay + r, j = ax + TT * cc;
+                    A[i * L.pa + j] = j <= i ? aa[r][cc] : 0.f;
+                }
+        if (tau && f.on)  // s_j = phi(k_j) . dphi(k_j), one partial per column tile
+#pragma unroll
+            for (int r = 0; r < 4; ++r) dA[(4 * f.y + r) * L.pa + f.x] = sdot[r];
         __syncthreads();
-        project_back(p, Xk, dAct, CL, W, dk, off, dw_acc, tau ? Kc : nullptr);
+        if (tau) {  // dk_j += 2 itau s_j k_j, dtau -= itau |k_j|^2 s_j
+            if (tid < L.T) {
+                float sj = 0.f;
+                for (int x = 0; x < L.CT; ++x) sj += dA[tid * L.pa + x];
+                red[kMaxT + tid] = 2.f * itau * sj;
+                if (tid < rows) dtau_acc = fmaf(-itau * (red[tid] - n20), sj, dtau_acc);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int n = 0; n < ND; ++n) {
+            const int id = tid + n * kThreads, y = id / d4, e = 4 * (id % d4);
+            if (y < TT) {
+                if (p.causal) mm_tn(A + 4 * y, L.pa, G + e, L.pd, L.T, dvt[n]);
+                if (tau)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int j = 4 * y + r;
+                        const float wj = V[j * L.pd + d], kc = red[kMaxT + j];
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            dvt[n][r][cc] *= wj;  // dv_j = w_j R_j^T phi(k_j)
+                            dx[n][r][cc] = fmaf(kc, Xk[j * L.pd + e + cc], dx[n][r][cc]);
+                        }
+                    }
+            }
+        }
+        store_rows<T, ND>(L, d, dvt, dv, base + (size_t)t0 * d, rows);
+        store_rows<T, ND>(L, d, dx, dk, base + (size_t)t0 * d, rows);
         __syncthreads();
     }
 
-    float* part = dw_part + (size_t)bh * Mc * d;
-#pragma unroll
-    for (int r = 0; r < kMaxDwPerThread; ++r) {
-        int e = r * kThreads + threadIdx.x;
-        if (e < Mc * d) part[e] = dw_acc[r];
-    }
-    if (tau) {  // this sequence's dtau: warp sums, then the warps in order
+    // ---- the sequence's dW and dtau: the cluster's partials in rank order ----
+    if (tau) {
         for (int o = 16; o > 0; o >>= 1) dtau_acc += __shfl_xor_sync(0xffffffffu, dtau_acc, o);
+        if ((tid & 31) == 0) red[tid >> 5] = dtau_acc;
         __syncthreads();
-        if ((threadIdx.x & 31) == 0) Kc[threadIdx.x >> 5] = dtau_acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             float t = 0.f;
-            for (int w = 0; w < kThreads / 32; ++w) t += Kc[w];
-            dtau_part[bh] = t;
+            for (int w = 0; w < kThreads / 32; ++w) t += red[w];
+            red[kMaxT] = t;
         }
     }
+    if (L.CL > 1)
+        tc::cluster_sync();
+    else
+        __syncthreads();
+    const int Mc = NS ? 2 * p.M : p.M;
+    float* part = dw_part + (size_t)bh * Mc * d;
+    const uint32_t dw_addr = tc::smem_u32(dW);
+    for (int i = rank * kThreads + tid; i < L.ng * gD / 4; i += L.CL * kThreads) {
+        const int row = 4 * i / d, e = 4 * i % d, g = row / L.KP, kk = row % L.KP;
+        const int fr = g * L.MG + (NS ? 2 * (kk >> 2) + ((kk >> 1) & 1) : kk);
+        if (fr >= p.M) continue;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (L.CL == 1) {
+            a = *reinterpret_cast<const float4*>(dW + 4 * i);
+        } else {
+            for (int r = 0; r < L.CL; ++r) {
+                const float4 x = tc::ld_cluster_v4(tc::mapa(dw_addr + 16 * i, r));
+                a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
+            }
+        }
+        // n: rows < M of the partial hold dU, rows >= M dV
+        *reinterpret_cast<float4*>(part + (size_t)(NS && (kk & 1) ? p.M + fr : fr) * d + e) = a;
+    }
+    if (tau && rank == 0 && tid == 0) {
+        float t = red[kMaxT];
+        for (int r = 1; r < L.CL; ++r) t += tc::ld_cluster_f32(tc::mapa(tc::smem_u32(red + kMaxT), r));
+        dtau_part[bh] = t;
+    }
+    if (L.CL > 1) tc::cluster_sync();  // no CTA leaves while another may read its partials
 }
 
 // Key weights of the norm prefactor for the tensor-core forwards: kw[row] =
@@ -649,34 +1077,159 @@ __global__ void dw_reduce_kernel(Problem p, const float* part, float* dW1, float
     }
 }
 
+
+// ---- sizes taken by the entry points ----------------------------------------------------
+// A sequence's frequencies and state (and eight tokens of every operand) have to fit one
+// CTA's shared memory: 227 KB of fp32.
+constexpr size_t kSmemFloats = 227 * 1024 / 4;
+constexpr size_t kMaxDw = 16384;  // Mc * d, the backward's frequency gradient
+
+bool fits_fwd(const Problem& p)
+{
+    const size_t d = p.d, D = 2 * (size_t)p.M, Mc = p.nonstat ? D : D / 2;
+    return Mc * (d + 1) + D * (d + 1) + 8 * (2 * d + 2 * (d + 1) + 2 * (D + 1) + 8) <= kSmemFloats;
+}
+bool fits_bwd(const Problem& p)
+{
+    const size_t d = p.d, D = 2 * (size_t)p.M, Mc = p.nonstat ? D : D / 2;
+    return Mc * d <= kMaxDw && Mc * (d + 1) + D * (d + 1) +
+                                       8 * (2 * d + 2 * (d + 1) + 3 * (D + 1) + 16 + Mc + 1 + 1) <=
+                                   kSmemFloats;
+}
+
+// The plan for groups of at most mg frequencies and T tokens per chunk, with or without
+// resident projection rows.
+Plan layout(const Problem& p, bool bwd, int mg, int T, bool wres)
+{
+    Plan L = {};
+    L.T = T;
+    L.wres = wres;
+    L.CL = 1;
+    L.ng = (p.M + mg - 1) / mg;
+    L.MG = ((p.M + L.ng - 1) / L.ng + 3) / 4 * 4;
+    L.CT = L.MG / 2;
+    L.F = 2 * L.MG;
+    L.KP = p.nonstat ? 2 * L.MG : L.MG;
+    L.pd = p.d + 4;
+    L.pp = L.F + 4;
+    L.pa = std::max(T, 16) + 4;
+    int o = 0;
+    auto take = [&](int n) {
+        const int at = o;
+        o += n;
+        return at;
+    };
+    const int rows = T * L.pd, feats = T * std::max(L.pp, L.pa);
+    L.S = take(L.ng * L.F * L.pd);
+    L.W = take((wres ? L.ng : 1) * L.KP * L.pd);
+    L.dW = bwd ? take(L.ng * L.KP * p.d) : 0;
+    // without the mask one pass holds only queries or only keys: their regions are one
+    L.Xk = take(rows);
+    L.Xq = p.causal ? take(rows) : L.Xk;
+    L.V = take(rows);
+    L.G = !bwd ? 0 : p.causal ? take(rows) : L.V;
+    L.Pk = take(feats);
+    L.Pq = p.causal ? take(feats) : L.Pk;
+    // forward: phi(Q) phi(K)^T replaces phi(Q); backward: dA has its own block (causal), and
+    // without the mask only the prefactor's s_j go there, after the features' last use
+    L.A = bwd && p.causal ? take(T * L.pa) : L.Pq;
+    L.red = take(2 * kMaxT);
+    L.total = o;
+    return L;
+}
+
+// The largest chunk that fits, with the projection rows resident when they fit beside it
+// (M <= 32 has one group, staged once either way); then the CTAs per sequence: the count
+// that minimises the rounds of CTAs on the SMs times the work of one, counted in chunks
+// (a range's own sums, needed when the sequence is split or not causal, cost about 0.4 of
+// a forward chunk, a backward chunk about 3; set-up about one).
+bool make_plan(const Problem& p, bool bwd, Plan* plan)
+{
+    if (!(bwd ? fits_bwd(p) : fits_fwd(p))) return false;
+    bool found = false;
+    for (int mg = kMaxMG; mg >= 4 && !found; mg /= 2)  // smaller groups: the largest shapes only
+        for (int T = kMaxT; T >= 8 && !found; T /= 2)
+            for (int wres = 1; wres >= 0 && !found; --wres) {
+                *plan = layout(p, bwd, mg, T, wres != 0);
+                found = (size_t)plan->total <= kSmemFloats;
+            }
+    if (!found) return false;
+    const int sms = std::max(1, tc::sm_count());
+    const int occ = !bwd && 2 * ((size_t)plan->total * 4 + 1024) <= 228 * 1024 ? 2 : 1;
+    const long long bh = (long long)p.B * p.H, nch = (p.N + plan->T - 1) / plan->T;
+    double best = 0.;
+    for (int cl = 1; cl <= kMaxCluster && (cl == 1 || cl <= nch); cl *= 2) {
+        const double per = (double)((nch + cl - 1) / cl);
+        const double pre = !p.causal || cl > 1 ? (bwd ? 0.8 : 0.4) : 0.;
+        const long long ctas = bh * cl;
+        double rounds = (double)((ctas + (long long)sms * occ - 1) / ((long long)sms * occ));
+        if (occ == 2 && ctas > sms) rounds *= 1.6;  // two CTAs share an SM
+        const double cost = rounds * (per * ((bwd ? 3. : 1.) + pre) + 1. + (cl > 1 ? 0.5 : 0.));
+        if (cl == 1 || cost < best) {
+            best = cost;
+            plan->CL = cl;
+        }
+    }
+    return true;
+}
+
+// Launches `kern` with CL CTAs per sequence as one cluster.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_plan(void (*kern)(KArgs...), const Problem& p, const Plan& L, cudaStream_t s,
+                        Args... args)
+{
+    const size_t smem = (size_t)L.total * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((long long)p.B * p.H * L.CL));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)L.CL;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, p, L, args...);
+}
+
+template <typename T, bool NS>
+cudaError_t launch_fwd_t(const Problem& p, const Plan& L, const void* q, const void* k,
+                         const void* v, const float* W1, const float* W2, const float* tau,
+                         void* out, float* den, cudaStream_t s)
+{
+    auto kern = p.d > 64 ? simt_fwd_kernel<T, NS, 2> : simt_fwd_kernel<T, NS, 1>;
+    return launch_plan(kern, p, L, s, (const T*)q, (const T*)k, (const T*)v, W1, W2, tau, (T*)out,
+                       den);
+}
+
+template <typename T, bool NS>
+cudaError_t launch_bwd_t(const Problem& p, const Plan& L, const void* q, const void* k,
+                         const void* v, const float* W1, const float* W2, const float* tau,
+                         const void* out, const float* den, const void* dout, void* dq, void* dk,
+                         void* dv, float* part, float* tpart, cudaStream_t s)
+{
+    auto kern = p.d > 64 ? simt_bwd_kernel<T, NS, 2> : simt_bwd_kernel<T, NS, 1>;
+    return launch_plan(kern, p, L, s, (const T*)q, (const T*)k, (const T*)v, W1, W2, tau,
+                       (const T*)out, den, (const T*)dout, (T*)dq, (T*)dk, (T*)dv, part, tpart);
+}
+
 }  // namespace
 
-size_t simt_fwd_smem_bytes(const Problem& p, int chunk)
+bool simt_fwd_supported(const Problem& p)
 {
-    return fwd_layout(p, chunk).total * sizeof(float);
+    Plan L;
+    return make_plan(p, false, &L);
 }
 
-size_t simt_bwd_smem_bytes(const Problem& p, int chunk)
+bool simt_bwd_supported(const Problem& p)
 {
-    return bwd_layout(p, chunk).total * sizeof(float);
-}
-
-static const size_t kSmemLimit = 227 * 1024;
-
-int simt_pick_chunk_fwd(const Problem& p)
-{
-    for (int c : {32, 16, 8})
-        if (simt_fwd_smem_bytes(p, c) <= kSmemLimit) return c;
-    return 0;
-}
-
-int simt_pick_chunk_bwd(const Problem& p)
-{
-    const int Mc = p.nonstat ? 2 * p.M : p.M;
-    if ((size_t)Mc * p.d > (size_t)kThreads * kMaxDwPerThread) return 0;
-    for (int c : {32, 16, 8})
-        if (simt_bwd_smem_bytes(p, c) <= kSmemLimit) return c;
-    return 0;
+    Plan L;
+    return make_plan(p, true, &L);
 }
 
 // dW partials [B*H][Mc][d], then dtau partials [B*H].
@@ -730,22 +1283,12 @@ cudaError_t launch_simt_fwd(const Problem& p, const void* q, const void* k, cons
                             const float* W1, const float* W2, const float* tau, void* out,
                             float* den, cudaStream_t s)
 {
-    const int C = simt_pick_chunk_fwd(p);
-    const size_t smem = simt_fwd_smem_bytes(p, C);
-    const int grid = p.B * p.H;
-    if (p.bf16) {
-        auto kern = simt_fwd_kernel<__nv_bfloat16>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kThreads, smem, s>>>(p, C, (const __nv_bfloat16*)q,
-                                          (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, W1,
-                                          W2, tau, (__nv_bfloat16*)out, den);
-    } else {
-        auto kern = simt_fwd_kernel<float>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kThreads, smem, s>>>(p, C, (const float*)q, (const float*)k,
-                                          (const float*)v, W1, W2, tau, (float*)out, den);
-    }
-    return cudaGetLastError();
+    Plan L;
+    if (!make_plan(p, false, &L)) return cudaErrorInvalidValue;
+    typedef __nv_bfloat16 B16;
+    auto run = p.bf16 ? (p.nonstat ? launch_fwd_t<B16, true> : launch_fwd_t<B16, false>)
+                      : (p.nonstat ? launch_fwd_t<float, true> : launch_fwd_t<float, false>);
+    return run(p, L, q, k, v, W1, W2, tau, out, den, s);
 }
 
 cudaError_t launch_simt_bwd(const Problem& p, const void* q, const void* k, const void* v,
@@ -754,28 +1297,15 @@ cudaError_t launch_simt_bwd(const Problem& p, const void* q, const void* k, cons
                             void* dk, void* dv, float* dW1, float* dW2, float* dtau,
                             void* scratch, cudaStream_t s)
 {
-    const int C = simt_pick_chunk_bwd(p);
-    const size_t smem = simt_bwd_smem_bytes(p, C);
-    const int grid = p.B * p.H;
+    Plan L;
+    if (!make_plan(p, true, &L)) return cudaErrorInvalidValue;
     const int Mc = p.nonstat ? 2 * p.M : p.M;
     float* part = (float*)scratch;
     float* tpart = part + (size_t)p.B * p.H * Mc * p.d;
-    if (p.bf16) {
-        typedef __nv_bfloat16 T;
-        auto kern = simt_bwd_kernel<T>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kThreads, smem, s>>>(p, C, (const T*)q, (const T*)k, (const T*)v, W1, W2,
-                                          tau, (const T*)out, den, (const T*)dout, (T*)dq,
-                                          (T*)dk, (T*)dv, part, tpart);
-    } else {
-        typedef float T;
-        auto kern = simt_bwd_kernel<T>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kThreads, smem, s>>>(p, C, (const T*)q, (const T*)k, (const T*)v, W1, W2,
-                                          tau, (const T*)out, den, (const T*)dout, (T*)dq,
-                                          (T*)dk, (T*)dv, part, tpart);
-    }
-    cudaError_t e = cudaGetLastError();
+    typedef __nv_bfloat16 B16;
+    auto run = p.bf16 ? (p.nonstat ? launch_bwd_t<B16, true> : launch_bwd_t<B16, false>)
+                      : (p.nonstat ? launch_bwd_t<float, true> : launch_bwd_t<float, false>);
+    cudaError_t e = run(p, L, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv, part, tpart, s);
     if (e != cudaSuccess) return e;
     const size_t work = (size_t)p.H * p.M * p.d;
     const int blocks = (int)std::min<size_t>((work + kThreads - 1) / kThreads, 152 * 8);
