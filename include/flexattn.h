@@ -69,8 +69,10 @@ enum flex_status {
 /* Human-readable text for a flex_status value. */
 const char* flex_strerror(int status);
 
-/* Workspace bytes needed by flex_linattn_fwd (backward = 0) or flex_linattn_bwd
- * (backward = 1) for this shape; 0 if the shape is invalid or unsupported. */
+/* Workspace bytes of flex_linattn_fwd (backward = 0) or flex_linattn_bwd (backward = 1) for
+ * this shape; 0 if the shape is invalid or unsupported.  (The causal backward of a small
+ * batch uses part of it to run each sequence in ranges; it accepts a smaller workspace that
+ * holds the uncut form's scratch and is slower with it.) */
 size_t flex_workspace_bytes(const flex_shape* shape, int causal, int backward);
 
 /* Feature map phi of Eq. phi_n (W2 == NULL) or Eq. phi_non (W2 != NULL), written out.

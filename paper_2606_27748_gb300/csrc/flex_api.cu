@@ -53,10 +53,12 @@ size_t kw_bytes(const Problem& p)
 }
 size_t fwd_ws_bytes(const Problem& p) { return header_bytes() + nc_scratch_bytes(p) + kw_bytes(p); }
 
-size_t bwd_ws_bytes(const Problem& p)
+// `least`: what a call needs; else what it makes use of (the causal tensor-core backward of
+// a small batch runs its sequences in ranges when the workspace has room for their states).
+size_t bwd_ws_bytes(const Problem& p, bool least)
 {
     size_t scratch = flex::simt_bwd_ws_bytes(p);
-    if (flex::tc_bwd_supported(p)) scratch = std::max(scratch, flex::tc_bwd_ws_bytes(p));
+    if (flex::tc_bwd_supported(p)) scratch = std::max(scratch, flex::tc_bwd_ws_bytes(p, least));
     return header_bytes() + flex::align_up(scratch, 256);
 }
 
@@ -95,7 +97,7 @@ size_t flex_workspace_bytes(const flex_shape* shape, int causal, int backward)
     if (make_problem(shape, nullptr, causal, &p) != FLEX_OK) return 0;
     // Size for the larger of the two variants' scratch.
     p.nonstat = 1;
-    return backward ? bwd_ws_bytes(p) : fwd_ws_bytes(p);
+    return backward ? bwd_ws_bytes(p, false) : fwd_ws_bytes(p);
 }
 
 int flex_featmap(const flex_shape* shape, const void* x, const float* W1, const float* W2,
@@ -161,14 +163,16 @@ int flex_linattn_bwd(const flex_shape* shape, const void* q, const void* k, cons
                           (const void*)dk, (const void*)dv, (const void*)dW1})
         if (!aligned(t, 16)) return FLEX_EINVAL;
     if ((W2 && !aligned(W2, 16)) || (dW2 && !aligned(dW2, 16))) return FLEX_EINVAL;
-    if ((rc = check_ws(ws, ws_bytes, bwd_ws_bytes(p)))) return rc;
+    if ((rc = check_ws(ws, ws_bytes, bwd_ws_bytes(p, true)))) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     void* scratch = (char*)ws + header_bytes();
-    if (flex::tc_bwd_supported(p))  // with tau: one more launch, the key weights
-        return count(flex::tc_bwd_launches(p, tau != nullptr),
+    if (flex::tc_bwd_supported(p)) {  // with tau: one more launch, the key weights
+        const size_t bytes = ws_bytes - header_bytes();
+        return count(flex::tc_bwd_launches(p, tau != nullptr, bytes),
                      flex::launch_tc_bwd(p, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv,
-                                         dW1, dW2, dtau, scratch, &((flex::WsHeader*)ws)->status,
-                                         s));
+                                         dW1, dW2, dtau, scratch, bytes,
+                                         &((flex::WsHeader*)ws)->status, s));
+    }
     if (!flex::simt_bwd_supported(p)) return FLEX_EUNSUPPORTED;
     return count(2, flex::launch_simt_bwd(p, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv,
                                           dW1, dW2, dtau, scratch, s));

@@ -86,13 +86,15 @@ cudaError_t launch_tc_nc(const Problem& p, const void* q, const void* k, const v
                          float* den, void* scratch, int* status, cudaStream_t s);
 
 bool tc_bwd_supported(const Problem& p);
-size_t tc_bwd_ws_bytes(const Problem& p);
-int tc_bwd_launches(const Problem& p, bool tau);  // kernels enqueued by launch_tc_bwd
+// Scratch bytes: what launch_tc_bwd makes use of, or the least it runs with (causal: without
+// cutting sequences into ranges).
+size_t tc_bwd_ws_bytes(const Problem& p, bool least);
+int tc_bwd_launches(const Problem& p, bool tau, size_t bytes);  // kernels launch_tc_bwd enqueues
 cudaError_t launch_tc_bwd(const Problem& p, const void* q, const void* k, const void* v,
                           const float* W1, const float* W2, const float* tau, const void* out,
                           const float* den, const void* dout, void* dq, void* dk, void* dv,
-                          float* dW1, float* dW2, float* dtau, void* scratch, int* status,
-                          cudaStream_t s);
+                          float* dW1, float* dW2, float* dtau, void* scratch, size_t bytes,
+                          int* status, cudaStream_t s);
 
 // ---- feature map on the tensor cores (bf16, d = 64, M in {64, 128}) ------------------
 bool tc_featmap_supported(const Problem& p);
