@@ -1278,88 +1278,121 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 }
 
 // dW over the batch (and the chunk splits) in a fixed order.  Partial slots
-// [pass][((b * H + h) * nsplit + s) * G + g][16 column quads][128 rows][4]; s: rows < 64 are frequencies
-// 64g + row (from the high bf16 part of da), rows >= 64 the same frequencies (from its low
-// part); n: rows < 64 are dU, rows >= 64 are dV of frequency 64g + row%64.
-__global__ void tc_dw_reduce_kernel(int B, int H, int M, int G, int nsplit, int nonstat,
-                                    const float* __restrict__ part, float* __restrict__ dW1,
-                                    float* __restrict__ dW2, const float* __restrict__ dtau_part,
-                                    float* __restrict__ dtau)
+// [pass][((b * H + h) * nsplit + s) * G + g][16 column quads][128 rows][4]; s: rows < 64 are
+// frequencies 64g + row (from the high bf16 part of da), rows >= 64 the same frequencies
+// (from its low part); n: rows < 64 are dU, rows >= 64 are dV of frequency 64g + row%64.
+// One block per (head, group, column quad): thread (row, lane) sums every fourth slot with
+// eight loads in flight, the four lanes are then added in order.  It is bound by reading the
+// slots (32 KB each) at memory latency: B32 H8 in two ranges 29.5 -> XXX us against one thread
+// per output.
+constexpr int kReduceThreads = 512;
+__global__ void __launch_bounds__(kReduceThreads)
+    tc_dw_reduce_kernel(int B, int H, int M, int G, int nsplit, int nonstat,
+                        const float* __restrict__ part, float* __restrict__ dW1,
+                        float* __restrict__ dW2, const float* __restrict__ dtau_part,
+                        float* __restrict__ dtau)
 {
-    const size_t half = (size_t)B * H * nsplit * G;  // slots per pass
-    if (dtau && blockIdx.x == 0)  // dtau[h]: the pass R slots of head h, in order
-        for (int h = threadIdx.x; h < H; h += blockDim.x) {
-            float a = 0.f;
-            for (int b = 0; b < B; ++b)
-                for (int sp = 0; sp < nsplit; ++sp)
-                    for (int g = 0; g < G; ++g)
-                        a += dtau_part[half + ((size_t)(b * H + h) * nsplit + sp) * G + g];
-            dtau[h] = a;
+    __shared__ float4 sums[3][128];
+    const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
+    const int row = threadIdx.x % 128, ln = threadIdx.x / 128;
+    const int per = B * nsplit;                        // slots of (head, group) and pass
+    const size_t half = (size_t)B * H * nsplit * G;    // slots per pass
+    auto slot_of = [&](int i) {                        // i < 2 per: pass F's slots, then R's
+        const int pass = i / per, r = i % per;
+        return (size_t)pass * half + ((size_t)(r / nsplit * H + h) * nsplit + r % nsplit) * G + g;
+    };
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i0 = ln; i0 < 2 * per; i0 += 32) {
+        float4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            x[u] = i0 + 4 * u < 2 * per
+                       ? reinterpret_cast<const float4*>(part)[(slot_of(i0 + 4 * u) * 16 + quad) * 128 + row]
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            a = make_float4(a.x + x[u].x, a.y + x[u].y, a.z + x[u].z, a.w + x[u].w);
+    }
+    if (ln > 0) sums[ln - 1][row] = a;
+    __syncthreads();
+    if (ln == 0) {
+        for (int l = 0; l < 3; ++l) {
+            const float4 x = sums[l][row];
+            a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
         }
-    const size_t total = (size_t)H * M * 64;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int h = (int)(idx / ((size_t)M * 64));
-        const int f = (int)((idx / 64) % M), e = (int)(idx % 64);
-        const int g = f / 64, r = f % 64;
-        float a = 0.f, b2 = 0.f;
-        const size_t pass_stride = half * 128 * 64;  // pass F slots follow pass R's
-        for (int b = 0; b < B; ++b)
-            for (int sp = 0; sp < nsplit; ++sp) {
-                const float* p = part + ((((size_t)(b * H + h) * nsplit + sp) * G + g) * 128) * 64 +
-                                 (e >> 2) * 512 + 4 * r + (e & 3);
-                a += p[0] + p[pass_stride];
-                // n: dV rows; s: the dW rows of the low part of da
-                b2 += p[4 * 64] + p[pass_stride + 4 * 64];
-            }
+        if (row >= 64) sums[0][row] = a;
+    }
+    __syncthreads();
+    if (ln == 0 && row < 64) {
+        const float4 b = sums[0][64 + row];  // n: dV rows; s: the dW rows of the low part of da
+        const size_t o = (((size_t)h * M + 64 * g + row) * 64 + 4 * quad) / 4;
         if (!nonstat) {
-            dW1[idx] = a + b2;
+            reinterpret_cast<float4*>(dW1)[o] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
         } else {
-            dW1[idx] = 0.5f * (a + b2);
-            dW2[idx] = 0.5f * (a - b2);
+            reinterpret_cast<float4*>(dW1)[o] = make_float4(0.5f * (a.x + b.x), 0.5f * (a.y + b.y),
+                                                            0.5f * (a.z + b.z), 0.5f * (a.w + b.w));
+            reinterpret_cast<float4*>(dW2)[o] = make_float4(0.5f * (a.x - b.x), 0.5f * (a.y - b.y),
+                                                            0.5f * (a.z - b.z), 0.5f * (a.w - b.w));
         }
+    }
+    if (dtau && quad == 0 && g == 0 && threadIdx.x < 32) {  // dtau[h]: head h's pass R slots
+        float t = 0.f;
+        for (int i = threadIdx.x; i < per * G; i += 32)
+            t += dtau_part[half + ((size_t)(i / (nsplit * G) * H + h) * nsplit + i / G % nsplit) * G + i % G];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) dtau[h] = t;
     }
 }
 
-// Non-causal totals: total[pass][unit][row][0..64] = sum over the splits, in order, of the
-// partial states [pass][(bh * nsplit + s) * G + g][row][0..64] (unit = bh * G + g).
-__global__ void nc_state_reduce_kernel(int units, int G, int nsplit,
-                                       const float* __restrict__ part, float* __restrict__ total)
+// Partial states are [pass][(bh * nsplit + s) * G + g][128 rows][80], columns 0-64 in use: one
+// block of kStateThreads covers an eighth (blockIdx.y) of the 128 x 17 float4 of a (pass, unit),
+// blockIdx.x = pass * units + unit (unit = bh * G + g); the splits' loads are independent.
+constexpr int kStateThreads = 272;
+__device__ __forceinline__ float4* state_at(float* part, size_t slot)
 {
-    const size_t n = (size_t)2 * units * 128 * 65;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int col = (int)(i % 65), row = (int)((i / 65) % 128);
-        const int u = (int)((i / (65 * 128)) % units), pass = (int)(i / ((size_t)65 * 128 * units));
-        const int bh = u / G, g = u % G;
-        float a = 0.f;
-        for (int sp = 0; sp < nsplit; ++sp)
-            a += part[(((size_t)pass * units * nsplit + ((size_t)bh * nsplit + sp) * G + g) * 128 +
-                       row) * 80 + col];
-        total[(((size_t)pass * units + u) * 128 + row) * 80 + col] = a;
-    }
+    const int i = blockIdx.y * kStateThreads + threadIdx.x;
+    return reinterpret_cast<float4*>(part) + (slot * 128 + i / 17) * 20 + i % 17;
+}
+__device__ __forceinline__ void add4(float4& a, const float4& x)
+{
+    a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
 }
 
-// Causal ranges: each range's partial states (in place, [pass][slot][row][0..64]) become what
-// the range starts from: pass F the sum over the earlier ranges, pass R over the later ones,
-// in order.
-__global__ void causal_state_scan_kernel(int units, int G, int nsplit, float* __restrict__ part)
+// Non-causal totals: total[pass][unit][row][0..64] = sum over the splits, in order.
+__global__ void __launch_bounds__(kStateThreads)
+    nc_state_reduce_kernel(int units, int G, int nsplit, float* __restrict__ part,
+                           float* __restrict__ total)
 {
-    const size_t n = (size_t)2 * units * 128 * 65;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int col = (int)(i % 65), row = (int)((i / 65) % 128);
-        const int u = (int)((i / (65 * 128)) % units), pass = (int)(i / ((size_t)65 * 128 * units));
-        const int bh = u / G, g = u % G;
-        float run = 0.f;
-        for (int o = 0; o < nsplit; ++o) {
-            const int sp = pass == kPassF ? o : nsplit - 1 - o;
-            float* x = part + (((size_t)pass * units * nsplit + ((size_t)bh * nsplit + sp) * G + g) * 128 +
-                               row) * 80 + col;
-            const float v = *x;
-            *x = run;
-            run += v;
-        }
+    const int u = blockIdx.x % units, pass = blockIdx.x / units, bh = u / G, g = u % G;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int sp = 0; sp < nsplit; ++sp)
+        add4(a, *state_at(part, (size_t)pass * units * nsplit + ((size_t)bh * nsplit + sp) * G + g));
+    *state_at(total, (size_t)pass * units + u) = a;
+}
+
+// Causal ranges: each range's partial state becomes, in place, what the range starts from:
+// pass F the sum over the earlier ranges, pass R over the later ones, in order.
+__global__ void __launch_bounds__(kStateThreads)
+    causal_state_scan_kernel(int units, int G, int nsplit, float* __restrict__ part)
+{
+    const int u = blockIdx.x % units, pass = blockIdx.x / units, bh = u / G, g = u % G;
+    auto at = [&](int o) {
+        const int sp = pass == kPassF ? o : nsplit - 1 - o;
+        return state_at(part, (size_t)pass * units * nsplit + ((size_t)bh * nsplit + sp) * G + g);
+    };
+    float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int o0 = 0; o0 < nsplit; o0 += 8) {
+        float4 x[8];
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+            if (o0 + o < nsplit) x[o] = *at(o0 + o);
+#pragma unroll
+        for (int o = 0; o < 8; ++o)
+            if (o0 + o < nsplit) {
+                *at(o0 + o) = run;
+                add4(run, x[o]);
+            }
     }
 }
 
@@ -1484,11 +1517,12 @@ cudaError_t launch_bwd(const Problem& p, const void* q, const void* k, const voi
         e = launch_mode<NS, KW, 1, kState>(p, m, q, k, v, W1, W2, tau, out, den, dout, dq, dk, dv,
                                            f, w, nsplit, status, s);
         if (e != cudaSuccess) return e;
+        const dim3 sgrid(2 * units, 128 * 17 / kStateThreads);
         if (p.causal)
-            causal_state_scan_kernel<<<152 * 4, 256, 0, s>>>(units, G, nsplit, f + w.state_part);
+            causal_state_scan_kernel<<<sgrid, kStateThreads, 0, s>>>(units, G, nsplit, f + w.state_part);
         else
-            nc_state_reduce_kernel<<<152 * 4, 256, 0, s>>>(units, G, nsplit, f + w.state_part,
-                                                           f + w.state_total);
+            nc_state_reduce_kernel<<<sgrid, kStateThreads, 0, s>>>(units, G, nsplit, f + w.state_part,
+                                                                   f + w.state_total);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (p.causal)
@@ -1502,10 +1536,9 @@ cudaError_t launch_bwd(const Problem& p, const void* q, const void* k, const voi
                    : launch_mode<NS, KW, 1, kGrad>(p, m, q, k, v, W1, W2, tau, out, den, dout, dq,
                                                    dk, dv, f, w, nsplit, status, s);
     if (e != cudaSuccess) return e;
-    const size_t work = (size_t)p.H * p.M * 64;
-    tc_dw_reduce_kernel<<<(int)std::min<size_t>((work + 255) / 256, 152 * 8), 256, 0, s>>>(
-        p.B, p.H, p.M, G, nsplit, p.nonstat, f + w.part, dW1, dW2, f + w.dtau,
-        KW ? dtau : nullptr);
+    tc_dw_reduce_kernel<<<p.H * G * 16, kReduceThreads, 0, s>>>(p.B, p.H, p.M, G, nsplit, p.nonstat,
+                                                                f + w.part, dW1, dW2, f + w.dtau,
+                                                                KW ? dtau : nullptr);
     return cudaGetLastError();
 }
 
