@@ -231,15 +231,9 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     const uint32_t partner = (uint32_t)rank ^ 1u;
 
     // A phase of `bar`, and the tensor-memory accesses ordered after it; `ph` is the caller's
-    // parity.  await: the issuer's thread; wwait: a whole compute warp (one verdict).
-    auto await = [&](uint64_t* bar, uint32_t& ph) -> bool {
-        const bool ok = bar_wait(bar, ph, &abort_flag, status);
-        ph ^= 1;
-        fence_after_sync();
-        return ok;
-    };
+    // parity.  Called by a whole warp (one verdict).
     auto wwait = [&](uint64_t* bar, uint32_t& ph) -> bool {
-        const bool ok = __all_sync(0xffffffffu, bar_wait(bar, ph, &abort_flag, status));
+        const bool ok = bar_wait_w(bar, ph, &abort_flag, status);
         ph ^= 1;
         fence_after_sync();
         return ok;
@@ -276,7 +270,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     auto issue_projection = [&](uint64_t dx, uint32_t col) {
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
-            mma_bf16(tm + col, adv(dx, ks * 32), adv(dW, ks * 32), I_PROJ, ks > 0);
+            wmma_bf16(tm + col, adv(dx, ks * 32), adv(dW, ks * 32), I_PROJ, ks > 0);
     };
     // features of this group into dst (K-major rows) from the projection at column tcol; this
     // thread: row t, frequencies 16 wg .. 16 wg + 15
@@ -424,11 +418,11 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         const uint64_t dAm = sdesc(a0, a1 - a0, 1024);
 #pragma unroll
         for (int ks = 0; ks < (NS ? 8 : 4); ++ks)  // K = P rows of W (s: the da block only)
-            mma_bf16(tm + T_X, adv(ks < 4 ? dA0 : dA1, (ks & 3) * 32), adv(dWmn, ks * 2048), I_KM64,
+            wmma_bf16(tm + T_X, adv(ks < 4 ? dA0 : dA1, (ks & 3) * 32), adv(dWmn, ks * 2048), I_KM64,
                      ks > 0);
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
-            mma_bf16(tm + T_DW, adv(dAm, ks * 2048), adv(d_x_mn, ks * 2048), I_MM64,
+            wmma_bf16(tm + T_DW, adv(dAm, ks * 2048), adv(d_x_mn, ks * 2048), I_MM64,
                      (dw_per_chunk ? ks > 0 : (!first || ks > 0)) ? 1u : 0u);
     };
     // dW rows of this chunk (lane = row of this group's projection) into the partial slot
@@ -467,7 +461,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     // ---- cluster exchange of the dq / dk / dv partials (CS = 2) ----
     // This CTA's receive region of exchange xi is free for the partner's next copies (issuer).
     auto signal_ready = [&](int xi) {
-        if (CS > 1) mbar_arrive_cluster(mapa(smem_u32(&xready[xi]), partner));
+        if (CS > 1 && elect_one()) mbar_arrive_cluster(mapa(smem_u32(&xready[xi]), partner));
     };
     // An exchange block holds 64 rows x 64 fp32 as eight pieces of 2 KB, one per warp (two row
     // halves x four column quarters): byte offset of 16-byte chunk j (0-3) of this lane's row
@@ -545,7 +539,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         if ((t >> 6) != rank) return true;  // uniform over a warp
         float v_[16];
         tmem_ld16(tm_row + col + 16 * wg, v_);
-        const bool ok = __all_sync(0xffffffffu, bar_wait(&xfull[xi], ph_xfull[xi], &abort_flag, status));
+        const bool ok = bar_wait_w(&xfull[xi], ph_xfull[xi], &abort_flag, status);
         ph_xfull[xi] ^= 1;
         tmem_wait_ld();
         if (!ok) return false;
@@ -615,10 +609,10 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     auto row_sum = [&](int r) { return (spart[r] + spart[128 + r]) + (spart[256 + r] + spart[384 + r]); };
     // TMA of one tile of chunk cn into shared memory, and of a chunk's rows into L2
     auto load_tile = [&](uint32_t dst, const CUtensorMap* map, int cn, uint64_t* bar) {
-        tma_load_3d(sb + dst, map, 0, cn * kC, bh, bar);
+        wtma_load_3d(sb + dst, map, 0, cn * kC, bh, bar);
     };
     auto to_l2 = [&](const __nv_bfloat16* p, int cn) {
-        prefetch_l2(p + base + (size_t)cn * kC * 64, (uint32_t)min(kC, N - cn * kC) * 128);
+        if (elect_one()) prefetch_l2(p + base + (size_t)cn * kC * 64, (uint32_t)min(kC, N - cn * kC) * 128);
     };
     // [D] (+)= A B over 128 rows of K (both MN-major), the state sums' form, N = 64, and the
     // c / ones column block (N = 16)
@@ -626,8 +620,8 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
             const uint32_t acc = (!first || ks > 0) ? 1u : 0u;
-            mma_bf16(tm + L::T_S, adv(dphi, ks * 2048), adv(dval, ks * 2048), I_MM64, acc);
-            mma_bf16(tm + L::T_S + 64, adv(dphi, ks * 2048),
+            wmma_bf16(tm + L::T_S, adv(dphi, ks * 2048), adv(dval, ks * 2048), I_MM64, acc);
+            wmma_bf16(tm + L::T_S + 64, adv(dphi, ks * 2048),
                      adv(dcol, (ks >> 2) * 2048 + (ks & 3) * 32), I_M16, acc);
         }
     };
@@ -661,15 +655,15 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
             relay_landings(n);
             __syncwarp();
         } else if (issuer) {
-            if (lane == 0) [&]() {
+            [&]() {
                 uint32_t p_tx = 0, p_rdy = 0, p_m0 = 0, p_m1 = 0, p_s = 0;
                 // q, k, v of a chunk complete on tx[0], dout and out on tg; each tile is loaded
                 // once its region is free
                 const int c0 = PASS == kPassF ? cbeg : cend - 1;
-                mbar_arrive_expect_tx(&tg, 2 * kTileBytes);
+                wmbar_arrive_expect_tx(&tg, 2 * kTileBytes);
                 load_tile(L::DO, &tmap_do, c0, &tg);
                 load_tile(L::O, &tmap_o, c0, &tg);
-                mbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
+                wmbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
                 load_tile(L::Q, &tmap_q, c0, &tx[0]);
                 load_tile(L::K, &tmap_k, c0, &tx[0]);
                 load_tile(L::V, &tmap_v, c0, &tx[0]);
@@ -677,97 +671,97 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                     const int c = PASS == kPassF ? cbeg + it : cend - 1 - it;
                     const int cn = PASS == kPassF ? c + 1 : c - 1;  // the next chunk, if any
                     const bool has_next = it + 1 < n;
-                    if (!await(&tx[0], p_tx) || !await(&rdy, p_rdy)) return;  // g; the previous rows are out of T_P, T_A
+                    if (!wwait(&tx[0], p_tx) || !wwait(&rdy, p_rdy)) return;  // g; the previous rows are out of T_P, T_A
                     issue_projection(dQ, L::T_P);
                     issue_projection(dK, L::T_D);
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)  // dA = g v^T
-                        mma_bf16(tm + L::T_A, adv(dG, ks * 32), adv(dV, ks * 32), I_KK128, ks > 0);
-                    mma_commit(&m0);
+                        wmma_bf16(tm + L::T_A, adv(dG, ks * 32), adv(dV, ks * 32), I_KK128, ks > 0);
+                    wmma_commit(&m0);
                     p_m0 ^= 1;
                     if (PASS == kPassF && has_next) {
-                        mbar_arrive_expect_tx(&tg, 2 * kTileBytes);
+                        wmbar_arrive_expect_tx(&tg, 2 * kTileBytes);
                         load_tile(L::DO, &tmap_do, cn, &tg);
                         load_tile(L::O, &tmap_o, cn, &tg);
-                        mbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
+                        wmbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
                     }
                     if (it + 2 < n) {  // the chunk after next into L2
                         const int c2 = PASS == kPassF ? c + 2 : c - 2;
                         to_l2(q, c2); to_l2(k, c2); to_l2(v, c2); to_l2(dout, c2); to_l2(outp, c2);
                     }
-                    if (!await(&rdy, p_rdy)) return;  // features (F: and the masked dA)
+                    if (!wwait(&rdy, p_rdy)) return;  // features (F: and the masked dA)
                     if (PASS == kPassF) {
                         // dphi(q) = dA phi(K) + g S^T; S += phi(K)^T v; z += phi(K)^T 1
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16_tmem_a(tm + L::T_D, tm + L::T_A + 32 * (ks >> 1) + 8 * (ks & 1),
+                            wmma_bf16_tmem_a(tm + L::T_D, tm + L::T_A + 32 * (ks >> 1) + 8 * (ks & 1),
                                             adv(dPKmn, ks * 2048), I_KM128, ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dG, ks * 32), adv(dSN, ks * 32), I_KK128, 1u);
-                        mma_commit(&m0);
+                            wmma_bf16(tm + L::T_D, adv(dG, ks * 32), adv(dSN, ks * 32), I_KK128, 1u);
+                        wmma_commit(&m0);
                         p_m0 ^= 1;
                         issue_state(dPKmn, dVmn, dC16, it == 0 && !seeded);
-                        mma_commit(&m1);
+                        wmma_commit(&m1);
                         if (kLate) signal_ready(0);  // DA2: the previous dq is finished
                         if (has_next) load_tile(L::K, &tmap_k, cn, &tx[0]);
-                        if (!await(&m1, p_m1)) return;
+                        if (!wwait(&m1, p_m1)) return;
                         if (!kLate) signal_ready(0);  // PK is free for the partner's dq partial
                         if (has_next) load_tile(L::V, &tmap_v, cn, &tx[0]);
-                        if (!await(&rdy, p_rdy)) return;  // da
+                        if (!wwait(&rdy, p_rdy)) return;  // da
                         issue_back(sb + L::PQ, sb + L::PQ + 16384, dQmn, it == 0);
-                        mma_commit(&m0);
-                        if (!await(&m0, p_m0)) return;
+                        wmma_commit(&m0);
+                        if (!wwait(&m0, p_m0)) return;
                         if (has_next) load_tile(L::Q, &tmap_q, cn, &tx[0]);
                     } else {
-                        if (kLate) mbar_arrive(&fin);
+                        if (kLate && elect_one()) mbar_arrive(&fin);
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {  // A = phi(Q) phi(K)^T
                             const uint32_t kofs = (ks >> 2) * 16384 + (ks & 3) * 32;
-                            mma_bf16(tm + L::T_D, adv(dPQ, kofs), adv(dPK, kofs), I_KK128, ks > 0);
+                            wmma_bf16(tm + L::T_D, adv(dPQ, kofs), adv(dPK, kofs), I_KK128, ks > 0);
                         }
-                        mma_commit(&m0);
+                        wmma_commit(&m0);
                         p_m0 ^= 1;
-                        if (!await(&rdy, p_rdy)) return;  // the masked dA and A
+                        if (!wwait(&rdy, p_rdy)) return;  // the masked dA and A
                         // n: u, w of k again for the chain rule; dphi(k) = dA^T phi(Q) + v R^T;
                         // dv = A^T g + phi(K) R; then R += phi(Q)^T g; r += phi(Q)^T c
                         if (NS) issue_projection(dK, L::T_P);
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dDAmn, ks * 2048), adv(dPQmn, ks * 2048), I_MM128,
+                            wmma_bf16(tm + L::T_D, adv(dDAmn, ks * 2048), adv(dPQmn, ks * 2048), I_MM128,
                                      ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dV, ks * 32), adv(dSN, ks * 32), I_KK128, 1u);
+                            wmma_bf16(tm + L::T_D, adv(dV, ks * 32), adv(dSN, ks * 32), I_KK128, 1u);
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16(tm + T_DV, adv(dAmn, ks * 2048), adv(dGmn, ks * 2048), I_MM64,
+                            wmma_bf16(tm + T_DV, adv(dAmn, ks * 2048), adv(dGmn, ks * 2048), I_MM64,
                                      ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
+                            wmma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
                                      adv(dSNmn, ks * 2048), I_KM64, 1u);
-                        mma_commit(&m0);
+                        wmma_commit(&m0);
                         p_m0 ^= 1;
                         issue_state(dPQmn, dGmn, dC16, it == 0 && !seeded);
-                        mma_commit(&m1);
+                        wmma_commit(&m1);
                         if (kLate) signal_ready(1);  // XR: the previous dk is finished
-                        if (!await(&m1, p_m1)) return;
+                        if (!wwait(&m1, p_m1)) return;
                         signal_ready(0);  // DA2 is free for the partner's dv partial
-                        if (!await(&rdy, p_rdy)) return;  // da
+                        if (!wwait(&rdy, p_rdy)) return;  // da
                         issue_back(sb + L::PK, sb + L::PK + 16384, dKmn, it == 0);
-                        mma_commit(&m0);
+                        wmma_commit(&m0);
                         if (has_next) {  // Q, V, DO, O are free
-                            mbar_arrive_expect_tx(&tg, 2 * kTileBytes);
+                            wmbar_arrive_expect_tx(&tg, 2 * kTileBytes);
                             load_tile(L::DO, &tmap_do, cn, &tg);
                             load_tile(L::O, &tmap_o, cn, &tg);
-                            mbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
+                            wmbar_arrive_expect_tx(&tx[0], 3 * kTileBytes);
                             load_tile(L::Q, &tmap_q, cn, &tx[0]);
                             load_tile(L::V, &tmap_v, cn, &tx[0]);
                         }
-                        if (!await(&m0, p_m0)) return;
+                        if (!wwait(&m0, p_m0)) return;
                         if (!kLate) signal_ready(1);  // PK is free for the partner's dk partial
-                        if (KW && !await(&srdy, p_s)) return;  // dk rows have read the k tile
+                        if (KW && !wwait(&srdy, p_s)) return;  // dk rows have read the k tile
                         if (has_next) load_tile(L::K, &tmap_k, cn, &tx[0]);
                     }
                 }
@@ -917,25 +911,25 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         const uint32_t pb[2] = {L::PQ, L::PK}, tb[2] = {L::T_P, L::T_A};
         if (relay) {
         } else if (issuer) {
-            if (lane == 0) [&]() {
+            [&]() {
                 uint32_t p_tx[2] = {0, 0}, p_tv[3] = {0, 0, 0}, p_rdy = 0, p_m1 = 0;
                 auto load_x = [&](int i) {
-                    mbar_arrive_expect_tx(&tx[i & 1], kTileBytes);
+                    wmbar_arrive_expect_tx(&tx[i & 1], kTileBytes);
                     load_tile(xb[i & 1], fq ? &tmap_q : &tmap_k, cbeg + i, &tx[i & 1]);
                 };
                 auto load_v = [&](int i) {
-                    mbar_arrive_expect_tx(&tv[i % 3], kTileBytes);
+                    wmbar_arrive_expect_tx(&tv[i % 3], kTileBytes);
                     load_tile(vb[i % 3], &tmap_v, cbeg + i, &tv[i % 3]);
                 };
                 auto load_g = [&](int i) {
-                    mbar_arrive_expect_tx(&tg, 2 * kTileBytes);
+                    wmbar_arrive_expect_tx(&tg, 2 * kTileBytes);
                     load_tile(L::DO, &tmap_do, cbeg + i, &tg);
                     load_tile(L::O, &tmap_o, cbeg + i, &tg);
                 };
                 auto project = [&](int i) {
-                    if (!await(&tx[i & 1], p_tx[i & 1])) return false;
+                    if (!wwait(&tx[i & 1], p_tx[i & 1])) return false;
                     issue_projection(sdesc(sb + xb[i & 1], 16, 1024), tb[i & 1]);
-                    mma_commit(&mt[i & 1]);
+                    wmma_commit(&mt[i & 1]);
                     return true;
                 };
                 for (int i = 0; i < min(2, n); ++i) load_x(i);
@@ -953,21 +947,21 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                         }
                     }
                     if (i + 1 < n && !project(i + 1)) return;
-                    if (!await(&rdy, p_rdy)) return;  // features (and g) of chunk i
+                    if (!wwait(&rdy, p_rdy)) return;  // features (and g) of chunk i
                     if (i + 2 < n) load_x(i + 2);
                     if (fq && i + 1 < n) load_g(i + 1);
-                    if (!fq && !await(&tv[i % 3], p_tv[i % 3])) return;
+                    if (!fq && !wwait(&tv[i % 3], p_tv[i % 3])) return;
                     // the sums of chunk i - 1 (waited for before the next commit on m1, so
                     // that no phase of it is missed): its v buffer is free
-                    if (i > 0 && !await(&m1, p_m1)) return;
+                    if (i > 0 && !wwait(&m1, p_m1)) return;
                     if (!fq && i + 2 < n) load_v(i + 2);
                     // [S | z] += phi(K)^T [V | 1]  or  [R | r] += phi(Q)^T [G | c]
                     issue_state(sdesc(sb + pb[i & 1], 16384, 1024),
                                 sdesc(sb + (fq ? gb[i & 1] : vb[i % 3]), 16384, 1024),
                                 sdesc(sb + cb[i & 1], 16, 1024), i == 0);
-                    mma_commit(&m1);
+                    wmma_commit(&m1);
                 }
-                if (n > 0) await(&m1, p_m1);
+                if (n > 0) wwait(&m1, p_m1);
             }();
             __syncwarp();
         } else {
@@ -1050,14 +1044,14 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                 relay_landings(n);
                 __syncwarp();
             } else if (issuer) {
-                if (lane == 0) [&]() {
+                [&]() {
                     uint32_t p_tx[2] = {0, 0}, p_rdy = 0, p_rdyg = 0, p_m1 = 0;
                     auto load_x = [&](int i) {
-                        mbar_arrive_expect_tx(&tx[i & 1], kTileBytes);
+                        wmbar_arrive_expect_tx(&tx[i & 1], kTileBytes);
                         load_tile(qb[i & 1], &tmap_q, cbeg + i, &tx[i & 1]);
                     };
                     auto load_g = [&](int i) {
-                        mbar_arrive_expect_tx(&tg, 2 * kTileBytes);
+                        wmbar_arrive_expect_tx(&tg, 2 * kTileBytes);
                         load_tile(L::DO, &tmap_do, cbeg + i, &tg);
                         load_tile(L::O, &tmap_o, cbeg + i, &tg);
                     };
@@ -1069,29 +1063,29 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                             const int c2 = cbeg + i + 2;
                             to_l2(q, c2); to_l2(dout, c2); to_l2(outp, c2);
                         }
-                        if (!await(&rdyg, p_rdyg)) return;  // g of chunk i; its dout, out are read
+                        if (!wwait(&rdyg, p_rdyg)) return;  // g of chunk i; its dout, out are read
                         if (i + 1 < n) load_g(i + 1);
-                        if (!await(&tx[i & 1], p_tx[i & 1])) return;
+                        if (!wwait(&tx[i & 1], p_tx[i & 1])) return;
                         // the projection, and dphi(q) = g S^T (+ c z in the chain rule)
                         issue_projection(sdesc(sb + qb[i & 1], 16, 1024), L::T_P);
                         const uint64_t dGi = sdesc(sb + gb[i & 1], 16, 1024);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dGi, ks * 32), adv(dSN, ks * 32), I_KK128, ks > 0);
+                            wmma_bf16(tm + L::T_D, adv(dGi, ks * 32), adv(dSN, ks * 32), I_KK128, ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dGi, ks * 32), adv(dSL, ks * 32), I_KK128, 1u);
-                        mma_commit(&m0);
+                            wmma_bf16(tm + L::T_D, adv(dGi, ks * 32), adv(dSL, ks * 32), I_KK128, 1u);
+                        wmma_commit(&m0);
                         if (i > 0) {
-                            if (!await(&m1, p_m1)) return;
+                            if (!wwait(&m1, p_m1)) return;
                             if (i + 1 < n) load_x(i + 1);
                         }
-                        if (!await(&rdy, p_rdy)) return;  // da; chunk i - 1's rows are finished
+                        if (!wwait(&rdy, p_rdy)) return;  // da; chunk i - 1's rows are finished
                         if (CS > 1 && i > 0) {
                             signal_ready(0);
                         }
                         issue_back(sb + L::PQ, da1, sdesc(sb + qb[i & 1], 16384, 1024), i == 0);
-                        mma_commit(&m1);
+                        wmma_commit(&m1);
                     }
                 }();
                 __syncwarp();
@@ -1131,11 +1125,11 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                 relay_landings(n);
                 __syncwarp();
             } else if (issuer) {
-                if (lane == 0) [&]() {
+                [&]() {
                     uint32_t p_tx[2] = {0, 0}, p_rdy = 0, p_m1 = 0, p_s = 0;
                     auto load_x = [&](int i) {
                         const int b = i % NB;
-                        mbar_arrive_expect_tx(&tx[b], 2 * kTileBytes);
+                        wmbar_arrive_expect_tx(&tx[b], 2 * kTileBytes);
                         load_tile(kb[b], &tmap_k, cbeg + i, &tx[b]);
                         load_tile(vb[b], &tmap_v, cbeg + i, &tx[b]);
                     };
@@ -1148,40 +1142,40 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                             to_l2(k, cbeg + i + 2);
                             to_l2(v, cbeg + i + 2);
                         }
-                        if (!await(&tx[b], p_tx[b])) return;
+                        if (!wwait(&tx[b], p_tx[b])) return;
                         // the projection, and dphi(k) = v R^T (+ r in the chain rule)
                         issue_projection(sdesc(sb + kb[b], 16, 1024), L::T_P);
                         const uint64_t dVi = sdesc(sb + vb[b], 16, 1024);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dVi, ks * 32), adv(dSN, ks * 32), I_KK128, ks > 0);
+                            wmma_bf16(tm + L::T_D, adv(dVi, ks * 32), adv(dSN, ks * 32), I_KK128, ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
-                            mma_bf16(tm + L::T_D, adv(dVi, ks * 32), adv(dSL, ks * 32), I_KK128, 1u);
-                        mma_commit(&m0);
+                            wmma_bf16(tm + L::T_D, adv(dVi, ks * 32), adv(dSL, ks * 32), I_KK128, 1u);
+                        wmma_commit(&m0);
                         if (NB == 2 && i > 0) {  // chunk i - 1's buffers: its MMAs and rows done
-                            if (!await(&m1, p_m1)) return;
-                            if (!await(&srdy, p_s)) return;
+                            if (!wwait(&m1, p_m1)) return;
+                            if (!wwait(&srdy, p_s)) return;
                             if (i + 1 < n) load_x(i + 1);
                         }
-                        if (!await(&rdy, p_rdy)) return;  // phi(k), da; chunk i - 1's rows finished
+                        if (!wwait(&rdy, p_rdy)) return;  // phi(k), da; chunk i - 1's rows finished
                         if (CS > 1 && i > 0) {
                             signal_ready(0);
                             signal_ready(1);
                         }
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)  // dv = phi(K) R
-                            mma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
+                            wmma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
                                      adv(dSNmn, ks * 2048), I_KM64, ks > 0);
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
+                            wmma_bf16(tm + T_DV, adv(dPK, (ks >> 2) * 16384 + (ks & 3) * 32),
                                      adv(dSLmn, ks * 2048), I_KM64, 1u);
                         issue_back(sb + L::GT, da1, sdesc(sb + kb[b], 16384, 1024), i == 0);
-                        mma_commit(&m1);
+                        wmma_commit(&m1);
                         if (NB == 1) {
-                            if (!await(&m1, p_m1)) return;
-                            if (!await(&srdy, p_s)) return;
+                            if (!wwait(&m1, p_m1)) return;
+                            if (!wwait(&srdy, p_s)) return;
                             if (i + 1 < n) load_x(i + 1);
                         }
                     }

@@ -132,6 +132,56 @@ __device__ __forceinline__ void mma_commit(void* mbar)
         : "memory");
 }
 
+// ---- the same, issued by a whole converged warp ------------------------------------------
+// One elected lane executes the operation; the operands (descriptors, addresses) are warp-
+// uniform, so they can stay in uniform registers.  A lone thread of a diverged warp issued
+// an MMA every 130-190 cycles and a tile load every 480 (GB300, backward kernel), slower than
+// the tensor core works.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(r)::"memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ void wmma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                          uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void wmma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                                 uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void wmma_commit(void* mbar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(
+            smem_u32(mbar))
+        : "memory");
+}
+
 // 32 lanes x 32 bits, 16 consecutive columns: thread i of the warp receives lane
 // (base lane + i), columns col .. col+15.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
@@ -279,6 +329,23 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int 
         : "memory");
 }
 
+__device__ __forceinline__ void wtma_load_3d(uint32_t dst, const void* tmap, int c0, int c1, int c2,
+                                             void* mbar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, "
+        "{%2, %3, %4}], [%5];\n\t}\n" ::"r"(dst),
+        "l"((uint64_t)tmap), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(mbar))
+        : "memory");
+}
+
+__device__ __forceinline__ void wmbar_arrive_expect_tx(void* mbar, uint32_t bytes)
+{
+    if (elect_one()) mbar_arrive_expect_tx(mbar, bytes);
+}
+
 // TMA: store a 3-D tile from shared memory (same tensor-map layout as the load), tracked by
 // the issuing thread's bulk groups.  Rows outside the tensor are not written.
 __device__ __forceinline__ void tma_store_3d(const void* tmap, uint32_t src, int c0, int c1, int c2)
@@ -334,6 +401,11 @@ __device__ __forceinline__ void tma_prefetch_3d(const void* tmap, int c0, int c1
                      (uint64_t)tmap),
                  "r"(c0), "r"(c1), "r"(c2)
                  : "memory");
+}
+
+__device__ __forceinline__ void wtma_prefetch_3d(const void* tmap, int c0, int c1, int c2)
+{
+    if (elect_one()) tma_prefetch_3d(tmap, c0, c1, c2);
 }
 
 // ---- register split between warpgroups ---------------------------------------------------

@@ -235,41 +235,41 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
         // the diagnostic stall ran out during set-up: nothing is issued
     } else if (warp == L::TMAV) {
         // ================= TMA producer: v =================
-        if (lane == 0) {
+        {
             uint32_t ph_vfree[2] = {0, 0};
             for (int c = 0; c < ce; ++c) {
                 const int vb = c & 1;
                 if (c >= 2) {
-                    if (!bar_wait(&bars.v_free[vb], ph_vfree[vb], &abort_flag, status)) break;
+                    if (!bar_wait_w(&bars.v_free[vb], ph_vfree[vb], &abort_flag, status)) break;
                     ph_vfree[vb] ^= 1;
                 }
-                if (c + 2 < ce && rank == 0) tma_prefetch_3d(&tmap_v, 0, (c + 2) * kC, bh);
-                mbar_arrive_expect_tx(&bars.v_full[vb], kTileBytes);
-                tma_load_3d(sb + (vb ? L::V1 : L::V0), &tmap_v, 0, c * kC, bh, &bars.v_full[vb]);
+                if (c + 2 < ce && rank == 0) wtma_prefetch_3d(&tmap_v, 0, (c + 2) * kC, bh);
+                wmbar_arrive_expect_tx(&bars.v_full[vb], kTileBytes);
+                wtma_load_3d(sb + (vb ? L::V1 : L::V0), &tmap_v, 0, c * kC, bh, &bars.v_full[vb]);
             }
         }
     } else if (warp == kWarpTMA) {
         // ================= TMA producer: q, k =================
         // Main chunks: q -> X0, k -> X1.  k-only prefix chunks alternate k between X1 and
         // X0, so the next tile loads while the current one is projected.
-        if (lane == 0) {
+        {
             uint32_t ph_xfree[2] = {0, 0};
             bool used_x[2] = {false, false};
             auto load = [&](int b, const CUtensorMap* map, int t0) -> bool {
                 if (used_x[b]) {
-                    if (!bar_wait(&bars.x_free[b], ph_xfree[b], &abort_flag, status)) return false;
+                    if (!bar_wait_w(&bars.x_free[b], ph_xfree[b], &abort_flag, status)) return false;
                     ph_xfree[b] ^= 1;
                 }
                 used_x[b] = true;
-                mbar_arrive_expect_tx(&bars.x_full[b], kTileBytes);
-                tma_load_3d(sb + (b ? L::X1 : L::X0), map, 0, t0, bh, &bars.x_full[b]);
+                wmbar_arrive_expect_tx(&bars.x_full[b], kTileBytes);
+                wtma_load_3d(sb + (b ? L::X1 : L::X0), map, 0, t0, bh, &bars.x_full[b]);
                 return true;
             };
             for (int c = 0; c < ce; ++c) {
                 const int t0 = c * kC;
                 if (c + 1 < ce && rank == 0) {  // next chunk's tiles into L2 (once per pair)
-                    if (c + 1 >= cb) tma_prefetch_3d(&tmap_q, 0, t0 + kC, bh);
-                    tma_prefetch_3d(&tmap_k, 0, t0 + kC, bh);
+                    if (c + 1 >= cb) wtma_prefetch_3d(&tmap_q, 0, t0 + kC, bh);
+                    wtma_prefetch_3d(&tmap_k, 0, t0 + kC, bh);
                 }
                 if (c >= cb) {
                     if (!load(0, &tmap_q, t0) || !load(1, &tmap_k, t0)) break;
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
             }
         }
     } else if (warp == kWarpMMA || warp == L::PROJ) {
-        // ================= MMA issue (one thread per role) =================
-        if (lane == 0) {
+        // ================= MMA issue (one warp per role) =================
+        {
             constexpr uint32_t I_PROJ = idesc_bf16(128, 64, 0, 0);
             constexpr uint32_t I_QK = idesc_bf16(128, 128, 0, 0);
             constexpr uint32_t I_QS = idesc_bf16(128, 80, 0, 1);
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
             bool ok = true;
             auto wait = [&](uint64_t* bar, uint32_t& ph) {
                 if (!ok) return;
-                ok = bar_wait(bar, ph, &abort_flag, status);
+                ok = bar_wait_w(bar, ph, &abort_flag, status);
                 ph ^= 1;
             };
             // Descriptors are built once; an operand K step adds its byte offset / 16 to
@@ -313,12 +313,12 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                             const uint64_t wd = adv(d_w, hf * 8192);
 #pragma unroll
                             for (int ks = 0; ks < 4; ++ks)
-                                mma_bf16(tm + L::T_P, adv(d_x[buf], ks * 32), adv(wd, ks * 32),
+                                wmma_bf16(tm + L::T_P, adv(d_x[buf], ks * 32), adv(wd, ks * 32),
                                          I_PROJ, ks > 0);
-                            mma_commit(&bars.p_full);
+                            wmma_commit(&bars.p_full);
                             ++nproj;
                         }
-                        mma_commit(&bars.x_free[buf]);
+                        wmma_commit(&bars.x_free[buf]);
                     }
                 }
             } else {
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                         fence_after_sync();
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
-                            mma_bf16_tmem_a(tm + t_o, tm + L::T_Q + 8 * ks, adv(d_sx, ks * 2048),
+                            wmma_bf16_tmem_a(tm + t_o, tm + L::T_Q + 8 * ks, adv(d_sx, ks * 2048),
                                             I_QS, ks > 0);
                     }
                     wait(&bars.phik_full, ph_phik);
@@ -353,11 +353,11 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                     if (main) {
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)  // A = phi(Q) phi(K)^T, K = 128 features
-                            mma_bf16_tmem_a(tm + L::T_A, tm + L::T_Q + 8 * ks,
+                            wmma_bf16_tmem_a(tm + L::T_A, tm + L::T_Q + 8 * ks,
                                             adv(d_pk, (ks >> 2) * 16384 + (ks & 3) * 32), I_QK,
                                             ks > 0);
-                        mma_commit(&bars.phiq_free);  // phi(Q) no longer read
-                        mma_commit(&bars.attn_done);
+                        wmma_commit(&bars.phiq_free);  // phi(Q) no longer read
+                        wmma_commit(&bars.attn_done);
                     }
                     wait(&bars.v_full[c & 1], ph_vfull[c & 1]);
                     if (!ok) break;
@@ -365,12 +365,12 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                     const uint32_t acc_s = c > 0 ? 1u : 0u;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)  // [S | z] += phi(K)^T [V | 1], K = 128 tokens
-                        mma_bf16(tm + L::T_S, adv(d_pk_mn, ks * 2048), adv(vd, ks * 2048), I_KV,
+                        wmma_bf16(tm + L::T_S, adv(d_pk_mn, ks * 2048), adv(vd, ks * 2048), I_KV,
                                  (acc_s | (ks > 0)) ? 1u : 0u);
-                    mma_commit(&bars.phik_free);  // phi(K) no longer read
-                    if (main || c == cb - 1) mma_commit(&bars.s_done);
+                    wmma_commit(&bars.phik_free);  // phi(K) no longer read
+                    if (main || c == cb - 1) wmma_commit(&bars.s_done);
                     if (!main) {
-                        mma_commit(&bars.v_free[c & 1]);
+                        wmma_commit(&bars.v_free[c & 1]);
                         continue;
                     }
                     wait(&bars.a_ready, ph_aready);
@@ -378,10 +378,10 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                     fence_after_sync();
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)  // keys 16ks..16ks+15: bf16 A columns
-                        mma_bf16_tmem_a(tm + t_o, tm + L::T_A + 64 * (ks >> 2) + 8 * (ks & 3),
+                        wmma_bf16_tmem_a(tm + t_o, tm + L::T_A + 64 * (ks >> 2) + 8 * (ks & 3),
                                         adv(vd, ks * 2048), I_AV, 1u);
-                    mma_commit(&bars.o_ready);
-                    mma_commit(&bars.v_free[c & 1]);
+                    wmma_commit(&bars.o_ready);
+                    wmma_commit(&bars.v_free[c & 1]);
                 }
             }
         }

@@ -159,27 +159,27 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
     if (warp == kWarpTMA) {
         // q or k tiles (v has its own thread: a v buffer frees late, after the state MMA two
         // chunks back, and must not hold up the next projection's tile)
-        if (lane == 0) {
+        {
             uint32_t ph_x[2] = {0, 0};
             for (int i = 0; i < nc; ++i) {
                 const int b = i & 1, t0 = (c0 + i) * kC;
-                if (i + kAhead < nc) tma_prefetch_3d(&tmap_x, 0, t0 + kAhead * kC, bh);  // into L2
+                if (i + kAhead < nc) wtma_prefetch_3d(&tmap_x, 0, t0 + kAhead * kC, bh);  // into L2
                 if (i >= 2) {
-                    if (!bar_wait(&bars.x_free[b], ph_x[b], &abort_flag, status)) break;
+                    if (!bar_wait_w(&bars.x_free[b], ph_x[b], &abort_flag, status)) break;
                     ph_x[b] ^= 1;
                 }
-                mbar_arrive_expect_tx(&bars.x_full[b], kTileBytes);
-                tma_load_3d(sb + (b ? L::X1 : L::X0), &tmap_x, 0, t0, bh, &bars.x_full[b]);
+                wmbar_arrive_expect_tx(&bars.x_full[b], kTileBytes);
+                wtma_load_3d(sb + (b ? L::X1 : L::X0), &tmap_x, 0, t0, bh, &bars.x_full[b]);
             }
         }
     } else if (warp == kWarpMMA || warp == kWarpCons) {
-        if (lane == 0) {
+        {
             constexpr uint32_t I_PROJ = idesc_bf16(128, L::P, 0, 0);
             constexpr uint32_t I_KV = idesc_bf16(128, 80, 1, 1);
             constexpr uint32_t I_QS = idesc_bf16(128, 80, 0, 0);
             bool ok = true;
             auto wait = [&](uint64_t* bar, uint32_t parity) {
-                if (ok) ok = bar_wait(bar, parity, &abort_flag, status);
+                if (ok) ok = bar_wait_w(bar, parity, &abort_flag, status);
             };
             auto adv = [](uint64_t d, uint32_t bytes) { return d + (bytes >> 4); };
             const uint64_t d_x[2] = {sdesc(sb + L::X0, 16, 1024), sdesc(sb + L::X1, 16, 1024)};
@@ -200,10 +200,10 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                     fence_after_sync();
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)  // K = 128 tokens
-                        mma_bf16(tm + L::T_S + 80 * g, adv(d_pb_mn[fb], ks * 2048),
+                        wmma_bf16(tm + L::T_S + 80 * g, adv(d_pb_mn[fb], ks * 2048),
                                  adv(d_v[ib], ks * 2048), I_KV, (i > 0 || ks > 0) ? 1u : 0u);
-                    mma_commit(&bars.phi_free[fb]);
-                    if (g == G - 1) mma_commit(&bars.v_free[ib]);
+                    wmma_commit(&bars.phi_free[fb]);
+                    if (g == G - 1) wmma_commit(&bars.v_free[ib]);
                 } else {
                     if (g == 0 && i >= 2) wait(&bars.o_free[ib], ((i - 2) >> 1) & 1);
                     if (!ok) return;
@@ -212,12 +212,12 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {  // K = 128 features of group g
                         const uint32_t kofs = (ks >> 2) * 16384 + (ks & 3) * 32;
-                        mma_bf16(tm + to, adv(d_pb[fb], kofs),
+                        wmma_bf16(tm + to, adv(d_pb[fb], kofs),
                                  adv(d_sx, g * L::SX_GROUP + (ks >> 2) * L::SX_BLOCK + (ks & 3) * 32),
                                  I_QS, (g > 0 || ks > 0) ? 1u : 0u);
                     }
-                    mma_commit(&bars.phi_free[fb]);
-                    if (g == G - 1) mma_commit(&bars.o_full[ib]);
+                    wmma_commit(&bars.phi_free[fb]);
+                    if (g == G - 1) wmma_commit(&bars.o_full[ib]);
                 }
             };
             // Projections and the state / output MMAs come from two threads, so a late v
@@ -232,14 +232,14 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                 const uint64_t wd = adv(d_w, g * L::P * 128);
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_bf16(tm + (pb ? L::T_P1 : L::T_P0), adv(d_x[ib], ks * 32), adv(wd, ks * 32),
+                    wmma_bf16(tm + (pb ? L::T_P1 : L::T_P0), adv(d_x[ib], ks * 32), adv(wd, ks * 32),
                              I_PROJ, ks > 0);
-                mma_commit(&bars.p_full[pb]);
-                if (g == G - 1) mma_commit(&bars.x_free[ib]);
+                wmma_commit(&bars.p_full[pb]);
+                if (g == G - 1) wmma_commit(&bars.x_free[ib]);
             }
             if (warp == kWarpCons) {
                 for (int j = 0; j < njobs && ok; ++j) consume(j);
-                if (ok && MODE == kState) mma_commit(&bars.state_done);
+                if (ok && MODE == kState) wmma_commit(&bars.state_done);
             }
         }
     } else if (warp < kWarpEW) {
@@ -306,18 +306,18 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
         const uint32_t tm_row = tm + ((uint32_t)(32 * quad) << 16);
         if (MODE == kState) {
             if (warp == kWarpEW + 3) {
-                // v tiles (tmap_v), issued by this warp's lane 0 before it joins the epilogue
-                if (lane == 0) {
+                // v tiles (tmap_v), issued by this warp before it joins the epilogue
+                {
                     uint32_t ph_v[2] = {0, 0};
                     for (int i = 0; i < nc; ++i) {
                         const int b = i & 1, t0 = (c0 + i) * kC;
-                        if (i + kAhead < nc) tma_prefetch_3d(&tmap_v, 0, t0 + kAhead * kC, bh);
+                        if (i + kAhead < nc) wtma_prefetch_3d(&tmap_v, 0, t0 + kAhead * kC, bh);
                         if (i >= 2) {
-                            if (!bar_wait(&bars.v_free[b], ph_v[b], &abort_flag, status)) break;
+                            if (!bar_wait_w(&bars.v_free[b], ph_v[b], &abort_flag, status)) break;
                             ph_v[b] ^= 1;
                         }
-                        mbar_arrive_expect_tx(&bars.v_full[b], kTileBytes);
-                        tma_load_3d(sb + (b ? L::V1 : L::V0), &tmap_v, 0, t0, bh, &bars.v_full[b]);
+                        wmbar_arrive_expect_tx(&bars.v_full[b], kTileBytes);
+                        wtma_load_3d(sb + (b ? L::V1 : L::V0), &tmap_v, 0, t0, bh, &bars.v_full[b]);
                     }
                 }
                 __syncwarp();

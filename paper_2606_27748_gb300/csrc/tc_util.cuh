@@ -152,6 +152,14 @@ __device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity, volatil
     }
 }
 
+// bar_wait by a whole converged warp: one verdict for all its lanes, so that warp-wide issue
+// (wmma_bf16 and the like) never runs with a lane missing.
+__device__ __forceinline__ bool bar_wait_w(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                           int* status)
+{
+    return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, status));
+}
+
 // The diagnostic stall of flex_debug_stall: when the workspace header asks for it
 // (stall_cycles > 0), one thread of the CTA waits that many clocks at most on `bar`, an
 // mbarrier that nothing arrives on, so the wait runs out exactly as a wait for a lost
