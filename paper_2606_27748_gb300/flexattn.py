@@ -45,6 +45,8 @@ _lib = None
 def load(path: str = LIBRARY) -> ctypes.CDLL:
     """Open the library (once).  Raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -102,12 +104,13 @@ def _ptr(t):
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("tensors must be contiguous CUDA tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()  # (an int: the declared argument types make it a pointer)
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None:  # the current device's current stream, without building a Stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def shape_of(x: torch.Tensor, W1: torch.Tensor) -> FlexShape:
