@@ -115,7 +115,7 @@ __global__ void featmap_kernel(Problem p, const T* x, const float* W1, const flo
 // up to 8 SMs instead of one.  Measured on GB300 against one CTA per sequence with
 // one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 23 us, bf16 n B32 H4
 // N1024 d32 M16 477 -> 104 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
-// 8.58 -> 0.51 ms (6.7 of the 78 TFLOP/s fp32 peak: per chunk the products run between
+// 8.58 -> 0.36 ms (9.5 of the 78 TFLOP/s fp32 peak: per chunk the products run between
 // barriers with one backward CTA per SM, so load latency and the barriers bound it).
 struct Plan {
     int T;              // tokens per chunk (a multiple of 8, at most kMaxT)
@@ -142,6 +142,7 @@ template <int NC>
 __device__ __forceinline__ void mm_nt(const float* a, int pa, const float* b, int pb, int K,
                                       float (&acc)[4][NC])
 {
+#pragma unroll 1
     for (int k = 0; k < K; k += 4) {
         float4 x[4], y[NC];
 #pragma unroll
@@ -165,6 +166,7 @@ __device__ __forceinline__ void mm_nt(const float* a, int pa, const float* b, in
 __device__ __forceinline__ void mm_nn(const float* a, int pa, const float* b, int o1, int o2,
                                       int o3, int step, int K, float (&acc)[4][4])
 {
+#pragma unroll 1
     for (int k = 0; k < K; k += 4, b += step) {
         float4 x[4], y[4];
 #pragma unroll
@@ -222,35 +224,59 @@ template <bool NS>
 __device__ void stage_projection(const Problem& p, const Plan& L, const float* W1,
                                  const float* W2, int h, int g, float* W)
 {
-    const int d = p.d, dq = d / 4;
-    for (int idx = threadIdx.x; idx < L.KP * dq; idx += kThreads) {
-        const int row = idx / dq, e = 4 * (idx % dq), c = row / L.CT, x = row % L.CT;
-        const int f = g * L.MG + 2 * x + (NS ? c >> 1 : c);
-        float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (f < p.M) {
-            const size_t o = ((size_t)h * p.M + f) * d + e;
-            w = *reinterpret_cast<const float4*>(W1 + o);
-            if (NS) {
-                const float4 w2 = *reinterpret_cast<const float4*>(W2 + o);
-                const float s = (c & 1) ? -1.f : 1.f;
-                w = make_float4(0.5f * (w.x + s * w2.x), 0.5f * (w.y + s * w2.y),
-                                0.5f * (w.z + s * w2.z), 0.5f * (w.w + s * w2.w));
+    const int d = p.d, dq = d / 4, total = L.KP * dq;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * kThreads) {  // four loads in flight
+        float4 w[4], w2[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = i0 + u * kThreads, row = idx / dq, c = row / L.CT, x = row % L.CT;
+            const int f = g * L.MG + 2 * x + (NS ? c >> 1 : c);
+            w[u] = w2[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (idx < total && f < p.M) {
+                const size_t o = ((size_t)h * p.M + f) * d + 4 * (idx % dq);
+                w[u] = *reinterpret_cast<const float4*>(W1 + o);
+                if (NS) w2[u] = *reinterpret_cast<const float4*>(W2 + o);
             }
         }
-        *reinterpret_cast<float4*>(W + row * L.pd + e) = w;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = i0 + u * kThreads, row = idx / dq;
+            if (idx >= total) break;
+            if (NS) {
+                const float sg = (row / L.CT & 1) ? -1.f : 1.f;
+                w[u] = make_float4(0.5f * (w[u].x + sg * w2[u].x), 0.5f * (w[u].y + sg * w2[u].y),
+                                   0.5f * (w[u].z + sg * w2[u].z), 0.5f * (w[u].w + sg * w2[u].w));
+            }
+            *reinterpret_cast<float4*>(W + row * L.pd + 4 * (idx % dq)) = w[u];
+        }
     }
 }
 
-// Rows of a chunk, zero from row CL on.
+// Rows of a chunk from one tensor, or from two (src2 non-null), zero from row `rows` on; the
+// loads of a thread (up to eight) are issued before its stores.
 template <typename T>
-__device__ void load_rows(const T* src, size_t base, int rows, int d, float* dst, int pitch,
-                          int nrows)
+__device__ void load_rows(const T* src, const T* src2, size_t base, int rows, int d, float* dst,
+                          float* dst2, int pitch, int nrows)
 {
-    const int dq = d / 4;
-    for (int idx = threadIdx.x; idx < nrows * dq; idx += kThreads) {
-        const int t = idx / dq, e = 4 * (idx % dq);
-        *reinterpret_cast<float4*>(dst + t * pitch + e) =
-            t < rows ? load_act4(src, base + (size_t)t * d + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int dq = d / 4, total = nrows * dq;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * kThreads) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = i0 + u * kThreads, t = idx / dq, e = 4 * (idx % dq);
+            x[u] = y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (t < rows) {
+                x[u] = load_act4(src, base + (size_t)t * d + e);
+                if (src2) y[u] = load_act4(src2, base + (size_t)t * d + e);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = i0 + u * kThreads, t = idx / dq, e = 4 * (idx % dq);
+            if (idx >= total) break;
+            *reinterpret_cast<float4*>(dst + t * pitch + e) = x[u];
+            if (src2) *reinterpret_cast<float4*>(dst2 + t * pitch + e) = y[u];
+        }
     }
 }
 
@@ -291,6 +317,16 @@ struct Place {
     bool on;
 };
 
+// sin and cos of one argument, as a call: inlined, sixteen copies of the accurate function's
+// fast and slow paths at each use made the kernels miss the instruction cache.
+__device__ __noinline__ float2 sincos_call(float x)
+{
+    float s, c;
+    sincosf(x, &s, &c);
+    return make_float2(s, c);
+}
+__device__ __noinline__ float cos_call(float x) { return cosf(x); }
+
 // Unscaled features of this thread's 4 rows x 2 frequencies: pf = (cos, sin) of each (times
 // cos w), zero for rows from `rows` on and frequencies past M.  With CHAIN also
 // qf = (cos u sin w, sin u sin w) (n), for the derivative with respect to w.
@@ -308,14 +344,10 @@ __device__ __forceinline__ void features(const Problem& p, const Plan& L, const 
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const bool ok = 4 * f.y + r < rows && g * L.MG + 2 * f.x + i < p.M;
-            float s, c, sw = 0.f, cw = 1.f;
-            sincosf(a[r][NS ? 2 * i : i], &s, &c);
-            if (NS) {
-                if (CHAIN)
-                    sincosf(a[r][NC / 2 * i + (NS ? 1 : 0)], &sw, &cw);
-                else
-                    cw = cosf(a[r][NC / 2 * i + (NS ? 1 : 0)]);
-            }
+            const float2 u = sincos_call(a[r][NS ? 2 * i : i]);
+            const float aw = a[r][NC / 2 * i + (NS ? 1 : 0)];
+            const float2 w = !NS ? make_float2(0.f, 1.f) : CHAIN ? sincos_call(aw) : make_float2(0.f, cos_call(aw));
+            const float s = u.x, c = u.y, sw = w.x, cw = w.y;
             pf[r][2 * i] = ok ? (NS ? c * cw : c) : 0.f;
             pf[r][2 * i + 1] = ok ? (NS ? s * cw : s) : 0.f;
             if (NS && CHAIN) {
@@ -440,8 +472,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (!p.causal || L.CL > 1) {  // this range's sums
         for (int c = cb; c < ce; ++c) {
             const int t0 = c * L.T, rows = min(L.T, N - t0);
-            load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
-            load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+            load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
             unit_weights(L, d, rows, V);
             __syncthreads();
             if (tau) weight_keys(L, Xk, rows, d, itau, V, red);
@@ -467,10 +498,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 
     for (int c = cb; c < ce; ++c) {
         const int t0 = c * L.T, rows = min(L.T, N - t0);
-        load_rows(q, base + (size_t)t0 * d, rows, d, Xq, L.pd, L.T);
+        load_rows(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
         if (p.causal) {
-            load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
-            load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+            load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
             unit_weights(L, d, rows, V);
         }
         __syncthreads();
@@ -707,12 +737,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int i = tid; i < L.ng * gD; i += kThreads) dW[i] = 0.f;
 
     auto load_kv = [&](int t0, int rows) {
-        load_rows(k, base + (size_t)t0 * d, rows, d, Xk, L.pd, L.T);
-        load_rows(v, base + (size_t)t0 * d, rows, d, V, L.pd, L.T);
+        load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
         unit_weights(L, d, rows, V);
     };
     auto load_qg = [&](int t0, int rows) {
-        load_rows(q, base + (size_t)t0 * d, rows, d, Xq, L.pd, L.T);
+        load_rows(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
         load_upstream(p, L, dout, out, den, base + (size_t)t0 * d, den_base + t0, rows, G);
     };
     auto group_W = [&](int g) {  // the group's projection rows, staged now unless resident
@@ -1154,16 +1183,20 @@ bool make_plan(const Problem& p, bool bwd, Plan* plan)
                 found = (size_t)plan->total <= kSmemFloats;
             }
     if (!found) return false;
-    const int sms = std::max(1, tc::sm_count());
+    // (16 sequences: 8 CTAs each take two rounds, 0.51 ms on the training shape above; 6 take one,
+    // 0.36 ms.)
+    // Clusters of 1..8 CTAs that run at once with one CTA per SM (cudaOccupancyMaxActiveClusters
+    // on GB300: 152 SMs in eight groups, of which a cluster takes its SMs from one).
+    static const int kClusters[kMaxCluster] = {152, 76, 46, 36, 28, 23, 15, 15};
     const int occ = !bwd && 2 * ((size_t)plan->total * 4 + 1024) <= 228 * 1024 ? 2 : 1;
     const long long bh = (long long)p.B * p.H, nch = (p.N + plan->T - 1) / plan->T;
     double best = 0.;
-    for (int cl = 1; cl <= kMaxCluster && (cl == 1 || cl <= nch); cl *= 2) {
+    for (int cl = 1; cl <= kMaxCluster && (cl == 1 || cl <= nch); ++cl) {
         const double per = (double)((nch + cl - 1) / cl);
         const double pre = !p.causal || cl > 1 ? (bwd ? 0.8 : 0.4) : 0.;
-        const long long ctas = bh * cl;
-        double rounds = (double)((ctas + (long long)sms * occ - 1) / ((long long)sms * occ));
-        if (occ == 2 && ctas > sms) rounds *= 1.6;  // two CTAs share an SM
+        const long long cap = (long long)kClusters[cl - 1] * occ;
+        double rounds = (double)((bh + cap - 1) / cap);
+        if (occ == 2 && bh > kClusters[cl - 1]) rounds *= 1.6;  // two CTAs share an SM
         const double cost = rounds * (per * ((bwd ? 3. : 1.) + pre) + 1. + (cl > 1 ? 0.5 : 0.));
         if (cl == 1 || cost < best) {
             best = cost;
