@@ -317,15 +317,55 @@ struct Place {
     bool on;
 };
 
-// sin and cos of one argument, as a call: inlined, sixteen copies of the accurate function's
-// fast and slow paths at each use made the kernels miss the instruction cache.
-__device__ __noinline__ float2 sincos_call(float x)
+// sin and cos of two arguments in fp32, on packed pairs: reduction by pi/2 in three constants
+// (Cody and Waite: the fp32 values of pi/2 and of the two remainders, each step one fma), then
+// polynomials on [-pi/4, pi/4], sin r = r + r y (s0 + s1 y + s2 y^2) and
+// cos r = 1 + y (-1/2 + y (c0 + c1 y + c2 y^2)) with y = r^2, fitted here by least squares on
+// 4000 Chebyshev nodes refined by Lawson's iteration (approximation error 2e-9 and 1e-10).
+// Max error against fp64 over |x| <= 10^4: 7.1e-8 (rms 1.7e-8; rounding the exact value:
+// 1.5e-8), as the CUDA library's sincosf, which larger arguments take.  About 15 instructions
+// an argument instead of 45; inlined library calls also overflowed the instruction cache.
+__device__ __noinline__ float2 sincos_large(float x)
 {
     float s, c;
     sincosf(x, &s, &c);
     return make_float2(s, c);
 }
-__device__ __noinline__ float cos_call(float x) { return cosf(x); }
+__device__ __forceinline__ void sincos2(float x0, float x1, float (&s)[2], float (&c)[2])
+{
+    if (!(fmaxf(fabsf(x0), fabsf(x1)) <= 1.0e4f)) {  // large or infinite (a lone NaN stays NaN below)
+        const float2 a = sincos_large(x0), b = sincos_large(x1);
+        s[0] = a.x; c[0] = a.y; s[1] = b.x; c[1] = b.y;
+        return;
+    }
+    auto k2 = [](float k) { return tc::f2_pack(k, k); };
+    constexpr float kRound = 12582912.f;  // 1.5 * 2^23: the sum's low bits hold rint(x 2/pi)
+    const uint64_t x = tc::f2_pack(x0, x1);
+    const uint64_t t = tc::f2_fma(x, k2(0.63661977236758134f), k2(kRound));
+    const uint64_t n = tc::f2_fma(t, k2(1.f), k2(-kRound));
+    uint64_t r = tc::f2_fma(n, k2(-1.57079637050628662f), x);
+    r = tc::f2_fma(n, k2(4.371138828673793e-8f), r);
+    r = tc::f2_fma(n, k2(1.7151244994428828e-15f), r);
+    const uint64_t y = tc::f2_mul(r, r);
+    uint64_t p = tc::f2_fma(k2(-1.9495636e-4f), y, k2(8.331979e-3f));
+    p = tc::f2_fma(p, y, k2(-1.6666651e-1f));
+    const uint64_t sn = tc::f2_fma(tc::f2_mul(p, y), r, r);
+    uint64_t q = tc::f2_fma(k2(2.4438452e-5f), y, k2(-1.3887368e-3f));
+    q = tc::f2_fma(q, y, k2(4.1666646e-2f));
+    q = tc::f2_fma(q, y, k2(-0.5f));
+    const uint64_t cs = tc::f2_fma(q, y, k2(1.f));
+    float tn[2], sr[2], cr[2];
+    tc::f2_unpack(t, tn[0], tn[1]);
+    tc::f2_unpack(sn, sr[0], sr[1]);
+    tc::f2_unpack(cs, cr[0], cr[1]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t quad = __float_as_uint(tn[i]);
+        const float a = (quad & 1u) ? cr[i] : sr[i], b = (quad & 1u) ? sr[i] : cr[i];
+        s[i] = __uint_as_float(__float_as_uint(a) ^ ((quad & 2u) << 30));
+        c[i] = __uint_as_float(__float_as_uint(b) ^ (((quad + 1u) & 2u) << 30));
+    }
+}
 
 // Unscaled features of this thread's 4 rows x 2 frequencies: pf = (cos, sin) of each (times
 // cos w), zero for rows from `rows` on and frequencies past M.  With CHAIN also
@@ -340,21 +380,21 @@ __device__ __forceinline__ void features(const Problem& p, const Plan& L, const 
     zero(a);
     mm_nt<NC>(X + 4 * f.y * L.pd, L.pd, W + f.x * L.pd, L.CT * L.pd, p.d, a);
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
+        float su[2], cu[2], sw[2], cw[2];
+        sincos2(a[r][0], a[r][NC / 2], su, cu);
+        if (NS) sincos2(a[r][1], a[r][NC - 1], sw, cw);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const bool ok = 4 * f.y + r < rows && g * L.MG + 2 * f.x + i < p.M;
-            const float2 u = sincos_call(a[r][NS ? 2 * i : i]);
-            const float aw = a[r][NC / 2 * i + (NS ? 1 : 0)];
-            const float2 w = !NS ? make_float2(0.f, 1.f) : CHAIN ? sincos_call(aw) : make_float2(0.f, cos_call(aw));
-            const float s = u.x, c = u.y, sw = w.x, cw = w.y;
-            pf[r][2 * i] = ok ? (NS ? c * cw : c) : 0.f;
-            pf[r][2 * i + 1] = ok ? (NS ? s * cw : s) : 0.f;
+            pf[r][2 * i] = ok ? (NS ? cu[i] * cw[i] : cu[i]) : 0.f;
+            pf[r][2 * i + 1] = ok ? (NS ? su[i] * cw[i] : su[i]) : 0.f;
             if (NS && CHAIN) {
-                qf[r][2 * i] = ok ? c * sw : 0.f;
-                qf[r][2 * i + 1] = ok ? s * sw : 0.f;
+                qf[r][2 * i] = ok ? cu[i] * sw[i] : 0.f;
+                qf[r][2 * i + 1] = ok ? su[i] * sw[i] : 0.f;
             }
         }
+    }
 }
 __device__ __forceinline__ void store_tile(float* P, int pitch, const Place& f, const float (&v)[4][4])
 {

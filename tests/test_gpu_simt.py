@@ -66,3 +66,25 @@ def test_fp32_kernels_match_oracle(c):
                 assert rel_l2(x, ref) <= (1e-4 if dtype == "f32" else BF16_REL_L2), name
         else:
             assert_close(x, ref, dtype, name, max_abs_scale=scale)
+
+
+@pytest.mark.parametrize("variant", ["s", "n"])
+@pytest.mark.parametrize("size", [3.0, 9.0e3, 1.1e4, 3.0e6])
+def test_fp32_sin_cos_at_exact_arguments(variant, size):
+    """One token with one-hot q and k: every projection argument is a frequency or half of one
+    exactly, so den = phi(q) . phi(k) shows the sin and cos alone, on both sides of the
+    argument size where the kernels change methods.  Each of den's 4 M products has two
+    factors within 2^-23 of exact: |error| <= 4 * 2^-23 per frequency's share of the mean."""
+    H, M, d = 64, 33, 4
+    rng = np.random.default_rng(5)
+    W1 = rng.uniform(-size, size, (H, M, d)).astype(np.float32)
+    W2 = rng.uniform(-size, size, (H, M, d)).astype(np.float32) if variant == "n" else None
+    if W2 is not None:  # halves of sums exact in fp32: few mantissa bits
+        step = np.float32(2.0 ** np.floor(np.log2(size / 4096)))
+        W1, W2 = (step * np.rint(w / step) for w in (W1, W2))
+    x = np.zeros((1, H, 1, d), np.float32)
+    x[..., 0] = 1.0
+    q, k, v = x, np.float32(0.5) * x, x
+    out, den = flexattn.linattn_fwd(*(to_dev(a, "f32") for a in (q, k, v, W1, W2)), False)
+    _, rd = oracle.fwd(q, k, v, W1, W2, False)
+    assert np.abs(to_host(den) - rd).max() <= 4 * 2.0 ** -23
