@@ -30,7 +30,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxCluster = 8;   // CTAs that share one sequence
-constexpr int kMaxT = 64;        // tokens per chunk
+constexpr int kMaxT = 128;       // tokens per chunk (over 64: the non-causal forward only)
 constexpr int kMaxMG = 32;       // frequencies per group (64 features)
 
 __device__ __forceinline__ float load_act(const float* p, size_t i) { return p[i]; }
@@ -114,11 +114,12 @@ __global__ void featmap_kernel(Problem p, const T* x, const float* W1, const flo
 // limit (one output per thread took two loads per fma), and a short sequence spreads over
 // up to 8 SMs instead of one.  Measured on GB300 against one CTA per sequence with
 // one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 23 us, bf16 n B32 H4
-// N1024 d32 M16 477 -> 104 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
-// 8.58 -> 0.36 ms (9.5 of the 78 TFLOP/s fp32 peak: per chunk the products run between
+// N1024 d32 M16 477 -> 73 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
+// 8.58 -> 0.33 ms (10 of the 78 TFLOP/s fp32 peak: per chunk the products run between
 // barriers with one backward CTA per SM, so load latency and the barriers bound it).
 struct Plan {
     int T;              // tokens per chunk (a multiple of 8, at most kMaxT)
+    int lpr;            // lanes per row in row-wise sums: 4, or 2 with 128 tokens
     int ng, MG;         // frequency groups; frequencies per group (a multiple of 4)
     int CT;             // feature column tiles of a group, MG / 2
     int F;              // features of a group, 2 MG
@@ -286,22 +287,22 @@ __device__ __forceinline__ void unit_weights(const Plan& L, int d, int rows, flo
     if (threadIdx.x < L.T) V[threadIdx.x * L.pd + d] = threadIdx.x < rows ? 1.f : 0.f;
 }
 
-// Prefactor: [v_j | 1] -> [w_j v_j | w_j], w_j = exp(|k_j|^2 itau); |k_j|^2 to kn2.  Four
+// Prefactor: [v_j | 1] -> [w_j v_j | w_j], w_j = exp(|k_j|^2 itau); |k_j|^2 to kn2.  lpr
 // lanes per row.
 __device__ __forceinline__ void weight_keys(const Plan& L, const float* Xk, int rows, int d,
                                             float itau, float* V, float* kn2)
 {
-    if (threadIdx.x >= 4 * L.T) return;
-    const int j = threadIdx.x >> 2, part = threadIdx.x & 3;
+    if (threadIdx.x >= L.lpr * L.T) return;
+    const int j = threadIdx.x / L.lpr, part = threadIdx.x % L.lpr, step = 4 * L.lpr;
     float n2 = 0.f;
-    for (int e = 4 * part; e < d; e += 16) {
+    for (int e = 4 * part; e < d; e += step) {
         const float4 x = *reinterpret_cast<const float4*>(Xk + j * L.pd + e);
         n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, n2))));
     }
     n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
-    n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+    if (L.lpr == 4) n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
     const float w = j < rows ? expf(n2 * itau) : 0.f;
-    for (int e = 4 * part; e < d; e += 16) {
+    for (int e = 4 * part; e < d; e += step) {
         float4* v = reinterpret_cast<float4*>(V + j * L.pd + e);
         if (j < rows) *v = make_float4(w * v->x, w * v->y, w * v->z, w * v->w);
     }
@@ -404,17 +405,36 @@ __device__ __forceinline__ void store_tile(float* P, int pitch, const Place& f, 
             make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
 }
 
+// acc = sum_k a[k pa + r] b[k pb + c] over K rows: ks (1, 2 or 4) neighbouring lanes share a
+// 4 x 4 tile, each sums every ks-th row, and every lane of the group returns the sum.
+__device__ __forceinline__ void mm_tn_split(const float* a, int pa, const float* b, int pb, int K,
+                                            int ks, float (&acc)[4][4])
+{
+    const int part = threadIdx.x & (ks - 1);
+    mm_tn(a + part * pa, ks * pa, b + part * pb, ks * pb, K / ks, acc);
+    for (int o = 1; o < ks; o *= 2)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] += __shfl_xor_sync(0xffffffffu, acc[r][c], o);
+}
+
 // State of one group: S[prow(f)][e] += sum_j P[j][f] Y[j][e] and, in column d, the sum
 // weighted by Y[j][d] (z, or r from G = [g | c]).
 __device__ __forceinline__ void state_update(const Plan& L, int d, const float* P, const float* Y,
                                              float* S)
 {
-    const int dq = d / 4;
-    for (int id = threadIdx.x; id < L.CT * dq; id += kThreads) {
+    const int dq = d / 4, tiles = L.CT * dq;
+    // over long chunks, lanes without a tile of their own share one
+    const int ks = L.T <= 64 ? 1 : 4 * tiles <= kThreads ? 4 : 2 * tiles <= kThreads ? 2 : 1;
+    for (int i0 = threadIdx.x & ~31; i0 < tiles * ks; i0 += kThreads) {
+        // (whole warps take part in the exchange: lanes past the end repeat the last tile)
+        const int at = i0 + (threadIdx.x & 31), id = min(at / ks, tiles - 1);
         const int x = id / dq, e = 4 * (id % dq);
         float acc[4][4];
         zero(acc);
-        mm_tn(P + 4 * x, L.pp, Y + e, L.pd, L.T, acc);
+        mm_tn_split(P + 4 * x, L.pp, Y + e, L.pd, L.T, ks, acc);
+        if (at >= tiles * ks || (at & (ks - 1))) continue;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             float4* s = reinterpret_cast<float4*>(S + (r * L.CT + x) * L.pd + e);
@@ -501,6 +521,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const Place f = {tid / L.CT, tid % L.CT, tid / L.CT < L.T / 4};
     const int TT = L.T / 4, ay = tid / TT, ax = tid % TT;  // T x T tile: rows 4 ay + r, cols ax + TT c
     const bool a_on = ay < TT;
+    const int lpr = L.lpr, row = tid / lpr, part = tid % lpr;  // row-wise sums
     int cb, ce;
     chunk_range(L, N, rank, &cb, &ce);
 
@@ -575,9 +596,9 @@ __global__ void __launch_bounds__(kThreads, 2)
                     mm_nn(Pq + 4 * y * L.pp, L.pp, Sg + e, L.CT * L.pd, 2 * L.CT * L.pd,
                           3 * L.CT * L.pd, L.pd, L.F, num[n]);
             }
-            if (tid < 4 * L.T)  // denominator: four lanes per row
-                for (int i = tid & 3; i < L.CT; i += 4) {
-                    const float4 x = *reinterpret_cast<const float4*>(Pq + (tid >> 2) * L.pp + 4 * i);
+            if (tid < lpr * L.T)  // denominator
+                for (int i = part; i < L.CT; i += lpr) {
+                    const float4 x = *reinterpret_cast<const float4*>(Pq + row * L.pp + 4 * i);
                     const float* z = Sg + i * L.pd + d;
                     dsum = fmaf(x.x, z[0], dsum);
                     dsum = fmaf(x.y, z[L.CT * L.pd], dsum);
@@ -607,17 +628,16 @@ __global__ void __launch_bounds__(kThreads, 2)
                     mm_nn(A + 4 * y * L.pa, L.pa, V + e, L.pd, 2 * L.pd, 3 * L.pd, 4 * L.pd, L.T,
                           num[n]);
             }
-            if (tid < 4 * L.T)
-                for (int j = tid & 3; j < L.T; j += 4)
-                    dsum = fmaf(A[(tid >> 2) * L.pa + j], V[j * L.pd + d], dsum);
+            if (tid < lpr * L.T)
+                for (int j = part; j < L.T; j += lpr)
+                    dsum = fmaf(A[row * L.pa + j], V[j * L.pd + d], dsum);
         }
-        if (tid < 4 * L.T) {
+        if (tid < lpr * L.T) {
             dsum += __shfl_xor_sync(0xffffffffu, dsum, 1);
-            dsum += __shfl_xor_sync(0xffffffffu, dsum, 2);
-            const int i = tid >> 2;
-            if ((tid & 3) == 0) {
-                red[kMaxT + i] = dsum;
-                if (den && i < rows) den[(size_t)bh * N + t0 + i] = dsum * inv_m;
+            if (lpr == 4) dsum += __shfl_xor_sync(0xffffffffu, dsum, 2);
+            if (part == 0) {
+                red[kMaxT + row] = dsum;
+                if (den && row < rows) den[(size_t)bh * N + t0 + row] = dsum * inv_m;
             }
         }
         __syncthreads();
@@ -1172,6 +1192,7 @@ Plan layout(const Problem& p, bool bwd, int mg, int T, bool wres)
 {
     Plan L = {};
     L.T = T;
+    L.lpr = T > 64 ? 2 : 4;
     L.wres = wres;
     L.CL = 1;
     L.ng = (p.M + mg - 1) / mg;
@@ -1216,8 +1237,17 @@ bool make_plan(const Problem& p, bool bwd, Plan* plan)
 {
     if (!(bwd ? fits_bwd(p) : fits_fwd(p))) return false;
     bool found = false;
+    // 128 tokens where 64 would give no more than half of the threads a tile of features and of
+    // the output (non-causal forward, long enough sequences): bf16 n B32 H4 N1024 d32 M16
+    // 90 -> 73 us.
+    const Plan small = layout(p, bwd, kMaxMG, 64, true);
+    const int tiles = 16 * std::max(small.CT, p.d / 4);
+    if (!bwd && !p.causal && 2 * tiles <= kThreads && p.N >= 512) {
+        *plan = layout(p, bwd, kMaxMG, 128, true);
+        found = 2 * ((size_t)plan->total * 4 + 1024) <= 228 * 1024;
+    }
     for (int mg = kMaxMG; mg >= 4 && !found; mg /= 2)  // smaller groups: the largest shapes only
-        for (int T = kMaxT; T >= 8 && !found; T /= 2)
+        for (int T = 64; T >= 8 && !found; T /= 2)
             for (int wres = 1; wres >= 0 && !found; --wres) {
                 *plan = layout(p, bwd, mg, T, wres != 0);
                 found = (size_t)plan->total <= kSmemFloats;

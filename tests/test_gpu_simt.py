@@ -23,6 +23,7 @@ CASES = [
     ("n", True, "f32", 1, 2, 100, 64, 100, True), ("s", False, "f32", 1, 1, 90, 88, 169, True),
     ("s", True, "f32", 1, 1, 90, 116, 129, False), ("n", True, "f32", 1, 1, 70, 16, 256, True),
     ("n", True, "bf16", 2, 2, 257, 32, 16, True), ("n", False, "bf16", 4, 3, 1024, 32, 16, False),
+    ("s", False, "bf16", 2, 3, 512, 32, 16, True), ("n", False, "f32", 1, 2, 641, 16, 5, True),
     ("s", True, "bf16", 1, 2, 140, 128, 24, True), ("s", False, "bf16", 1, 2, 191, 64, 16, True),
 ]
 
