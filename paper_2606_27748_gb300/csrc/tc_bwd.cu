@@ -147,9 +147,10 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     __shared__ uint32_t tmem_base_sh;
     // tiles landed: tx[buffer] (q, k, v as the mode reads them), tg (dout and out), tv[buffer]
     // (v in kState); compute -> issuer, one arrival
-    // per warp: rdy (operands written, tensor memory read), rdyg (the g tile), srdy (the dk
+    // per warp: rdy (operands written, tensor memory read), rdyg (the g tile), rdys[buffer]
+    // (kState, where a warp may be a chunk ahead of another), srdy (the dk
     // rows taken); fin: every warp's rdy has been seen (kLate); MMA groups complete: m0, m1, mt[buffer]
-    __shared__ __align__(8) uint64_t tx[2], tg, tv[3], rdy, rdyg, srdy, fin, m0, m1, mt[2];
+    __shared__ __align__(8) uint64_t tx[2], tg, tv[3], rdy, rdyg, rdys[2], srdy, fin, m0, m1, mt[2];
     // cluster exchange i (0: dq (F) or dv (R), 1: dk (R)): xready: the partner's receive region
     // is free; xfull: the partner's partial landed (transaction count); xdone: this CTA's
     // partial landed there, so its staging region may be rewritten
@@ -199,7 +200,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     if (tid == 0) {
         for (uint64_t* b : {&tx[0], &tx[1], &tg, &tv[0], &tv[1], &tv[2], &m0, &m1, &mt[0], &mt[1]})
             mbar_init(b, 1);
-        for (uint64_t* b : {&rdy, &rdyg, &srdy}) mbar_init(b, kComputeWarps);
+        for (uint64_t* b : {&rdy, &rdyg, &rdys[0], &rdys[1], &srdy}) mbar_init(b, kComputeWarps);
         mbar_init(&fin, 1);
         mbar_init(&xready[0], 1);
         mbar_init(&xready[1], 1);
@@ -912,7 +913,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         if (relay) {
         } else if (issuer) {
             [&]() {
-                uint32_t p_tx[2] = {0, 0}, p_tv[3] = {0, 0, 0}, p_rdy = 0, p_m1 = 0;
+                uint32_t p_tx[2] = {0, 0}, p_tv[3] = {0, 0, 0}, p_rdys[2] = {0, 0}, p_m1 = 0;
                 auto load_x = [&](int i) {
                     wmbar_arrive_expect_tx(&tx[i & 1], kTileBytes);
                     load_tile(xb[i & 1], fq ? &tmap_q : &tmap_k, cbeg + i, &tx[i & 1]);
@@ -947,7 +948,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                         }
                     }
                     if (i + 1 < n && !project(i + 1)) return;
-                    if (!wwait(&rdy, p_rdy)) return;  // features (and g) of chunk i
+                    if (!wwait(&rdys[i & 1], p_rdys[i & 1])) return;  // features (and g) of chunk i
                     if (i + 2 < n) load_x(i + 2);
                     if (fq && i + 1 < n) load_g(i + 1);
                     if (!fq && !wwait(&tv[i % 3], p_tv[i % 3])) return;
@@ -982,7 +983,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                     build_g(sb + gb[i & 1], crow, sb + cb[i & 1], den_r, CL, true, true);
                     den_r = load_den(t0 + kC);
                 }
-                arrive(&rdy);
+                arrive(&rdys[i & 1]);
             }
         }
         __syncthreads();  // reached after an abort as well: the last sums are complete
