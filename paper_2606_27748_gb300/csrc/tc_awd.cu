@@ -22,6 +22,7 @@
 // partial slots, summed per sequence in a fixed order.  Every wait is bounded.  For the
 // gradient the same kernel also writes each row's statistics (below).
 #include <algorithm>
+#include <type_traits>
 
 #include "flex_internal.h"
 #include "tc_common.cuh"
@@ -52,6 +53,13 @@ __device__ __forceinline__ float lg2f(float x)
 {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcpf(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -283,31 +291,49 @@ __global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* __restric
 //   dphi(q_i) = sigma sum_j G_ij phi~(k_j),   dphi~(k_j) = sigma sum_i G_ij phi(q_i).
 // A sequence's query side holds blocks of 128 queries and streams the key blocks; its key
 // side holds blocks of 128 keys and streams the query blocks; each side's held blocks are
-// split over `hsplit` CTAs.  Per streamed block thread 0 issues S = X_own X_other^T and
-// A = Phi_own Phi_other^T into tensor memory; 16 warps (four per lane quadrant, each on 32
-// of the 128 columns) turn their part of the rows into G (two SFU operations per entry:
-// ex2 and a divide), write it as bf16 in place over the columns they read, and G Phi_other
-// (A operand in tensor memory, features MN-major) accumulates into T_D.  With M = 64 the
-// streamed tiles are double-buffered: the next block's load is issued as soon as the
-// current one has landed.  Then, per group of 64 frequencies, the chain rule through the
-// feature map runs on the tensor cores: the projection X_own W'^T is recomputed, the
-// epilogue forms da (du | dw for Flexformer_n) from T_D, and dW' += da^T X_own.  The rows of
+// split over `hsplit` CTAs.  The other side's rows are streamed 64 at a time: S = X_own
+// X_other^T and A = Phi_own Phi_other^T into one of two tensor-memory buffers, the buffer's
+// group of 8 compute warps turns them into G (ex2 and a reciprocal an entry), writes it as
+// bf16 in place over A, and G Phi_other (A operand in tensor memory, features MN-major)
+// accumulates into T_D.  A loader warp and an issuing warp run ahead of the compute warps,
+// which only meet them at mbarriers.  M = 64: the held block's x and features are tensor-memory
+// operands and the next held block is loaded meanwhile.  Then, per group of 64 frequencies, the
+// chain rule through the feature map runs on the tensor cores: the projection X_own W'^T is
+// recomputed, the epilogue forms da (du | dw for Flexformer_n) from T_D, and dW' += da^T X_own.
+// What bounds it: per step of 128 x 64 entries the 16 small MMAs (about 0.4 us) and the two
+// groups' arithmetic (0.7 us each, overlapping); per CTA about a third of the time is set-up
+// and the chain rule.  Measured, one distillation step n B32 H8 N512 M64: 361 us with all
+// warps in step and thread 0 issuing, 307 us now (mask and side as compile-time cases 357 ->
+// 333, the held block as a tensor-memory operand -> 324, loads by their own warp -> 307).  The rows of
 // dW' are added into this CTA's slot; a reduction sums the slots over the sides, the batch
 // and the splits in a fixed order, so the result does not depend on scheduling.  On the
 // key side, with the prefactor, the chain rule takes dphi(k_j) = w_j dphi~(k_j) and dtau
 // gains -(phi~(k_j) . dphi~(k_j)) |k_j|^2 exp(-tau).  Every wait is bounded.
-constexpr int kThreadsG = 512;
-
+constexpr int kComputeG = 16;                    // compute warps, four per lane quadrant
+constexpr int kThreadsG = 32 * kComputeG + 64;   // and the issuer's and the loader's warps
+constexpr int kHalf = 64;                        // streamed rows per step
 template <int G2>
 struct AwdBwCfg {
-    static constexpr int STAGES = G2 == 2 ? 2 : 1;          // streamed tiles in flight
-    static constexpr uint32_t XO = 0, PO = 16384, ST0 = PO + G2 * 16384;
-    static constexpr uint32_t STAGE_BYTES = (1 + G2) * 16384;  // x tile, then features
+    // M = 64 has tensor memory left for the held block's x and features (bf16) as operands, so
+    // every step's S and A read only the streamed rows from shared memory; it also has two
+    // buffers for held blocks, the features' place taking da once they are copied.
+    static constexpr bool OWN_T = G2 == 2;
+    static constexpr int STAGES = OWN_T ? 4 : 2, OWN = OWN_T ? 2 : 1;  // steps, blocks in flight
+    static constexpr uint32_t OWN_BYTES = (1 + G2) * 16384;     // x tile, then features
+    static constexpr uint32_t ST0 = OWN * OWN_BYTES;
+    static constexpr uint32_t STAGE_BYTES = (1 + G2) * 8192;    // x rows, then features
     static constexpr uint32_t WG = ST0 + STAGES * STAGE_BYTES;  // W' rows of every group
-    static constexpr uint32_t BYTES = WG + (G2 / 2) * 16384;   // (at most 16 KB a group)
-    static constexpr uint32_t DA = ST0 + 16384;  // after the streamed blocks: da [du | dw]
-    static constexpr uint32_t T_S = 0, T_A = 128, T_D = 256;
+    static constexpr uint32_t BYTES = WG + (G2 / 2) * 16384;    // (at most 16 KB a group)
+    __host__ __device__ static constexpr uint32_t XO(int ob) { return OWN_T ? (uint32_t)(ob & 1) * OWN_BYTES : 0u; }
+    __host__ __device__ static constexpr uint32_t PO(int ob) { return XO(ob) + 16384; }
+    // da [du | dw], after the streamed steps
+    __host__ __device__ static constexpr uint32_t DA(int ob) { return OWN_T ? PO(ob) : ST0; }
+    // tensor memory: two buffers of S (64 columns) and A (64), the projection and dW' of the
+    // chain rule over them, dphi
+    static constexpr uint32_t T_SA = 0, T_C = 0, T_W = 128, T_D = 256;
+    static constexpr uint32_t T_XO = 384, T_PO = 416;
     static_assert(G2 >= 2 && BYTES + 1024 <= 232448, "shared memory budget");
+    static_assert(OWN_T || STAGES * STAGE_BYTES >= 32768, "da fits the stages");
 };
 
 template <int G2, bool NS, bool KW>
@@ -325,14 +351,18 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     using L = AwdBwCfg<G2>;
     constexpr int P = NS ? 128 : 64;  // projection rows per group of 64 frequencies
     constexpr int G = G2 / 2;
-    constexpr int S = L::STAGES;
+    constexpr int ST = L::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t sb = smem_u32(sm);
     __shared__ uint32_t tmem_base_sh;
-    __shared__ __align__(8) uint64_t mbar, tma_bar[S];
+    // tiles landed: town[buffer] (held block), tx[stage]; their last use done: ofree, sfree; one arrival per compute warp: rdy[buffer] (G of
+    // a step, from the group of warps that takes that buffer's steps), rdyc (start of a held block, chain rule); MMA groups complete: msa[buffer]
+    // (S and A of a step), md (dphi of a step), mc (chain rule)
+    __shared__ __align__(8) uint64_t town[L::OWN], ofree[L::OWN], tx[ST], sfree[ST], rdy[2],
+        rdyc, msa[2], md, mc;
     __shared__ volatile int abort_flag;
-    __shared__ float4 ostat[kC];  // key side: statistics of the streamed query rows
+    __shared__ float4 ostat[4][kHalf];  // key side: statistics of the streamed query rows
     __shared__ float wsum[kThreadsG / 32];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -344,7 +374,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     const CUtensorMap* x_oth = kside ? &tmap_q : &tmap_k;
     const CUtensorMap* f_own = kside ? &tmap_pk : &tmap_pq;
     const CUtensorMap* f_oth = kside ? &tmap_pq : &tmap_pk;
-    const int nblk = (N + kC - 1) / kC;
+    const int nblk = (N + kC - 1) / kC, nhalf = (N + kHalf - 1) / kHalf;
     const int hb0 = split * nblk / hsplit, hb1 = (split + 1) * nblk / hsplit;
     const float sigma = -dloss[bh] / (float)N;
     const float itau = KW ? expf(-tau[h]) : 0.f;
@@ -352,8 +382,18 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     float dtau_acc = 0.f;
 
     if (tid == 0) {
-        mbar_init(&mbar, 1);
-        for (int s = 0; s < S; ++s) mbar_init(&tma_bar[s], 1);
+        for (int s = 0; s < L::OWN; ++s) {
+            mbar_init(&town[s], 1);
+            mbar_init(&ofree[s], 1);
+        }
+        for (int s = 0; s < ST; ++s) {
+            mbar_init(&tx[s], 1);
+            mbar_init(&sfree[s], 1);
+        }
+        mbar_init(&rdy[0], kComputeG / 2);
+        mbar_init(&rdy[1], kComputeG / 2);
+        mbar_init(&rdyc, kComputeG);
+        for (uint64_t* b : {&msa[0], &msa[1], &md, &mc}) mbar_init(b, 1);
         abort_flag = 0;
         fence_mbar_init();
     }
@@ -361,315 +401,403 @@ __global__ void __launch_bounds__(kThreadsG, 1)
         tmem_alloc(&tmem_base_sh, 512);
         tmem_relinquish();
     }
+    // this head's W' rows, all groups, once
+    if (warp < kComputeG) stage_freq_rows<NS, G, 32 * kComputeG>(sb + L::WG, W1, W2, h, M, tid);
+    fence_proxy_async();
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     const uint32_t tm = tmem_base_sh;
     const uint32_t tm_row = tm + ((uint32_t)(32 * quad) << 16);
-    uint32_t phase = 0, tph = 0;  // tph: bit st = parity of stage st's barrier
-    auto adv = [](uint64_t dsc, uint32_t bytes) { return dsc + (bytes >> 4); };
-    auto xt = [](int st) { return L::ST0 + (uint32_t)st * L::STAGE_BYTES; };
-    const uint64_t dXO = sdesc(sb + L::XO, 16, 1024), dPO = sdesc(sb + L::PO, 16, 1024);
-    const uint64_t dDAmn = sdesc(sb + L::DA, 16384, 1024), dXOmn = sdesc(sb + L::XO, 16384, 1024);
-    constexpr uint32_t I_KK128 = idesc_bf16(128, 128, 0, 0);
-    constexpr uint32_t I_DPHI = idesc_bf16(128, 64 * G2, 0, 1);  // N = 2M features
-    constexpr uint32_t I_PROJ = idesc_bf16(128, P, 0, 0);
-    constexpr uint32_t I_DW = idesc_bf16(128, 64, 1, 1);
-
-    auto handoff = [&]() {
+    auto wwait = [&](uint64_t* bar, uint32_t& ph) -> bool {  // a whole warp, one verdict
+        const bool ok = bar_wait_w(bar, ph, &abort_flag, status);
+        ph ^= 1;
+        fence_after_sync();
+        return ok;
+    };
+    auto arrive = [&](uint64_t* bar) {  // this warp's shared- and tensor-memory accesses are done
         fence_proxy_async();
         fence_before_sync();
-        __syncthreads();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
     };
-    auto commit_wait = [&]() -> bool {  // thread 0 has issued MMAs: commit, all wait
-        if (tid == 0) mma_commit(&mbar);
-        bool ok_ = bar_wait(&mbar, phase, &abort_flag, status);
-        phase ^= 1;
-        ok_ = !__syncthreads_or(!ok_);
-        fence_after_sync();
-        return ok_;
-    };
-    // streamed block ot into stage st (and first the held block ob): one arrival per phase
-    auto load = [&](int ob, int ot, int st, bool own_too) {
-        mbar_arrive_expect_tx(&tma_bar[st], (1 + G2) * kTileBytes * (own_too ? 2 : 1));
-        if (own_too) {
-            tma_load_3d(sb + L::XO, x_own, 0, ob * kC, bh, &tma_bar[st]);
-            for (int g = 0; g < G2; ++g)
-                tma_load_3d(sb + L::PO + g * 16384, f_own, 64 * g, ob * kC, bh, &tma_bar[st]);
-        }
-        tma_load_3d(sb + xt(st), x_oth, 0, ot * kC, bh, &tma_bar[st]);
-        for (int g = 0; g < G2; ++g)
-            tma_load_3d(sb + xt(st) + 16384 + g * 16384, f_oth, 64 * g, ot * kC, bh,
-                        &tma_bar[st]);
-    };
-    // streamed blocks of held block ob: causal queries see keys j <= i
-    auto first_other = [&](int ob) { return (kside && causal) ? ob : 0; };
-    auto last_other = [&](int ob) { return (!kside && causal) ? ob : nblk - 1; };
+    // streamed steps (64 rows) of held block ob: causal queries see keys j <= i
+    auto first_step = [&](int ob) { return (kside && causal) ? 2 * ob : 0; };
+    auto last_step = [&](int ob) { return (!kside && causal) ? min(nhalf, 2 * ob + 2) : nhalf; };
 
-    bool ok = true;
-    if (tid == 0) load(hb0, first_other(hb0), 0, true);
-    // this head's W' rows, all groups, once (overlaps the first load; made visible to the
-    // tensor cores by the fence here and the barrier at the first wait)
-    stage_freq_rows<NS, G, kThreadsG>(sb + L::WG, W1, W2, h, M, tid);
-    fence_proxy_async();
-    for (int ob = hb0; ob < hb1 && ok; ++ob) {
-        const int own_row = ob * kC + t;
-        const bool own_valid = own_row < N;
-        float4 qs = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!kside && own_valid) qs = rowstat[(size_t)bh * N + own_row];
-        const int o0 = first_other(ob), o1 = last_other(ob);
-        for (int ot = o0; ot <= o1; ++ot) {
-            const int st = S == 2 ? (ot - o0) & 1 : 0;
-            if (kside && tid < kC) {
-                const int r = ot * kC + tid;
-                ostat[tid] = r < N ? rowstat[(size_t)bh * N + r] : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            ok = bar_wait(&tma_bar[st], (tph >> st) & 1u, &abort_flag, status);
-            tph ^= 1u << st;
-            ok = !__syncthreads_or(!ok);
-            if (!ok) break;
-            fence_after_sync();
-            if (tid == 0) {
-                // the other stage was last read by the previous block's MMAs, now complete
-                if (S == 2 && ot < o1) load(ob, ot + 1, st ^ 1, false);
-                const uint64_t dXT = sdesc(sb + xt(st), 16, 1024);
-                const uint64_t dPT = sdesc(sb + xt(st) + 16384, 16, 1024);
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_bf16(tm + L::T_S, adv(dXO, ks * 32), adv(dXT, ks * 32), I_KK128, ks > 0);
-#pragma unroll
-                for (int ks = 0; ks < 4 * G2; ++ks) {
-                    const uint32_t kofs = (ks >> 2) * 16384 + (ks & 3) * 32;
-                    mma_bf16(tm + L::T_A, adv(dPO, kofs), adv(dPT, kofs), I_KK128, ks > 0);
+    if (warp == kComputeG + 1) {
+        // ================= loader (a tile load takes the issuing warp about 0.2 us) ==========
+        [&]() {
+            int gs = 0;  // steps loaded so far: stage gs % ST
+            for (int ob = hb0; ob < hb1; ++ob) {
+                const int io = ob - hb0, b = io % L::OWN;
+                if (io >= L::OWN && !bar_wait_w(&ofree[b], (io / L::OWN - 1) & 1, &abort_flag, status))
+                    return;
+                const uint32_t xo = sb + L::XO(io);
+                wmbar_arrive_expect_tx(&town[b], L::OWN_BYTES);
+                for (int r = 0; r < 2; ++r) {  // (64-row boxes)
+                    wtma_load_3d(xo + r * 8192, x_own, 0, ob * kC + r * 64, bh, &town[b]);
+                    for (int g = 0; g < G2; ++g)
+                        wtma_load_3d(xo + 16384 + g * 16384 + r * 8192, f_own, 64 * g, ob * kC + r * 64, bh,
+                                     &town[b]);
+                }
+                const int n = last_step(ob) - first_step(ob);
+                for (int j = 0; j < n; ++j, ++gs) {
+                    const int st = gs % ST;
+                    if (gs >= ST && !bar_wait_w(&sfree[st], (gs / ST - 1) & 1, &abort_flag, status)) return;
+                    const uint32_t dst = sb + L::ST0 + (uint32_t)st * L::STAGE_BYTES;
+                    const int r0 = (first_step(ob) + j) * kHalf;
+                    wmbar_arrive_expect_tx(&tx[st], L::STAGE_BYTES);
+                    wtma_load_3d(dst, x_oth, 0, r0, bh, &tx[st]);
+                    for (int g = 0; g < G2; ++g)
+                        wtma_load_3d(dst + 8192 + g * 8192, f_oth, 64 * g, r0, bh, &tx[st]);
                 }
             }
-            if (!(ok = commit_wait())) break;
-            // G over this thread's 32 columns (two rounds of 16), bf16 in place over A in
-            // the first 16 of them; a block with no masked entry skips the mask tests
-            const bool full = (ot + 1) * kC <= N && (ob + 1) * kC <= N &&
-                              (!causal || (kside ? ot > ob : ot < ob));
+        }();
+        __syncwarp();
+    } else if (warp == kComputeG) {
+        // ================= issuer (a whole warp, one elected lane per operation) =============
+        constexpr uint32_t I_S = idesc_bf16(128, kHalf, 0, 0);
+        constexpr uint32_t I_DPHI = idesc_bf16(128, 64 * G2, 0, 1);  // N = 2M features
+        constexpr uint32_t I_PROJ = idesc_bf16(128, P, 0, 0);
+        constexpr uint32_t I_DW = idesc_bf16(128, 64, 1, 1);
+        [&]() {
+            auto adv = [](uint64_t dsc, uint32_t bytes) { return dsc + (bytes >> 4); };
+            uint32_t p_rdy[2] = {0, 0}, p_rdyc = 0, p_md = 0, p_mc = 0;
+            int gs0 = 0;  // steps of the earlier held blocks
+            for (int ob = hb0; ob < hb1; ++ob) {
+                const int io = ob - hb0, n = last_step(ob) - first_step(ob);
+                const uint32_t xo = sb + L::XO(io), po = sb + L::PO(io);
+                const uint64_t dXO = sdesc(xo, 16, 1024), dPO = sdesc(po, 16, 1024);
+                const uint64_t dXOmn = sdesc(xo, 16384, 1024);
+                const uint64_t dDAmn = sdesc(sb + L::DA(io), 16384, 1024);
+                // dphi += G Phi of step j (G bf16 over its A columns, 16 keys in 8 columns)
+                auto issue_dphi = [&](int j) {
+                    const uint64_t dPT = sdesc(
+                        sb + L::ST0 + (uint32_t)((gs0 + j) % ST) * L::STAGE_BYTES + 8192, 8192, 1024);
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const uint32_t col = 32 * qd + 16 * b;
-                float sv[16], av[16];
-                tmem_ld16(tm_row + L::T_S + col, sv);
-                tmem_ld16(tm_row + L::T_A + col, av);
-                tmem_wait_ld();
-                uint32_t pk[8];
+                    for (int ks = 0; ks < 4; ++ks)
+                        wmma_bf16_tmem_a(tm + L::T_D, tm + L::T_SA + 128 * (j & 1) + 64 + 16 * ks,
+                                         adv(dPT, ks * 2048), I_DPHI, (j > 0 || ks > 0) ? 1u : 0u);
+                    wmma_commit(&md);
+                    wmma_commit(&sfree[(gs0 + j) % ST]);
+                };
+                // the compute warps are done with the previous held block (M = 64: and this one
+                // is in tensor memory)
+                if (!wwait(&rdyc, p_rdyc)) return;
+                if (!bar_wait_w(&town[io % L::OWN], (io / L::OWN) & 1, &abort_flag, status)) return;
+                fence_after_sync();
+                for (int j = 0; j <= n; ++j) {
+                    // (waited for before the next commit on md)
+                    if (j >= 2 && !wwait(&md, p_md)) return;
+                    if (j < n) {
+                        const int gs = gs0 + j, st = gs % ST;
+                        if (!bar_wait_w(&tx[st], (gs / ST) & 1, &abort_flag, status)) return;
+                        fence_after_sync();
+                        // (step j - 2's dphi, which reads this buffer, is complete)
+                        const uint32_t sa = tm + L::T_SA + 128 * (j & 1);
+                        const uint32_t xs = sb + L::ST0 + (uint32_t)st * L::STAGE_BYTES;
+                        const uint64_t dXT = sdesc(xs, 16, 1024), dPT = sdesc(xs + 8192, 16, 1024);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    float gv[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int c = (int)col + 2 * i + e;
-                        const float4 sts = kside ? ostat[c] : qs;
-                        const float a = av[2 * i + e];
-                        const float p = ex2f(fmaf(sv[2 * i + e], score_scale, -sts.x));
-                        const float g = (a * sts.y > 0.f ? __fdividef(p, a) : 0.f) - sts.z;
-                        if (full) {
-                            gv[e] = g;
-                        } else {
-                            const int orow = ot * kC + c;
-                            const int qi = kside ? orow : own_row, kj = kside ? own_row : orow;
-                            gv[e] = (own_valid && orow < N && (!causal || kj <= qi)) ? g : 0.f;
+                        for (int ks = 0; ks < 4; ++ks) {
+                            if (L::OWN_T)
+                                wmma_bf16_tmem_a(sa, tm + L::T_XO + 8 * ks, adv(dXT, ks * 32), I_S, ks > 0);
+                            else
+                                wmma_bf16(sa, adv(dXO, ks * 32), adv(dXT, ks * 32), I_S, ks > 0);
                         }
+#pragma unroll
+                        for (int ks = 0; ks < 4 * G2; ++ks) {
+                            const uint64_t pt = adv(dPT, (ks >> 2) * 8192 + (ks & 3) * 32);
+                            if (L::OWN_T)
+                                wmma_bf16_tmem_a(sa + 64, tm + L::T_PO + 8 * ks, pt, I_S, ks > 0);
+                            else
+                                wmma_bf16(sa + 64, adv(dPO, (ks >> 2) * 16384 + (ks & 3) * 32), pt, I_S,
+                                          ks > 0);
+                        }
+                        wmma_commit(&msa[j & 1]);
                     }
-                    pk[i] = pack_bf16(gv[0], gv[1]);
+                    if (j > 0) {
+                        if (!wwait(&rdy[(j - 1) & 1], p_rdy[(j - 1) & 1])) return;  // G of step j - 1
+                        issue_dphi(j - 1);
+                    }
                 }
-                tmem_st8(tm_row + L::T_A + 32 * qd + 8 * b, pk);
+                // chain rule through the feature map, one group of 64 frequencies at a time; it
+                // writes over the buffer the last step's dphi reads
+                if (!wwait(&md, p_md)) return;
+                for (int g = 0; g < G; ++g) {
+                    if (g > 0 && !wwait(&rdyc, p_rdyc)) return;  // the previous group's dW' is read
+                    const uint64_t dWg = sdesc(sb + L::WG + (uint32_t)g * P * 128, 16, 1024);
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks)
+                        wmma_bf16(tm + L::T_C, adv(dXO, ks * 32), adv(dWg, ks * 32), I_PROJ, ks > 0);
+                    wmma_commit(&mc);
+                    p_mc ^= 1;
+                    if (!wwait(&rdyc, p_rdyc)) return;  // da
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        wmma_bf16(tm + L::T_W, adv(dDAmn, ks * 2048), adv(dXOmn, ks * 2048), I_DW, ks > 0);
+                    wmma_commit(&mc);
+                    if (g + 1 == G) wmma_commit(&ofree[io % L::OWN]);
+                    if (!wwait(&mc, p_mc)) return;
+                }
+                gs0 += n;
             }
-            tmem_wait_st();
-            handoff();
-            if (tid == 0) {
-                fence_after_sync();
-                const uint64_t dPTmn = sdesc(sb + xt(st) + 16384, 16384, 1024);
+        }();
+        __syncwarp();
+    } else {
+        // ================= compute =================
+        // Steps: warps 0-7 take the even ones, 8-15 the odd ones (their tensor-memory latency
+        // then falls into the other group's arithmetic), a warp 32 of the 64 columns.
+        const int grp = warp / (kComputeG / 2);
+        uint32_t p_own[2] = {0, 0}, p_msa = 0, p_mc = 0;
+        for (int ob = hb0; ob < hb1; ++ob) {
+            const int own_row = ob * kC + t;
+            const bool own_valid = own_row < N;
+            const int o0 = first_step(ob), n = last_step(ob) - o0;
+            float4 qs = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!kside && own_valid) qs = rowstat[(size_t)bh * N + own_row];
+            // Key side: the streamed queries' statistics of step j, written by the group that
+            // takes it while that group's previous step runs (its other warps are past step
+            // j - 4, which had the slot).
+            auto stage_stat = [&](int j) {
+                const int c = tid & (32 * kComputeG / 2 - 1);
+                if (kside && c < kHalf && j < n) {
+                    const int r = (o0 + j) * kHalf + c;
+                    ostat[j & 3][c] =
+                        r < N ? rowstat[(size_t)bh * N + r] : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            };
+            stage_stat(grp);
+            if (!L::OWN_T) arrive(&rdyc);
+            const int ow = L::OWN_T ? (ob - hb0) & 1 : 0;
+            const uint32_t xo = L::XO(ob - hb0), po = L::PO(ob - hb0), da = sb + L::DA(ob - hb0);
+            if (!wwait(&town[ow], p_own[ow])) goto done;
+            if (L::OWN_T) {  // row t: x columns 16 qd .. + 15, features 32 qd .. + 31
+                auto to_tmem = [&](uint32_t src, uint32_t col, int chunk) {  // 16 values
+                    uint32_t r[8];
+                    *reinterpret_cast<uint4*>(&r[0]) =
+                        *reinterpret_cast<const uint4*>(sm + src + swz128(t, 8 * chunk));
+                    *reinterpret_cast<uint4*>(&r[4]) =
+                        *reinterpret_cast<const uint4*>(sm + src + swz128(t, 8 * chunk + 8));
+                    tmem_st8(tm_row + col, r);
+                };
+                to_tmem(xo, L::T_XO + 8 * qd, 2 * qd);
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)  // K = streamed rows 16 ks .. 16 ks + 15
-                    mma_bf16_tmem_a(tm + L::T_D, tm + L::T_A + 32 * (ks >> 1) + 8 * (ks & 1),
-                                    adv(dPTmn, ks * 2048), I_DPHI, (ot > o0 || ks > 0) ? 1u : 0u);
+                for (int b = 0; b < 2; ++b)
+                    to_tmem(po + (qd >> 1) * 16384, L::T_PO + 16 * qd + 8 * b, 4 * (qd & 1) + 2 * b);
+                tmem_wait_st();
+                arrive(&rdyc);
             }
-            if (!(ok = commit_wait())) break;
-            if (S == 1 && tid == 0 && ot < o1) load(ob, ot + 1, 0, false);
-        }
-        if (!ok) break;
-
-        // chain rule through the feature map, one group of 64 frequencies at a time
-        const float wk = (KW && kside && own_valid) ? kw[(size_t)bh * N + own_row] : 1.f;
-        const float scl = sigma * wk;  // dphi(x) = scl T_D (key side: dphi = w dphi~)
-        float sdot = 0.f;              // key side: phi(k) . T_D over this thread's features
-        float kk = 0.f;                // key side: |k_j|^2 from the held tile (read before
-        if (KW && kside) {             // the group loop: the next block's load reuses it)
+            float kk = 0.f;  // key side: |k_j|^2 from the held tile
+            if (KW && kside) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint4 k4 = *reinterpret_cast<const uint4*>(sm + L::XO + swz128(t, 8 * j));
-                const uint32_t kw4[4] = {k4.x, k4.y, k4.z, k4.w};
+                for (int j = 0; j < 8; ++j) {
+                    const uint4 k4 = *reinterpret_cast<const uint4*>(sm + xo + swz128(t, 8 * j));
+                    const uint32_t kw4[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float k0 = __uint_as_float(kw4[e] << 16);
-                    const float k1 = __uint_as_float(kw4[e] & 0xFFFF0000u);
-                    kk = fmaf(k0, k0, fmaf(k1, k1, kk));
+                    for (int e = 0; e < 4; ++e) {
+                        const float k0 = __uint_as_float(kw4[e] << 16);
+                        const float k1 = __uint_as_float(kw4[e] & 0xFFFF0000u);
+                        kk = fmaf(k0, k0, fmaf(k1, k1, kk));
+                    }
                 }
             }
-        }
-        for (int g = 0; g < G && ok; ++g) {
-            if (tid == 0) {
-                fence_after_sync();  // after the previous group's barrier
-                const uint64_t dWg = sdesc(sb + L::WG + (uint32_t)g * P * 128, 16, 1024);
+            for (int j = grp; j < n; j += 2) {
+                if (!wwait(&msa[grp], p_msa)) goto done;
+                stage_stat(j + 2);
+                // G over this warp's 32 columns, sixteen at a time, bf16 over the first 8 of the
+                // sixteen in A; a step with no masked entry skips the mask tests.  The step's
+                // two conditions are compile-time: tested per entry they cost as much as G.
+                const int r0 = (o0 + j) * kHalf;
+                const bool full = r0 + kHalf <= N && (ob + 1) * kC <= N &&
+                                  (!causal || (kside ? r0 >= ob * kC + kC - 1 : r0 + kHalf - 1 <= ob * kC));
+                auto form_g = [&](auto full_tag, auto kside_tag) {
+                    constexpr bool FULL = decltype(full_tag)::value, KS = decltype(kside_tag)::value;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_bf16(tm + L::T_S, adv(dXO, ks * 32), adv(dWg, ks * 32), I_PROJ, ks > 0);
+                    for (int b = 0; b < 2; ++b) {
+                        const int c0 = 32 * (qd & 1) + 16 * b;
+                        const uint32_t sa = tm_row + L::T_SA + 128 * grp + c0;
+                        float sv[16], av[16];
+                        tmem_ld16(sa, sv);
+                        tmem_ld16(sa + 64, av);
+                        tmem_wait_ld();
+                        uint32_t pk[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            float gv[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int c = c0 + 2 * i + e;
+                                const float4 sts = KS ? ostat[j & 3][c] : qs;
+                                const float a = av[2 * i + e];
+                                const float p = ex2f(fmaf(sv[2 * i + e], score_scale, -sts.x));
+                                // (branch-free: what p / a gives at a <= 0 is not used)
+                                gv[e] = (a * sts.y > 0.f ? p * rcpf(a) : 0.f) - sts.z;
+                                if (!FULL) {
+                                    const int orow = r0 + c;
+                                    const int qi = KS ? orow : own_row, kj = KS ? own_row : orow;
+                                    if (!(own_valid && orow < N && (!causal || kj <= qi))) gv[e] = 0.f;
+                                }
+                            }
+                            pk[i] = pack_bf16(gv[0], gv[1]);
+                        }
+                        tmem_st8(sa + 64, pk);
+                    }
+                };
+                if (kside)
+                    full ? form_g(std::true_type{}, std::true_type{})
+                         : form_g(std::false_type{}, std::true_type{});
+                else
+                    full ? form_g(std::true_type{}, std::false_type{})
+                         : form_g(std::false_type{}, std::false_type{});
+                tmem_wait_st();
+                arrive(&rdy[grp]);
             }
-            if (!(ok = commit_wait())) break;
-            // this thread's 16 frequencies of the group: 64 g + 16 qd + [0, 16)
-            float dc[16], ds[16], u[16], w[16];
-            tmem_ld16(tm_row + L::T_D + 64 * g + 16 * qd, dc);
-            tmem_ld16(tm_row + L::T_D + M + 64 * g + 16 * qd, ds);
-            float mu, mw = 0.f;  // max |x| per load
-            tmem_ld16_maxabs(tm_row + L::T_S + 16 * qd, u, mu);
-            if (NS) tmem_ld16_maxabs(tm_row + L::T_S + 64 + 16 * qd, w, mw);
-            tmem_wait_ld();
-            if (NS)
-                reduce_2pi_if_needed(u, w, fmaxf(mu, mw));
-            else
-                reduce_2pi_if_needed(u, mu);
-            uint32_t o1[8], o2[8];
+            const float wk = (KW && kside && own_valid) ? kw[(size_t)bh * N + own_row] : 1.f;
+            const float scl = sigma * wk;  // dphi(x) = scl T_D (key side: dphi = w dphi~)
+            float sdot = 0.f;              // key side: phi(k) . T_D over this thread's features
+            for (int g = 0; g < G; ++g) {
+                if (!wwait(&mc, p_mc)) goto done;  // dphi complete, the projection of group g
+                // this thread's 16 frequencies of the group: 64 g + 16 qd + [0, 16)
+                float dc[16], ds[16], u[16], w[16];
+                tmem_ld16(tm_row + L::T_D + 64 * g + 16 * qd, dc);
+                tmem_ld16(tm_row + L::T_D + M + 64 * g + 16 * qd, ds);
+                float mu, mw = 0.f;  // max |x| per load
+                tmem_ld16_maxabs(tm_row + L::T_C + 16 * qd, u, mu);
+                if (NS) tmem_ld16_maxabs(tm_row + L::T_C + 64 + 16 * qd, w, mw);
+                tmem_wait_ld();
+                if (NS)
+                    reduce_2pi_if_needed(u, w, fmaxf(mu, mw));
+                else
+                    reduce_2pi_if_needed(u, mu);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                float r1[2], r2[2];
+                for (int j = 0; j < 2; ++j) {
+                    uint32_t o1[4], o2[4];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int f = 2 * i + e;
-                    float su, cu;
-                    __sincosf(u[f], &su, &cu);
-                    float cw = 1.f, sw = 0.f;
-                    if (NS) __sincosf(w[f], &sw, &cw);
-                    const float dpc = scl * dc[f], dps = scl * ds[f];
-                    r1[e] = cM * cw * (-su * dpc + cu * dps);
-                    r2[e] = NS ? -cM * sw * (cu * dpc + su * dps) : 0.f;
-                    if (KW) sdot = fmaf(cu * cw, dc[f], fmaf(su * cw, ds[f], sdot));
-                    if (!own_valid) r1[e] = r2[e] = 0.f;
+                    for (int i = 0; i < 4; ++i) {
+                        float r1[2], r2[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int f = 8 * j + 2 * i + e;
+                            float su, cu;
+                            __sincosf(u[f], &su, &cu);
+                            float cw = 1.f, sw = 0.f;
+                            if (NS) __sincosf(w[f], &sw, &cw);
+                            const float dpc = scl * dc[f], dps = scl * ds[f];
+                            r1[e] = cM * cw * (-su * dpc + cu * dps);
+                            r2[e] = NS ? -cM * sw * (cu * dpc + su * dps) : 0.f;
+                            if (KW) sdot = fmaf(cu * cw, dc[f], fmaf(su * cw, ds[f], sdot));
+                            if (!own_valid) r1[e] = r2[e] = 0.f;
+                        }
+                        o1[i] = pack_bf16(r1[0], r1[1]);
+                        o2[i] = pack_bf16(r2[0], r2[1]);
+                    }
+                    const uint32_t off = swz128(t, (2 * qd + j) * 8);
+                    st_shared_v4(da + off, o1[0], o1[1], o1[2], o1[3]);
+                    st_shared_v4(da + 16384 + off, o2[0], o2[1], o2[2], o2[3]);
                 }
-                o1[i] = pack_bf16(r1[0], r1[1]);
-                o2[i] = pack_bf16(r2[0], r2[1]);
-            }
+                arrive(&rdyc);
+                if (!wwait(&mc, p_mc)) goto done;
+                // rows of dW' (lane = projection row), this thread's 16 columns, into the slot
+                // ([16 column quads][128 rows][4]: a warp's accesses are contiguous)
+                float v[16];
+                tmem_ld16(tm_row + L::T_W + 16 * qd, v);
+                tmem_wait_ld();
+                float4* dst = reinterpret_cast<float4*>(slots) +
+                              (((size_t)blockIdx.x * G + g) * 16 + 4 * qd) * 128 + t;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint32_t off = swz128(t, (2 * qd + j) * 8);
-                st_shared_v4(sb + L::DA + off, o1[4 * j], o1[4 * j + 1], o1[4 * j + 2], o1[4 * j + 3]);
-                st_shared_v4(sb + L::DA + 16384 + off, o2[4 * j], o2[4 * j + 1], o2[4 * j + 2],
-                             o2[4 * j + 3]);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 old = ob == hb0 ? make_float4(0.f, 0.f, 0.f, 0.f) : dst[128 * j];
+                    dst[128 * j] = make_float4(old.x + v[4 * j], old.y + v[4 * j + 1],
+                                               old.z + v[4 * j + 2], old.w + v[4 * j + 3]);
+                }
+                if (g + 1 < G) arrive(&rdyc);  // (after the last group: the next block's arrival)
             }
-            handoff();
-            if (tid == 0) {
-                fence_after_sync();
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_bf16(tm + L::T_A, adv(dDAmn, ks * 2048), adv(dXOmn, ks * 2048), I_DW, ks > 0);
-            }
-            if (!(ok = commit_wait())) break;
-            // rows of dW' (lane = projection row), this thread's 16 columns, into the slot
-            float v[16];
-            tmem_ld16(tm_row + L::T_A + 16 * qd, v);
-            tmem_wait_ld();
-            float4* dst = reinterpret_cast<float4*>(
-                slots + (((size_t)blockIdx.x * G + g) * 128 + t) * 64 + 16 * qd);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 old = ob == hb0 ? make_float4(0.f, 0.f, 0.f, 0.f) : dst[j];
-                dst[j] = make_float4(old.x + v[4 * j], old.y + v[4 * j + 1], old.z + v[4 * j + 2],
-                                     old.w + v[4 * j + 3]);
-            }
-            // tensor memory, the W' rows and the da tiles are free once every thread is here
-            fence_before_sync();
-            __syncthreads();
+            if (KW && kside && own_valid)  // s_j = phi~(k_j) . dphi~(k_j) = w cM sigma sdot
+                dtau_acc -= wk * cM * sigma * sdot * kk * itau;
         }
-        if (!ok) break;
-        if (KW && kside && own_valid)  // s_j = phi~(k_j) . dphi~(k_j) = w cM sigma sdot
-            dtau_acc -= wk * cM * sigma * sdot * kk * itau;
-        if (tid == 0 && ob + 1 < hb1) load(ob + 1, first_other(ob + 1), 0, true);
     }
 
+done:
+    __syncthreads();
+    if (abort_flag && tid == 0) {  // gave up: let copies into this CTA's shared memory land
+        const long long t0 = clock64();
+        while (clock64() - t0 < kDrainCycles) {
+        }
+    }
     // dtau partial of this CTA, summed in a fixed order
     float dsum = dtau_acc;
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
     if (lane == 0) wsum[warp] = dsum;
-    __syncthreads();
-    if (tid == 0) {
-        float tot = 0.f;
-        for (int w8 = 0; w8 < kThreadsG / 32; ++w8) tot += wsum[w8];
-        dtau_part[blockIdx.x] = tot;
-    }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
+    if (tid == 0) {
+        float tot = 0.f;
+        for (int w8 = 0; w8 < kComputeG; ++w8) tot += wsum[w8];
+        dtau_part[blockIdx.x] = tot;
+    }
     if (warp == 0) tmem_dealloc(tm, 512);
 }
 
-// dW1, dW2 [H][M][64] and dtau [H] from the slots [2 sides][B*H][hsplit][G][128 rows][64].
-// One block of 512 threads per (head, frequency): column c = tid % 64, lane = tid / 64 sums
-// the slots s = lane, lane + 8, ... (s in (side, batch entry, split) order), eight loads in
-// flight; the eight lane sums are then added in lane order, so the order is fixed.  For
-// Flexformer_n rows 0-63 of a group are dU, rows 64-127 dV (U = (W1+W2)/2, V = (W1-W2)/2),
-// so dW1 = (dU+dV)/2, dW2 = (dU-dV)/2.
-constexpr int kReduceLanes = 8;
-__global__ void __launch_bounds__(64 * kReduceLanes)
+// dW1, dW2 [H][M][64] and dtau [H] from the slots [2 sides][B*H][hsplit][G][16 column
+// quads][128 rows][4].  One block per (head, group, column quad): thread (row, lane) sums
+// every fourth slot (slots in (side, batch entry, split) order) with eight loads in flight;
+// the four lanes are then added in order.  For Flexformer_n rows 0-63 of a group are dU, rows
+// 64-127 dV (U = (W1+W2)/2, V = (W1-W2)/2), so dW1 = (dU+dV)/2, dW2 = (dU-dV)/2.
+constexpr int kReduceThreads = 512;
+__global__ void __launch_bounds__(kReduceThreads)
     awd_dw_reduce_kernel(int B, int H, int M, int nonstat, int hsplit,
                          const float* __restrict__ slots, const float* __restrict__ dtau_part,
                          float* __restrict__ dW1, float* __restrict__ dW2,
                          float* __restrict__ dtau)
 {
-    __shared__ float part[2][kReduceLanes][64];
+    __shared__ float4 sums[3][128];
     const int BH = B * H, G = M / 64, per_side = B * hsplit, nslot = 2 * per_side;
-    const size_t slot_floats = (size_t)G * 128 * 64;
-    const int c = threadIdx.x % 64, lane = threadIdx.x / 64;
-    const int f = blockIdx.x % M, h = blockIdx.x / M;
-    const float* base = slots + ((size_t)(f / 64) * 128 + f % 64) * 64 + c;
-    float su = 0.f, sv = 0.f;
-    for (int s0 = lane; s0 < nslot; s0 += 8 * kReduceLanes) {
-        float a[8], bq[8];
+    const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
+    const int row = threadIdx.x % 128, ln = threadIdx.x / 128;
+    auto add = [](float4& a, const float4& x) {
+        a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
+    };
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = ln; s0 < nslot; s0 += 32) {
+        float4 x[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const int s = s0 + e * kReduceLanes;
-            a[e] = bq[e] = 0.f;
-            if (s < nslot) {
-                const int side = s / per_side, rem = s % per_side;
-                const size_t cta = (size_t)(side * BH + (rem / hsplit) * H + h) * hsplit +
-                                   rem % hsplit;
-                a[e] = base[cta * slot_floats];
-                if (nonstat) bq[e] = base[cta * slot_floats + 64 * 64];
-            }
+            const int s = s0 + 4 * e, side = s / per_side, rem = s % per_side;
+            const size_t cta = (size_t)(side * BH + (rem / hsplit) * H + h) * hsplit + rem % hsplit;
+            x[e] = s < nslot ? reinterpret_cast<const float4*>(slots)[((cta * G + g) * 16 + quad) * 128 + row]
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            su += a[e];
-            sv += bq[e];
-        }
+        for (int e = 0; e < 8; ++e) add(a, x[e]);
     }
-    part[0][lane][c] = su;
-    part[1][lane][c] = sv;
+    if (ln > 0) sums[ln - 1][row] = a;
     __syncthreads();
-    if (lane == 0) {
-        float tu = 0.f, tv = 0.f;
-        for (int l = 0; l < kReduceLanes; ++l) {
-            tu += part[0][l][c];
-            tv += part[1][l][c];
-        }
-        const size_t idx = ((size_t)h * M + f) * 64 + c;
+    if (ln == 0) {
+        for (int l = 0; l < 3; ++l) add(a, sums[l][row]);
+        if (row >= 64) sums[0][row] = a;
+    }
+    __syncthreads();
+    if (ln == 0 && row < 64) {
+        const size_t o = (((size_t)h * M + 64 * g + row) * 64 + 4 * quad) / 4;
         if (nonstat) {
-            dW1[idx] = 0.5f * (tu + tv);
-            dW2[idx] = 0.5f * (tu - tv);
+            const float4 b = sums[0][64 + row];
+            reinterpret_cast<float4*>(dW1)[o] = make_float4(0.5f * (a.x + b.x), 0.5f * (a.y + b.y),
+                                                            0.5f * (a.z + b.z), 0.5f * (a.w + b.w));
+            reinterpret_cast<float4*>(dW2)[o] = make_float4(0.5f * (a.x - b.x), 0.5f * (a.y - b.y),
+                                                            0.5f * (a.z - b.z), 0.5f * (a.w - b.w));
         } else {
-            dW1[idx] = tu;
+            reinterpret_cast<float4*>(dW1)[o] = a;
         }
     }
-    if (dtau && blockIdx.x == 0)
-        for (int hh = threadIdx.x; hh < H; hh += blockDim.x) {
-            float sd = 0.f;
-            for (int b = 0; b < B; ++b)
-                for (int r = 0; r < hsplit; ++r)  // key side
-                    sd += dtau_part[(size_t)(BH + b * H + hh) * hsplit + r];
-            dtau[hh] = sd;
-        }
+    if (dtau && quad == 0 && g == 0 && threadIdx.x < 32) {  // the key side's partials of head h
+        float t = 0.f;
+        for (int i = threadIdx.x; i < per_side; i += 32)
+            t += dtau_part[(size_t)(BH + i / hsplit * H + h) * hsplit + i % hsplit];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) dtau[h] = t;
+    }
 }
 
 template <int G2>
@@ -714,8 +842,9 @@ cudaError_t launch_bwd_typed(const Problem& p, const void* q, const void* k, con
 {
     const int BH = p.B * p.H;
     CUtensorMap mq, mk, mpq, mpk;
-    if (!make_act_map(&mq, q, BH, p.N) || !make_act_map(&mk, k, BH, p.N) ||
-        !make_feat_map(&mpq, pq, BH, p.N, 2 * p.M) || !make_feat_map(&mpk, pk, BH, p.N, 2 * p.M))
+    if (!make_feat_map(&mq, q, BH, p.N, 64, kHalf) || !make_feat_map(&mk, k, BH, p.N, 64, kHalf) ||
+        !make_feat_map(&mpq, pq, BH, p.N, 2 * p.M, kHalf) ||
+        !make_feat_map(&mpk, pk, BH, p.N, 2 * p.M, kHalf))
         return cudaErrorInvalidValue;
     const int smem = (int)AwdBwCfg<G2>::BYTES + 1024;
     auto kern = tc_awd_bwd_kernel<G2, NS, KW>;
@@ -727,7 +856,7 @@ cudaError_t launch_bwd_typed(const Problem& p, const void* q, const void* k, con
                                               score_scale, rowstat, dloss, W1, W2, kw, tau, slots,
                                               dtau_part, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    awd_dw_reduce_kernel<<<p.H * p.M, 64 * kReduceLanes, 0, s>>>(
+    awd_dw_reduce_kernel<<<p.H * (p.M / 64) * 16, kReduceThreads, 0, s>>>(
         p.B, p.H, p.M, p.nonstat, hs, slots, dtau_part, dW1, dW2, tau ? dtau : nullptr);
     return cudaGetLastError();
 }

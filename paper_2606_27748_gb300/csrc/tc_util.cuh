@@ -343,15 +343,15 @@ __device__ __forceinline__ void stage_freq_rows_split(uint32_t dst_hi, uint32_t 
     }
 }
 
-// [BH][N][F] bf16 rows of F features (F a multiple of 64), box 64 x 128, 128B swizzle:
-// a load at x = 64 g brings feature block g of 128 rows.
-inline bool make_feat_map(CUtensorMap* m, const void* base, int BH, int N, int F)
+// [BH][N][F] bf16 rows of F features (F a multiple of 64), box 64 x `rows`, 128B swizzle:
+// a load at x = 64 g brings feature block g of that many rows.
+inline bool make_feat_map(CUtensorMap* m, const void* base, int BH, int N, int F, int rows = 128)
 {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
     cuuint64_t dims[3] = {(cuuint64_t)F, (cuuint64_t)N, (cuuint64_t)BH};
     cuuint64_t strides[2] = {(cuuint64_t)F * 2, (cuuint64_t)N * F * 2};
-    cuuint32_t box[3] = {64, 128, 1};
+    cuuint32_t box[3] = {64, (cuuint32_t)rows, 1};
     cuuint32_t es[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
                box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
