@@ -484,6 +484,30 @@ __device__ __forceinline__ void bulk_copy_cluster(uint32_t dst_cluster, uint32_t
         : "memory");
 }
 
+// Bulk copy of `bytes` from global memory into this CTA's shared memory, completing that
+// transaction count on an mbarrier.  Addresses 16-byte aligned, size a multiple of 16.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, void* mbar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            dst),
+        "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+        : "memory");
+}
+
+// ---- programmatic dependent launch --------------------------------------------------------
+// In a kernel launched with the stream-serialization attribute: wait for the preceding grid to
+// finish (its results are visible afterwards); anywhere: let the following such grid's CTAs
+// start once every CTA of this grid has started.
+__device__ __forceinline__ void grid_dep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Arrive on an mbarrier of a CTA of the cluster (shared::cluster address), releasing this
 // thread's earlier shared-memory writes at cluster scope.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr)

@@ -7,8 +7,9 @@
 //   1. state:  every (b, h, split) unit runs over its chunks of 128 tokens: projection of
 //              k (TMEM) -> cos/sin features (CUDA cores, bf16 in shared memory) ->
 //              [S | z]_part += phi(K)^T [V | 1] (TMEM), then writes its partial in fp32;
-//   2. reduce: the partials of a sequence are summed in a fixed order (deterministic);
-//   3. output: every unit loads the total as a bf16 operand and runs over its chunks:
+//   2. reduce: the partials of a sequence are summed in a fixed order (deterministic) and
+//              written as the output kernel's bf16 operand;
+//   3. output: every unit copies that operand into shared memory and runs over its chunks:
 //              projection of q -> features -> phi(Q) [S | z] (TMEM) -> out = num / den.
 //
 // z rides as column 64 of [S | z]: the state MMA multiplies by [V | 1] (a constant ones
@@ -52,7 +53,7 @@ struct NcCfg {
     static constexpr uint32_t W = 81920;
     static constexpr uint32_t PB0 = W + G * P * 128, PB1 = PB0 + 32768;
     static constexpr uint32_t SX = PB1 + 32768;
-    static constexpr uint32_t SX_BLOCK = 80 * 128, SX_GROUP = 2 * SX_BLOCK;
+    static constexpr uint32_t SX_BLOCK = 80 * 128, SX_GROUP = 2 * SX_BLOCK;  // as kSxBlock, kSxGroup
     static constexpr uint32_t BYTES = SX + G * SX_GROUP;
     static constexpr uint32_t T_P0 = 0, T_P1 = 128, T_S = 256, T_O0 = 256, T_O1 = 336;
     static_assert(T_S + 80 * G <= 512 && T_O1 + 80 <= 512, "tensor memory budget");
@@ -62,11 +63,15 @@ struct NcCfg {
 struct NcBars {
     uint64_t x_full[2], x_free[2], v_full[2], v_free[2];
     uint64_t p_full[2], p_free[2], phi_full[2], phi_free[2];
-    uint64_t o_full[2], o_free[2], state_done;
+    uint64_t o_full[2], o_free[2], state_done, sx_full;
 };
 
-// partial / total [S | z] rows: [unit][group][feature 128][80 floats]
-constexpr int kRow = 80;
+// Partial [S | z]: [unit][group][17 column quads][128 features] float4 (columns 0-64 in use; a
+// warp's lanes are features, so its accesses are contiguous).
+constexpr int kQuads = 17, kPartFloats = kQuads * 128 * 4;
+// Total: the output kernel's operand as it lies in shared memory, per (sequence, group): two
+// blocks of 64 features, each 80 rows (S columns, z, zeros) of 128 bytes, bf16, 128-byte swizzle.
+constexpr uint32_t kSxBlock = 80 * 128, kSxGroup = 2 * kSxBlock;
 
 // KW: key weights of the norm prefactor given (compile-time; the plain kernel is unchanged)
 template <int MODE, bool NS, int G, bool KW>
@@ -75,7 +80,7 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                  const __grid_constant__ CUtensorMap tmap_v, int H, int N, int M, int splits,
                  const float* __restrict__ W1, const float* __restrict__ W2,
                  const float* __restrict__ kw, float* __restrict__ part,
-                 const float* __restrict__ total, __nv_bfloat16* __restrict__ out,
+                 const uint8_t* __restrict__ total, __nv_bfloat16* __restrict__ out,
                  float* __restrict__ den, int* status)
 {
     using L = NcCfg<NS, G>;
@@ -92,41 +97,15 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
     const int c0 = (int)((long long)sp * nch / splits), c1 = (int)((long long)(sp + 1) * nch / splits);
     const int nc = c1 - c0;  // chunks of this unit (>= 1: splits <= nch)
 
-    // ---- set-up: frequencies, [V | 1] ones block, [S | z] snapshot (output phase) ----
-    for (int idx = tid; idx < G * L::P * 8; idx += kThreadsNC) {
-        const int row = idx >> 3, c = idx & 7;
-        const int g = row / L::P, r = row % L::P;
-        const int f = 64 * g + (r & 63);
-        const float* w1 = W1 + ((size_t)h * M + f) * 64 + c * 8;
-        float x[8];
-        if (!NS) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) x[e] = w1[e];
-        } else {
-            const float* w2 = W2 + ((size_t)h * M + f) * 64 + c * 8;
-            const float sgn = r < 64 ? 1.f : -1.f;  // U = (W1+W2)/2, V = (W1-W2)/2
-#pragma unroll
-            for (int e = 0; e < 8; ++e) x[e] = 0.5f * (w1[e] + sgn * w2[e]);
-        }
-        st_shared_v4(sb + L::W + g * L::P * 128 + swz128(r, c * 8), pack_bf16(x[0], x[1]),
-                     pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
-    }
+    // ---- set-up: frequencies, [V | 1] ones block ----
+    if (MODE == kState) grid_dep_launch();
+    if (tid < 512) stage_freq_rows<NS, G, 512>(sb + L::W, W1, W2, h, M, tid);
     if (MODE == kState) {
         for (int idx = tid; idx < 16384 / 16; idx += kThreadsNC)
             st_shared_v4(sb + L::VONE + idx * 16, 0, 0, 0, 0);
         __syncthreads();
         for (int r = tid; r < kC; r += kThreadsNC)
             *reinterpret_cast<uint16_t*>(sm + L::VONE + swz128(r, 0)) = 0x3F80u;  // 1.0
-    } else {
-        // K-major [S | z]: row e (dcol e, z at 64, zero rows 65-79) over features f
-        const float* tot = total + (size_t)bh * G * 128 * kRow;
-        for (int idx = tid; idx < G * 128 * 80; idx += kThreadsNC) {
-            const int g = idx / (128 * 80), rem = idx % (128 * 80);
-            const int e = rem / 128, f = rem % 128;
-            const float val = e <= 64 ? tot[((size_t)g * 128 + f) * kRow + e] : 0.f;
-            *reinterpret_cast<__nv_bfloat16*>(sm + L::SX + g * L::SX_GROUP + (f >> 6) * L::SX_BLOCK +
-                                              swz128(e, f & 63)) = __float2bfloat16_rn(val);
-        }
     }
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
@@ -142,6 +121,7 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
             mbar_init(&bars.o_free[i], 4);
         }
         mbar_init(&bars.state_done, 1);
+        mbar_init(&bars.sx_full, 1);
         abort_flag = 0;
         fence_mbar_init();
     }
@@ -238,6 +218,14 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                 if (g == G - 1) wmma_commit(&bars.x_free[ib]);
             }
             if (warp == kWarpCons) {
+                if (MODE == kOut) {  // the totals: the only thing here that an earlier kernel wrote
+                    wmbar_arrive_expect_tx(&bars.sx_full, G * L::SX_GROUP);
+                    grid_dep_wait();
+                    if (elect_one())
+                        bulk_load(sb + L::SX, total + (size_t)bh * G * kSxGroup, G * L::SX_GROUP,
+                                  &bars.sx_full);
+                    wait(&bars.sx_full, 0);
+                }
                 for (int j = 0; j < njobs && ok; ++j) consume(j);
                 if (ok && MODE == kState) wmma_commit(&bars.state_done);
             }
@@ -324,19 +312,21 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
             }
             if (bar_wait(&bars.state_done, 0, &abort_flag, status)) {
                 fence_after_sync();
-                float* dst = part + ((size_t)blockIdx.x * G * 128 + t) * kRow;
-                for (int g = 0; g < G; ++g) {
-                    float4* d4 = reinterpret_cast<float4*>(dst + (size_t)g * 128 * kRow);
+                float4* dst = reinterpret_cast<float4*>(part) + (size_t)blockIdx.x * G * kQuads * 128 + t;
+                for (int g = 0; g < G; ++g, dst += kQuads * 128) {
 #pragma unroll
-                    for (int j = 0; j < 5; ++j) {  // 16 columns at a time (register budget)
+                    for (int j = 0; j < 4; ++j) {  // 16 columns at a time (register budget)
                         float s_[16];
                         tmem_ld16(tm_row + L::T_S + 80 * g + 16 * j, s_);
                         tmem_wait_ld();
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            d4[4 * j + e] = make_float4(s_[4 * e], s_[4 * e + 1], s_[4 * e + 2],
-                                                        s_[4 * e + 3]);
+                            dst[(4 * j + e) * 128] = make_float4(s_[4 * e], s_[4 * e + 1],
+                                                                 s_[4 * e + 2], s_[4 * e + 3]);
                     }
+                    const float z = tmem_ld1(tm_row + L::T_S + 80 * g + 64);
+                    tmem_wait_ld();
+                    dst[16 * 128] = make_float4(z, 0.f, 0.f, 0.f);
                 }
             }
         } else {
@@ -400,19 +390,58 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
     if (warp == kWarpMMA) tmem_dealloc(tm, 512);
 }
 
-// total[bh][g][f][e] = sum over splits, in split order.
-__global__ void nc_reduce_kernel(int BH, int splits, int G, const float* __restrict__ part,
-                                 float* __restrict__ total)
+// Sums of a sequence's partials in split order, rounded to bf16 and laid out as the output
+// kernel's operand.  One block per (sequence, group, 64 features): thread -> (column quad,
+// feature), the splits' loads independent.
+constexpr int kReduceThreads = 544;  // half of the 17 x 64 float4 of a block
+__global__ void __launch_bounds__(kReduceThreads)
+    nc_reduce_kernel(int splits, int G, const float* __restrict__ part, uint8_t* __restrict__ total)
 {
-    const size_t per = (size_t)G * 128 * kRow;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < (size_t)BH * per;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = idx / per, e = idx % per;
-        const float* p = part + b * splits * per + e;
-        float acc = 0.f;
-        for (int s = 0; s < splits; ++s) acc += p[(size_t)s * per];
-        total[idx] = acc;
+    __shared__ __align__(16) uint8_t image[kSxBlock];
+    const int fb = blockIdx.x & 1, g = (blockIdx.x >> 1) % G, bh = (blockIdx.x >> 1) / G;
+    grid_dep_launch();
+    for (int i = threadIdx.x; i < (int)kSxBlock / 16; i += kReduceThreads)
+        reinterpret_cast<uint4*>(image)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    grid_dep_wait();
+    const float4* src = reinterpret_cast<const float4*>(part) +
+                        ((size_t)bh * splits * G + g) * kQuads * 128 + 64 * fb;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int i = threadIdx.x + r * kReduceThreads, q = i / 64, f = i % 64;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int s = 0; s < splits; ++s) {
+            const float4 x = src[(size_t)s * G * kQuads * 128 + q * 128 + f];
+            a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
+        }
+        const float v[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            *reinterpret_cast<__nv_bfloat16*>(image + swz128(4 * q + e, f)) = __float2bfloat16_rn(v[e]);
     }
+    __syncthreads();
+    uint4* dst = reinterpret_cast<uint4*>(total + ((size_t)bh * G + g) * kSxGroup + fb * kSxBlock);
+    for (int i = threadIdx.x; i < (int)kSxBlock / 16; i += kReduceThreads)
+        dst[i] = reinterpret_cast<const uint4*>(image)[i];
+}
+
+// Launch that may overlap the preceding kernel's end (which the kernel waits for itself).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_after(void (*kern)(KArgs...), unsigned blocks, int threads, int smem,
+                         cudaStream_t s, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <bool NS, int G>
@@ -426,7 +455,7 @@ cudaError_t launch_nc(const Problem& p, const void* q, const void* k, const void
         !make_act_map(&mv, v, BH, p.N) || !make_act_map(&mo, out, BH, p.N))
         return cudaErrorInvalidValue;
     float* part = static_cast<float*>(scratch);
-    float* total = part + (size_t)BH * splits * G * 128 * kRow;
+    uint8_t* total = reinterpret_cast<uint8_t*>(part + (size_t)BH * splits * G * kPartFloats);
     const int smem = (int)NcCfg<NS, G>::BYTES + 1024;
     auto k_state = kw ? tc_nc_kernel<kState, NS, G, true> : tc_nc_kernel<kState, NS, G, false>;
     auto k_out = tc_nc_kernel<kOut, NS, G, false>;
@@ -437,13 +466,12 @@ cudaError_t launch_nc(const Problem& p, const void* q, const void* k, const void
     k_state<<<BH * splits, kThreadsNC, smem, s>>>(mk, mv, p.H, p.N, p.M, splits, W1, W2, kw,
                                                  part, nullptr, nullptr, nullptr, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t n = (size_t)BH * G * 128 * kRow;
-    nc_reduce_kernel<<<(int)std::min<size_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(BH, splits, G,
-                                                                                    part, total);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_out<<<BH * splits, kThreadsNC, smem, s>>>(mq, mo, p.H, p.N, p.M, splits, W1, W2, nullptr,
-                                               nullptr, total, (__nv_bfloat16*)out, den, status);
-    return cudaGetLastError();
+    e = launch_after(nc_reduce_kernel, 2u * BH * G, kReduceThreads, 0, s, splits, G,
+                     (const float*)part, total);
+    if (e != cudaSuccess) return e;
+    return launch_after(k_out, (unsigned)(BH * splits), kThreadsNC, smem, s, mq, mo, p.H, p.N, p.M,
+                        splits, W1, W2, (const float*)nullptr, (float*)nullptr,
+                        (const uint8_t*)total, (__nv_bfloat16*)out, den, status);
 }
 
 }  // namespace
@@ -478,7 +506,7 @@ int tc_nc_splits(const Problem& p)
 size_t tc_nc_ws_bytes(const Problem& p)
 {
     const size_t G = (size_t)p.M / 64, BH = (size_t)p.B * p.H;
-    return (BH * tc_nc_splits(p) + BH) * G * 128 * kRow * sizeof(float);
+    return (BH * tc_nc_splits(p) + BH) * G * 128 * 80 * sizeof(float);  // (17 of 20 quads in use)
 }
 
 cudaError_t launch_tc_nc(const Problem& p, const void* q, const void* k, const void* v,
