@@ -110,7 +110,7 @@ int flex_featmap(const flex_shape* shape, const void* x, const float* W1, const 
     if (!aligned(x, 16) || !aligned(W1, 16) || !aligned(phi, 16) || (W2 && !aligned(W2, 16)))
         return FLEX_EINVAL;
     if (flex::tc_featmap_supported(p))  // tensor-core projection (no workspace: no status)
-        return count(1, flex::launch_tc_featmap(p, x, W1, W2, nullptr, phi, nullptr,
+        return count(1, flex::launch_tc_featmap(p, x, W1, W2, nullptr, phi, nullptr, false,
                                                 (cudaStream_t)stream));
     return count(1, flex::launch_featmap(p, x, W1, W2, phi, (cudaStream_t)stream));
 }
@@ -251,9 +251,9 @@ int flex_awd_loss(const flex_shape* shape, const void* q, const void* k, const f
     float* kw = tau ? (float*)(base + w.kw) : nullptr;
     if (tau && (rc = count(1, flex::launch_key_weights(p, k, tau, kw, s)))) return rc;
     int* status = &((flex::WsHeader*)ws)->status;
-    if ((rc = count(1, flex::launch_tc_featmap(p, q, W1, W2, nullptr, base + w.pq, status, s))))
+    if ((rc = count(1, flex::launch_tc_featmap(p, q, W1, W2, nullptr, base + w.pq, status, tau != nullptr, s))))
         return rc;
-    if ((rc = count(1, flex::launch_tc_featmap(p, k, W1, W2, kw, base + w.pk, status, s))))
+    if ((rc = count(1, flex::launch_tc_featmap(p, k, W1, W2, kw, base + w.pk, status, true, s))))
         return rc;
     return count(2, flex::launch_tc_awd(p, q, k, base + w.pq, base + w.pk, (float*)(base + w.part),
                                         loss, status, s));
@@ -290,9 +290,9 @@ int flex_awd_loss_bwd(const flex_shape* shape, const void* q, const void* k, con
     float* kw = tau ? (float*)(base + w.kw) : nullptr;
     if (tau && (rc = count(1, flex::launch_key_weights(p, k, tau, kw, s)))) return rc;
     int* status = &((flex::WsHeader*)ws)->status;
-    if ((rc = count(1, flex::launch_tc_featmap(p, q, W1, W2, nullptr, base + w.pq, status, s))))
+    if ((rc = count(1, flex::launch_tc_featmap(p, q, W1, W2, nullptr, base + w.pq, status, tau != nullptr, s))))
         return rc;
-    if ((rc = count(1, flex::launch_tc_featmap(p, k, W1, W2, kw, base + w.pk, status, s))))
+    if ((rc = count(1, flex::launch_tc_featmap(p, k, W1, W2, kw, base + w.pk, status, true, s))))
         return rc;
     return count(loss ? 4 : 3,
                  flex::launch_tc_awd_bwd(p, q, k, base + w.pq, base + w.pk, W1, W2, kw, tau, dloss,

@@ -98,8 +98,10 @@ cudaError_t launch_tc_bwd(const Problem& p, const void* q, const void* k, const 
 
 // ---- feature map on the tensor cores (bf16, d = 64, M in {64, 128}) ------------------
 bool tc_featmap_supported(const Problem& p);
+// (after: may start before the kernel ahead of it in the stream has finished)
 cudaError_t launch_tc_featmap(const Problem& p, const void* x, const float* W1, const float* W2,
-                              const float* rowscale, void* phi, int* status, cudaStream_t s);
+                              const float* rowscale, void* phi, int* status, bool after,
+                              cudaStream_t s);
 
 // ---- attention-weight distillation loss (tensor cores: bf16, d = 64, M in {64, 128}) ---
 bool tc_awd_supported(const Problem& p);

@@ -1103,6 +1103,7 @@ __global__ void __launch_bounds__(kThreads) key_weights_bf16_d64_kernel(Problem 
                                                                          const float* tau,
                                                                          float* kw)
 {
+    tc::grid_dep_launch();
     constexpr int kUnroll = 4;
     const size_t rows = (size_t)p.B * p.H * p.N;
     const int lane = threadIdx.x & 31, sub = lane & 7;
@@ -1139,6 +1140,7 @@ __global__ void __launch_bounds__(kThreads) key_weights_bf16_d64_kernel(Problem 
 __global__ void dw_reduce_kernel(Problem p, const float* part, float* dW1, float* dW2,
                                  const float* dtau_part, float* dtau)
 {
+    tc::grid_dep_wait();
     const int d = p.d, M = p.M, Mc = p.nonstat ? 2 * M : M;
     const size_t per = (size_t)M * d;
     if (dtau && blockIdx.x == 0)  // dtau[h] = sum over the batch, in order
@@ -1412,8 +1414,8 @@ cudaError_t launch_simt_bwd(const Problem& p, const void* q, const void* k, cons
     if (e != cudaSuccess) return e;
     const size_t work = (size_t)p.H * p.M * p.d;
     const int blocks = (int)std::min<size_t>((work + kThreads - 1) / kThreads, 152 * 8);
-    dw_reduce_kernel<<<blocks, kThreads, 0, s>>>(p, part, dW1, dW2, tpart, tau ? dtau : nullptr);
-    return cudaGetLastError();
+    return tc::launch_after(dw_reduce_kernel, dim3((unsigned)blocks), kThreads, 0, 0, true, s, p, (const float*)part,
+                            dW1, dW2, (const float*)tpart, tau ? dtau : (float*)nullptr);
 }
 
 }  // namespace flex

@@ -73,8 +73,8 @@ __global__ void __launch_bounds__(kThreadsA, 1)
                   const __grid_constant__ CUtensorMap tmap_k,
                   const __grid_constant__ CUtensorMap tmap_pq,
                   const __grid_constant__ CUtensorMap tmap_pk, int N, int causal,
-                  float score_scale, int nqb, float* __restrict__ part,
-                  float4* __restrict__ rowstat, int* status)
+                  float score_scale, int nqb, float* part,
+                  float4* rowstat, int* status)
 {
     using L = AwdCfg<G2>;
     extern __shared__ uint8_t smem_raw[];
@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(kThreadsA, 1)
         tmem_alloc(&tmem_base_sh, 256);
         tmem_relinquish();
     }
+    grid_dep_launch();
+    grid_dep_wait();  // the feature maps
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -271,9 +273,11 @@ __global__ void __launch_bounds__(kThreadsA, 1)
     if (warp == 0) tmem_dealloc(tm, 256);
 }
 
-__global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* __restrict__ part,
+__global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* part,
                                   float* __restrict__ loss)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < BH; u += gridDim.x * blockDim.x) {
         float s = 0.f;
         for (int b = 0; b < nqb; ++b) s += part[(size_t)u * nqb + b];  // fixed order
@@ -343,10 +347,10 @@ __global__ void __launch_bounds__(kThreadsG, 1)
                       const __grid_constant__ CUtensorMap tmap_pq,
                       const __grid_constant__ CUtensorMap tmap_pk, int BH, int H, int N, int M,
                       int causal, int hsplit, float score_scale,
-                      const float4* __restrict__ rowstat, const float* __restrict__ dloss,
+                      const float4* rowstat, const float* __restrict__ dloss,
                       const float* __restrict__ W1, const float* __restrict__ W2,
-                      const float* __restrict__ kw, const float* __restrict__ tau,
-                      float* __restrict__ slots, float* __restrict__ dtau_part, int* status)
+                      const float* kw, const float* __restrict__ tau,
+                      float* slots, float* dtau_part, int* status)
 {
     using L = AwdBwCfg<G2>;
     constexpr int P = NS ? 128 : 64;  // projection rows per group of 64 frequencies
@@ -403,6 +407,8 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     }
     // this head's W' rows, all groups, once
     if (warp < kComputeG) stage_freq_rows<NS, G, 32 * kComputeG>(sb + L::WG, W1, W2, h, M, tid);
+    grid_dep_launch();
+    grid_dep_wait();  // the feature maps, the rows' statistics
     fence_proxy_async();
     fence_before_sync();
     __syncthreads();
@@ -748,10 +754,11 @@ done:
 constexpr int kReduceThreads = 512;
 __global__ void __launch_bounds__(kReduceThreads)
     awd_dw_reduce_kernel(int B, int H, int M, int nonstat, int hsplit,
-                         const float* __restrict__ slots, const float* __restrict__ dtau_part,
+                         const float* slots, const float* dtau_part,
                          float* __restrict__ dW1, float* __restrict__ dW2,
                          float* __restrict__ dtau)
 {
+    grid_dep_wait();
     __shared__ float4 sums[3][128];
     const int BH = B * H, G = M / 64, per_side = B * hsplit, nslot = 2 * per_side;
     const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
@@ -815,12 +822,11 @@ cudaError_t launch_typed(const Problem& p, const void* q, const void* k, const v
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const float score_scale = 1.4426950408889634f / sqrtf((float)p.d);  // log2(e) / sqrt(d)
-    kern<<<BH * nqb, kThreadsA, smem, s>>>(mq, mk, mpq, mpk, p.N, p.causal, score_scale, nqb,
-                                           part, rowstat, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (!loss) return cudaSuccess;
-    awd_reduce_kernel<<<(BH + 255) / 256, 256, 0, s>>>(BH, nqb, p.N, part, loss);
-    return cudaGetLastError();
+    e = launch_after(kern, dim3((unsigned)(BH * nqb)), kThreadsA, smem, 0, true, s, mq, mk, mpq, mpk, p.N,
+                     p.causal, score_scale, nqb, part, rowstat, status);
+    if (e != cudaSuccess || !loss) return e;
+    return launch_after(awd_reduce_kernel, dim3((BH + 255) / 256), 256, 0, 0, true, s, BH, nqb, p.N,
+                        (const float*)part, loss);
 }
 
 // CTAs per (side, sequence) of the gradient kernel: held blocks are split until the grid
@@ -852,13 +858,13 @@ cudaError_t launch_bwd_typed(const Problem& p, const void* q, const void* k, con
     if (e != cudaSuccess) return e;
     const float score_scale = 1.4426950408889634f / sqrtf((float)p.d);
     const int hs = awd_hsplit(p);
-    kern<<<2 * BH * hs, kThreadsG, smem, s>>>(mq, mk, mpq, mpk, BH, p.H, p.N, p.M, p.causal, hs,
-                                              score_scale, rowstat, dloss, W1, W2, kw, tau, slots,
-                                              dtau_part, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    awd_dw_reduce_kernel<<<p.H * (p.M / 64) * 16, kReduceThreads, 0, s>>>(
-        p.B, p.H, p.M, p.nonstat, hs, slots, dtau_part, dW1, dW2, tau ? dtau : nullptr);
-    return cudaGetLastError();
+    e = launch_after(kern, dim3((unsigned)(2 * BH * hs)), kThreadsG, smem, 0, true, s, mq, mk, mpq, mpk, BH,
+                     p.H, p.N, p.M, p.causal, hs, score_scale, rowstat, dloss, W1, W2, kw, tau, slots,
+                     dtau_part, status);
+    if (e != cudaSuccess) return e;
+    return launch_after(awd_dw_reduce_kernel, dim3((unsigned)(p.H * (p.M / 64) * 16)), kReduceThreads, 0, 0,
+                        true, s, p.B, p.H, p.M, p.nonstat, hs, (const float*)slots,
+                        (const float*)dtau_part, dW1, dW2, tau ? dtau : (float*)nullptr);
 }
 
 template <int G2>

@@ -126,9 +126,9 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     const float* __restrict__ W1, const float* __restrict__ W2,
     const __nv_bfloat16* __restrict__ outp, const float* __restrict__ den,
     const __nv_bfloat16* __restrict__ dout, __nv_bfloat16* __restrict__ dq,
-    __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv, float* __restrict__ dw_part,
-    const float* __restrict__ kw, const float* __restrict__ tau, float* __restrict__ dtau_part,
-    int units, int nsplit, float* __restrict__ state_part, const float* __restrict__ state_total,
+    __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv, float* dw_part,
+    const float* kw, const float* __restrict__ tau, float* dtau_part,
+    int units, int nsplit, float* state_part, const float* state_total,
     int* status)
 {
     using L = BwCfg<NS>;
@@ -165,15 +165,10 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     float* crow = reinterpret_cast<float*>(sm + L::CROW);
     float* spart = reinterpret_cast<float*>(sm + L::SPART);
     const float itau = KW ? expf(-tau[h]) : 0.f;
-    // dtau = -sum_j ln(w_j) s_j with s_j = phi~(k_j) . dphi~(k_j) = dL / d ln(w_j).  Scaling
-    // every key weight of a sequence by one factor leaves every output row unchanged, so the
-    // s_j of a sequence sum to zero and any per-sequence constant may be subtracted from
-    // ln(w_j); the log weight of the sequence's first key removes the common part, whose
-    // terms would otherwise cancel only to the rounding of the s_j.
-    const float lw0 = KW ? logf(kw[(size_t)bh * N]) : 0.f;
     float dtau_acc = 0.f;
 
     // ---- set-up: this group's projection rows, zero state, C16 ----
+    grid_dep_launch();
     for (int idx = tid; idx < L::P * 8; idx += kThreadsB) {
         const int r = idx >> 3, c = idx & 7, f = 64 * g + (r & 63);
         const float* w1 = W1 + ((size_t)h * M + f) * 64 + c * 8;
@@ -219,6 +214,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         tmem_alloc(&tmem_base_sh, 512);
         tmem_relinquish();
     }
+    grid_dep_wait();  // the key weights, partial states or totals (set-up needs none of them)
     fence_proxy_async();
     fence_before_sync();
     if (CS > 1)
@@ -228,6 +224,12 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     fence_after_sync();
     const uint32_t tm = tmem_base_sh;
     const uint32_t tm_row = tm + ((uint32_t)(32 * quad) << 16);
+    // dtau = -sum_j ln(w_j) s_j with s_j = phi~(k_j) . dphi~(k_j) = dL / d ln(w_j).  Scaling
+    // every key weight of a sequence by one factor leaves every output row unchanged, so the
+    // s_j of a sequence sum to zero and any per-sequence constant may be subtracted from
+    // ln(w_j); the log weight of the sequence's first key removes the common part, whose
+    // terms would otherwise cancel only to the rounding of the s_j.
+    const float lw0 = KW ? logf(kw[(size_t)bh * N]) : 0.f;
     uint32_t ph_xfull[2] = {0, 0};
     const uint32_t partner = (uint32_t)rank ^ 1u;
 
@@ -1254,10 +1256,10 @@ __global__ void __launch_bounds__(kThreadsB, 1)
                   const __nv_bfloat16* __restrict__ outp, const float* __restrict__ den,
                   const __nv_bfloat16* __restrict__ dout, __nv_bfloat16* __restrict__ dq,
                   __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                  float* __restrict__ dw_part,
-                  const float* __restrict__ kw, const float* __restrict__ tau,
-                  float* __restrict__ dtau_part, int units, int nsplit,
-                  float* __restrict__ state_part, const float* __restrict__ state_total,
+                  float* dw_part,
+                  const float* kw, const float* __restrict__ tau,
+                  float* dtau_part, int units, int nsplit,
+                  float* state_part, const float* state_total,
                   int* status)
 {
     if ((int)blockIdx.x < units * nsplit)
@@ -1283,11 +1285,12 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 constexpr int kReduceThreads = 512;
 __global__ void __launch_bounds__(kReduceThreads)
     tc_dw_reduce_kernel(int B, int H, int M, int G, int nsplit, int nonstat,
-                        const float* __restrict__ part, float* __restrict__ dW1,
-                        float* __restrict__ dW2, const float* __restrict__ dtau_part,
+                        const float* part, float* __restrict__ dW1,
+                        float* __restrict__ dW2, const float* dtau_part,
                         float* __restrict__ dtau)
 {
     __shared__ float4 sums[3][128];
+    grid_dep_wait();
     const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
     const int row = threadIdx.x % 128, ln = threadIdx.x / 128;
     const int per = B * nsplit;                        // slots of (head, group) and pass
@@ -1355,10 +1358,12 @@ __device__ __forceinline__ void add4(float4& a, const float4& x)
 
 // Non-causal totals: total[pass][unit][row][0..64] = sum over the splits, in order.
 __global__ void __launch_bounds__(kStateThreads)
-    nc_state_reduce_kernel(int units, int G, int nsplit, float* __restrict__ part,
-                           float* __restrict__ total)
+    nc_state_reduce_kernel(int units, int G, int nsplit, float* part,
+                           float* total)
 {
     const int u = blockIdx.x % units, pass = blockIdx.x / units, bh = u / G, g = u % G;
+    grid_dep_launch();
+    grid_dep_wait();
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int sp = 0; sp < nsplit; ++sp)
@@ -1369,9 +1374,11 @@ __global__ void __launch_bounds__(kStateThreads)
 // Causal ranges: each range's partial state becomes, in place, what the range starts from:
 // pass F the sum over the earlier ranges, pass R over the later ones, in order.
 __global__ void __launch_bounds__(kStateThreads)
-    causal_state_scan_kernel(int units, int G, int nsplit, float* __restrict__ part)
+    causal_state_scan_kernel(int units, int G, int nsplit, float* part)
 {
     const int u = blockIdx.x % units, pass = blockIdx.x / units, bh = u / G, g = u % G;
+    grid_dep_launch();
+    grid_dep_wait();
     auto at = [&](int o) {
         const int sp = pass == kPassF ? o : nsplit - 1 - o;
         return state_at(part, (size_t)pass * units * nsplit + ((size_t)bh * nsplit + sp) * G + g);
@@ -1471,23 +1478,13 @@ cudaError_t launch_mode(const Problem& p, const BwdArgs& m, const void* q, const
     typedef const __nv_bfloat16* CB;
     typedef __nv_bfloat16* B16;
     const int units = p.B * p.H * (p.M / 64);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * units * nsplit));
-    cfg.blockDim = dim3(kThreadsB);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CS;  // the frequency groups of one (pass, sequence, split)
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kb, m.mq, m.mk, m.mv, m.mdo, m.mo, p.H, p.N, p.M, p.M / 64,
-                              p.causal, (CB)q, (CB)k, (CB)v, W1, W2, (CB)out, den, (CB)dout,
-                              (B16)dq, (B16)dk, (B16)dv, f + w.part, KW ? f + w.kw : nullptr, tau,
-                              f + w.dtau, units, nsplit, f + w.state_part,
-                              (const float*)(f + w.state_total), status);
+    // (the first kernel of a call, without key weights, starts in stream order)
+    const bool after = KW || MODE == kGrad || (MODE == kCausal && nsplit > 1);
+    return launch_after(kb, dim3((unsigned)(2 * units * nsplit)), kThreadsB, smem, CS, after, s, m.mq, m.mk,
+                        m.mv, m.mdo, m.mo, p.H, p.N, p.M, p.M / 64, p.causal, (CB)q, (CB)k, (CB)v, W1,
+                        W2, (CB)out, den, (CB)dout, (B16)dq, (B16)dk, (B16)dv, f + w.part,
+                        KW ? (const float*)(f + w.kw) : (const float*)nullptr, tau, f + w.dtau, units,
+                        nsplit, f + w.state_part, (const float*)(f + w.state_total), status);
 }
 
 template <bool NS, bool KW>
@@ -1513,12 +1510,11 @@ cudaError_t launch_bwd(const Problem& p, const void* q, const void* k, const voi
                                            f, w, nsplit, status, s);
         if (e != cudaSuccess) return e;
         const dim3 sgrid(2 * units, 128 * 17 / kStateThreads);
-        if (p.causal)
-            causal_state_scan_kernel<<<sgrid, kStateThreads, 0, s>>>(units, G, nsplit, f + w.state_part);
-        else
-            nc_state_reduce_kernel<<<sgrid, kStateThreads, 0, s>>>(units, G, nsplit, f + w.state_part,
-                                                                   f + w.state_total);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = p.causal ? launch_after(causal_state_scan_kernel, sgrid, kStateThreads, 0, 0, true, s, units,
+                                    G, nsplit, f + w.state_part)
+                     : launch_after(nc_state_reduce_kernel, sgrid, kStateThreads, 0, 0, true, s, units, G,
+                                    nsplit, f + w.state_part, f + w.state_total);
+        if (e != cudaSuccess) return e;
     }
     if (p.causal)
         e = G == 2 ? launch_mode<NS, KW, 2, kCausal>(p, m, q, k, v, W1, W2, tau, out, den, dout, dq,
@@ -1531,10 +1527,9 @@ cudaError_t launch_bwd(const Problem& p, const void* q, const void* k, const voi
                    : launch_mode<NS, KW, 1, kGrad>(p, m, q, k, v, W1, W2, tau, out, den, dout, dq,
                                                    dk, dv, f, w, nsplit, status, s);
     if (e != cudaSuccess) return e;
-    tc_dw_reduce_kernel<<<p.H * G * 16, kReduceThreads, 0, s>>>(p.B, p.H, p.M, G, nsplit, p.nonstat,
-                                                                f + w.part, dW1, dW2, f + w.dtau,
-                                                                KW ? dtau : nullptr);
-    return cudaGetLastError();
+    return launch_after(tc_dw_reduce_kernel, dim3((unsigned)(p.H * G * 16)), kReduceThreads, 0, 0, true, s,
+                        p.B, p.H, p.M, G, nsplit, p.nonstat, (const float*)(f + w.part), dW1, dW2,
+                        (const float*)(f + w.dtau), KW ? dtau : (float*)nullptr);
 }
 
 }  // namespace

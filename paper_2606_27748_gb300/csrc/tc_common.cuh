@@ -498,7 +498,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 // ---- programmatic dependent launch --------------------------------------------------------
 // In a kernel launched with the stream-serialization attribute: wait for the preceding grid to
 // finish (its results are visible afterwards); anywhere: let the following such grid's CTAs
-// start once every CTA of this grid has started.
+// start once every CTA of this grid has started.  What the preceding grid wrote is read through
+// plain pointers: `const __restrict__` would let the compiler load it before the wait.
 __device__ __forceinline__ void grid_dep_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

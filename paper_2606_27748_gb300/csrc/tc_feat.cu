@@ -31,7 +31,7 @@ template <bool NS, int G>  // G = M / 64 frequency groups
 __global__ void __launch_bounds__(kThreadsF)
     tc_featmap_kernel(const __grid_constant__ CUtensorMap tmap_x, int H, int N, int M,
                       const float* __restrict__ W1, const float* __restrict__ W2,
-                      const float* __restrict__ rowscale, float scale,
+                      const float* rowscale, float scale,
                       __nv_bfloat16* __restrict__ phi, int* status)
 {
     constexpr int P = NS ? 128 : 64;        // projection rows (= tensor memory columns) per group
@@ -51,6 +51,8 @@ __global__ void __launch_bounds__(kThreadsF)
     const int bh = blockIdx.x / nchunk, b0 = (blockIdx.x % nchunk) * kBlocksPerCta, h = bh % H;
     const int nb = min(kBlocksPerCta, nblk - b0);
 
+    grid_dep_launch();
+    if (rowscale) grid_dep_wait();  // written by the kernel before (nothing else here is)
     stage_freq_rows_split<NS, G, kThreadsF>(sb + W, sb + WLO, W1, W2, h, M, tid);  // once
     if (tid == 0) {
         mbar_init(&mbar, 1);
@@ -156,11 +158,12 @@ __global__ void __launch_bounds__(kThreadsF)
     __syncthreads();
     fence_after_sync();
     if (warp == 0) tmem_dealloc(tm, NCOLS);
+    if (!rowscale) grid_dep_wait();  // so that a kernel that waits for this one has both
 }
 
 template <bool NS, int G>
 cudaError_t launch_typed(const Problem& p, const void* x, const float* W1, const float* W2,
-                         const float* rowscale, void* phi, int* status, cudaStream_t s)
+                         const float* rowscale, void* phi, int* status, bool after, cudaStream_t s)
 {
     CUtensorMap mx;
     const int BH = p.B * p.H;
@@ -173,10 +176,8 @@ cudaError_t launch_typed(const Problem& p, const void* x, const float* W1, const
     const int nblk = (p.N + kC - 1) / kC;
     const long long blocks = (long long)BH * ((nblk + kBlocksPerCta - 1) / kBlocksPerCta);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    kern<<<(unsigned)blocks, kThreadsF, smem, s>>>(mx, p.H, p.N, p.M, W1, W2, rowscale,
-                                                   1.0f / sqrtf((float)p.M),
-                                                   (__nv_bfloat16*)phi, status);
-    return cudaGetLastError();
+    return launch_after(kern, dim3((unsigned)blocks), kThreadsF, smem, 0, after, s, mx, p.H, p.N, p.M, W1,
+                        W2, rowscale, 1.0f / sqrtf((float)p.M), (__nv_bfloat16*)phi, status);
 }
 
 }  // namespace
@@ -187,13 +188,14 @@ bool tc_featmap_supported(const Problem& p)
 }
 
 cudaError_t launch_tc_featmap(const Problem& p, const void* x, const float* W1, const float* W2,
-                              const float* rowscale, void* phi, int* status, cudaStream_t s)
+                              const float* rowscale, void* phi, int* status, bool after,
+                              cudaStream_t s)
 {
     if (p.nonstat)
-        return p.M == 64 ? launch_typed<true, 1>(p, x, W1, W2, rowscale, phi, status, s)
-                         : launch_typed<true, 2>(p, x, W1, W2, rowscale, phi, status, s);
-    return p.M == 64 ? launch_typed<false, 1>(p, x, W1, W2, rowscale, phi, status, s)
-                     : launch_typed<false, 2>(p, x, W1, W2, rowscale, phi, status, s);
+        return p.M == 64 ? launch_typed<true, 1>(p, x, W1, W2, rowscale, phi, status, after, s)
+                         : launch_typed<true, 2>(p, x, W1, W2, rowscale, phi, status, after, s);
+    return p.M == 64 ? launch_typed<false, 1>(p, x, W1, W2, rowscale, phi, status, after, s)
+                     : launch_typed<false, 2>(p, x, W1, W2, rowscale, phi, status, after, s);
 }
 
 }  // namespace flex

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                          const __grid_constant__ CUtensorMap tmap_v,
                          const __grid_constant__ CUtensorMap tmap_o, int H, int N, int M,
                          int splits, const float* __restrict__ W1,
-                         const float* __restrict__ W2, const float* __restrict__ kw,
+                         const float* __restrict__ W2, const float* kw,
                          __nv_bfloat16* __restrict__ out, float* __restrict__ den, int* status)
 {
     using L = Cfg<NS, CS>;
@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
         tmem_alloc(&tmem_base_sh, 512);
         tmem_relinquish();
     }
+    if (KW) grid_dep_wait();  // the key weights
     fence_proxy_async();
     fence_before_sync();
     if (CS > 1)
@@ -737,20 +738,10 @@ cudaError_t launch_one(const Problem& p, const void* q, const void* k, const voi
     const int smem = (int)Cfg<NS, CS>::BYTES + 1024;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(BH * splits * CS));
-    cfg.blockDim = dim3(Cfg<NS, CS>::THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, mq, mk, mv, mo, p.H, p.N, p.M, splits, W1, W2, kw,
-                              (__nv_bfloat16*)out, den, status);
+    // (with key weights: after the kernel that writes them)
+    return launch_after(kern, dim3((unsigned)(BH * splits * CS)), Cfg<NS, CS>::THREADS, smem, CS, KW, s,
+                        mq, mk, mv, mo, p.H, p.N, p.M, splits, W1, W2, kw, (__nv_bfloat16*)out, den,
+                        status);
 }
 
 }  // namespace

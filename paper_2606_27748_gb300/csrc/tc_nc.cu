@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
     tc_nc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                  const __grid_constant__ CUtensorMap tmap_v, int H, int N, int M, int splits,
                  const float* __restrict__ W1, const float* __restrict__ W2,
-                 const float* __restrict__ kw, float* __restrict__ part,
-                 const uint8_t* __restrict__ total, __nv_bfloat16* __restrict__ out,
+                 const float* kw, float* part,
+                 const uint8_t* total, __nv_bfloat16* __restrict__ out,
                  float* __restrict__ den, int* status)
 {
     using L = NcCfg<NS, G>;
@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
         tmem_alloc(&tmem_base_sh, 512);
         tmem_relinquish();
     }
+    if (MODE == kState && KW) grid_dep_wait();  // the key weights
     fence_proxy_async();
     fence_before_sync();
     __syncthreads();
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
 // feature), the splits' loads independent.
 constexpr int kReduceThreads = 544;  // half of the 17 x 64 float4 of a block
 __global__ void __launch_bounds__(kReduceThreads)
-    nc_reduce_kernel(int splits, int G, const float* __restrict__ part, uint8_t* __restrict__ total)
+    nc_reduce_kernel(int splits, int G, const float* part, uint8_t* total)
 {
     __shared__ __align__(16) uint8_t image[kSxBlock];
     const int fb = blockIdx.x & 1, g = (blockIdx.x >> 1) % G, bh = (blockIdx.x >> 1) / G;
@@ -426,24 +427,6 @@ __global__ void __launch_bounds__(kReduceThreads)
         dst[i] = reinterpret_cast<const uint4*>(image)[i];
 }
 
-// Launch that may overlap the preceding kernel's end (which the kernel waits for itself).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_after(void (*kern)(KArgs...), unsigned blocks, int threads, int smem,
-                         cudaStream_t s, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 template <bool NS, int G>
 cudaError_t launch_nc(const Problem& p, const void* q, const void* k, const void* v,
                       const float* W1, const float* W2, const float* kw, void* out, float* den,
@@ -463,14 +446,16 @@ cudaError_t launch_nc(const Problem& p, const void* q, const void* k, const void
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_out, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_state<<<BH * splits, kThreadsNC, smem, s>>>(mk, mv, p.H, p.N, p.M, splits, W1, W2, kw,
-                                                 part, nullptr, nullptr, nullptr, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    e = launch_after(nc_reduce_kernel, 2u * BH * G, kReduceThreads, 0, s, splits, G,
+    // (with key weights: after the kernel that writes them)
+    e = launch_after(k_state, dim3((unsigned)(BH * splits)), kThreadsNC, smem, 0, kw != nullptr, s, mk,
+                     mv, p.H, p.N, p.M, splits, W1, W2, kw, part, (const uint8_t*)nullptr,
+                     (__nv_bfloat16*)nullptr, (float*)nullptr, status);
+    if (e != cudaSuccess) return e;
+    e = launch_after(nc_reduce_kernel, dim3(2u * BH * G), kReduceThreads, 0, 0, true, s, splits, G,
                      (const float*)part, total);
     if (e != cudaSuccess) return e;
-    return launch_after(k_out, (unsigned)(BH * splits), kThreadsNC, smem, s, mq, mo, p.H, p.N, p.M,
-                        splits, W1, W2, (const float*)nullptr, (float*)nullptr,
+    return launch_after(k_out, dim3((unsigned)(BH * splits)), kThreadsNC, smem, 0, true, s, mq, mo, p.H,
+                        p.N, p.M, splits, W1, W2, (const float*)nullptr, (float*)nullptr,
                         (const uint8_t*)total, (__nv_bfloat16*)out, den, status);
 }
 
