@@ -474,13 +474,11 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
         return piece + 64u * lane + (((uint32_t)j ^ ((uint32_t)(lane >> 1) & 3u)) << 4);
     };
     auto store_quarter = [&](__nv_bfloat16* out, int t0, const float (&v_)[16]) {
-        uint4* dst = reinterpret_cast<uint4*>(out + base + (size_t)(t0 + t) * 64 + 16 * wg);
-#pragma unroll
-        for (int cc = 0; cc < 2; ++cc)
-            dst[cc] = make_uint4(pack_bf16(v_[8 * cc], v_[8 * cc + 1]),
-                                 pack_bf16(v_[8 * cc + 2], v_[8 * cc + 3]),
-                                 pack_bf16(v_[8 * cc + 4], v_[8 * cc + 5]),
-                                 pack_bf16(v_[8 * cc + 6], v_[8 * cc + 7]));
+        store_32b(out + base + (size_t)(t0 + t) * 64 + 16 * wg,
+                  make_uint4(pack_bf16(v_[0], v_[1]), pack_bf16(v_[2], v_[3]), pack_bf16(v_[4], v_[5]),
+                             pack_bf16(v_[6], v_[7])),
+                  make_uint4(pack_bf16(v_[8], v_[9]), pack_bf16(v_[10], v_[11]),
+                             pack_bf16(v_[12], v_[13]), pack_bf16(v_[14], v_[15])));
     };
     // Rows of the [128 x 64] block at tensor-memory column `col` -> bf16 rows of `out` for the
     // chunk at t0.  kcoef != 0 adds kcoef * k_t (the prefactor's dk term; k from the tile at

@@ -495,6 +495,23 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
         : "memory");
 }
 
+// 32 bytes of a row of global memory, p 16-byte aligned: one store where p allows it.  (One row
+// per thread: two 16-byte stores write every 32-byte sector in two halves, and the queue those
+// stores fill also carries the mbarrier polls and the feature warps' shared stores.  With it:
+// forward n causal B4 H16 N16384 M128 390 -> 370 us, training step s causal B8 H12 N8192 M128
+// 1773 -> 1748 us, n non-causal B32 H8 N4000 M64 950 -> 918 us.)
+__device__ __forceinline__ void store_32b(void* p, const uint4& a, const uint4& b)
+{
+    if ((reinterpret_cast<uintptr_t>(p) & 31) == 0) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x),
+                     "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                     : "memory");
+    } else {
+        static_cast<uint4*>(p)[0] = a;
+        static_cast<uint4*>(p)[1] = b;
+    }
+}
+
 // ---- programmatic dependent launch --------------------------------------------------------
 // In a kernel launched with the stream-serialization attribute: wait for the preceding grid to
 // finish (its results are visible afterwards); anywhere: let the following such grid's CTAs

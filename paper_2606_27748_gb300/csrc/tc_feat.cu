@@ -142,12 +142,13 @@ __global__ void __launch_bounds__(kThreadsF)
                 ps[i] = pack_bf16(s0 * k0, s1 * k1);
             }
             if (valid) {  // frequencies 64 g + 32 wg .. + 31: 64 contiguous bytes each
-                uint4* dc = reinterpret_cast<uint4*>(out + 64 * g + 32 * wg);
-                uint4* ds = reinterpret_cast<uint4*>(out + M + 64 * g + 32 * wg);
+                __nv_bfloat16 *dc = out + 64 * g + 32 * wg, *ds = dc + M;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    dc[j] = make_uint4(pc[4 * j], pc[4 * j + 1], pc[4 * j + 2], pc[4 * j + 3]);
-                    ds[j] = make_uint4(ps[4 * j], ps[4 * j + 1], ps[4 * j + 2], ps[4 * j + 3]);
+                for (int j = 0; j < 2; ++j) {
+                    store_32b(dc + 16 * j, make_uint4(pc[8 * j], pc[8 * j + 1], pc[8 * j + 2], pc[8 * j + 3]),
+                              make_uint4(pc[8 * j + 4], pc[8 * j + 5], pc[8 * j + 6], pc[8 * j + 7]));
+                    store_32b(ds + 16 * j, make_uint4(ps[8 * j], ps[8 * j + 1], ps[8 * j + 2], ps[8 * j + 3]),
+                              make_uint4(ps[8 * j + 4], ps[8 * j + 5], ps[8 * j + 6], ps[8 * j + 7]));
                 }
             }
         }

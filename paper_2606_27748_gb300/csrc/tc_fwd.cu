@@ -699,14 +699,15 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                     __syncwarp();
                 } else if (valid) {
                     const float inv = 1.f / dn;
-                    uint4* dst =
-                        reinterpret_cast<uint4*>(out + base + (size_t)(t0 + t) * 64 + 32 * eh);
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc)
-                        dst[cc] = make_uint4(pack_bf16(o[8 * cc] * inv, o[8 * cc + 1] * inv),
-                                             pack_bf16(o[8 * cc + 2] * inv, o[8 * cc + 3] * inv),
-                                             pack_bf16(o[8 * cc + 4] * inv, o[8 * cc + 5] * inv),
-                                             pack_bf16(o[8 * cc + 6] * inv, o[8 * cc + 7] * inv));
+                    __nv_bfloat16* dst = out + base + (size_t)(t0 + t) * 64 + 32 * eh;
+                    auto quad16 = [&](int e) {  // 8 values
+                        return make_uint4(pack_bf16(o[e] * inv, o[e + 1] * inv),
+                                          pack_bf16(o[e + 2] * inv, o[e + 3] * inv),
+                                          pack_bf16(o[e + 4] * inv, o[e + 5] * inv),
+                                          pack_bf16(o[e + 6] * inv, o[e + 7] * inv));
+                    };
+                    store_32b(dst, quad16(0), quad16(8));
+                    store_32b(dst + 16, quad16(16), quad16(24));
                     if (den && eh == 0) den[(size_t)bh * N + t0 + t] = dn / (float)M;
                 }
             }
