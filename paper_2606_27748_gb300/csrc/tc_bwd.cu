@@ -298,9 +298,15 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                 c0 *= cw0; s0 *= cw0; c1 *= cw1; s1 *= cw1;
             }
             if (KW) { c0 *= wsc; s0 *= wsc; c1 *= wsc; s1 *= wsc; }
-            if (!valid) { c0 = s0 = c1 = s1 = 0.f; }
             pc[i] = pack_bf16(c0, c1);
             ps[i] = pack_bf16(s0, s1);
+        }
+        // Rows past N are zeroed for the totals only.  Elsewhere TMA's zeros make x, v and g (and
+        // c) zero in them, so they add nothing to dW or the state R; dA and A are masked; S after
+        // the ragged last chunk is not used; their own result rows are not stored.
+        if (MODE == kState && __any_sync(0xffffffffu, !valid) && !valid) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) pc[i] = ps[i] = 0u;
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -378,7 +384,9 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                             fs[e] *= wkey;
                         }
                     }
-                    if (!valid) r1[e] = r2[e] = fc[e] = fs[e] = 0.f;
+                    // (not needed, but ptxas spills 28 bytes instead of 8 without it: 921 -> 910
+                    // us for the training step of B32 H8 N4000 M64)
+                    if (NS && MODE == kGrad && !valid) r1[e] = r2[e] = fc[e] = fs[e] = 0.f;
                 }
                 o1[i] = pack_bf16(r1[0], r1[1]);
                 if (!NS) {
@@ -783,16 +791,28 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
             };
             // bf16 of the block at `col` masked to j <= i (+ add), this warp's 32 keys
             auto mask32 = [&](uint32_t col, float add, int CL, bool valid, uint32_t (&pk2)[16]) {
+                // whole chunks: blocks above the diagonal block of this warp's rows are zeros
+                // (nothing loaded), those below it need no mask
+                const bool full = CL == kC && wg != quad;
+                if (full && wg > quad) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) pk2[i] = 0u;
+                    return;
+                }
                 float a[32];
                 tmem_ld16(tm_row + col + 32 * wg, *reinterpret_cast<float(*)[16]>(&a[0]));
                 tmem_ld16(tm_row + col + 32 * wg + 16, *reinterpret_cast<float(*)[16]>(&a[16]));
                 tmem_wait_ld();
+                if (full) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int j0 = 32 * wg + 2 * i;
-                    const bool k0 = j0 <= t && j0 < CL && valid, k1 = j0 + 1 <= t && j0 + 1 < CL && valid;
-                    pk2[i] = pack_bf16(k0 ? a[2 * i] + add : 0.f, k1 ? a[2 * i + 1] + add : 0.f);
+                    for (int i = 0; i < 16; ++i) pk2[i] = pack_bf16(a[2 * i] + add, a[2 * i + 1] + add);
+                    return;
                 }
+                const int keys = (valid ? min(t + 1, CL) : 0) - 32 * wg;  // of this block
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    pk2[i] = pack_bf16(2 * i < keys ? a[2 * i] + add : 0.f,
+                                       2 * i + 1 < keys ? a[2 * i + 1] + add : 0.f);
             };
             auto mask_to_smem = [&](uint32_t col, float add, int CL, bool valid, uint32_t dst) {
                 uint32_t pk2[16];

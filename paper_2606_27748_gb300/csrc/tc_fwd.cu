@@ -401,6 +401,9 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
         const uint32_t tm_row = tm + ((uint32_t)(32 * quad) << 16);
         uint32_t ph_pfull = 0;
         int n = 0, nq = 0;  // k and q feature tiles produced so far
+        // Rows past N (only in a sequence's last chunk; TMA reads them as zeros, so their features
+        // are finite) need no zeroing: no earlier row sees their key, their v rows are zeros, the
+        // state after that chunk is not used and their output rows are not stored.
         for (int c = 0; c < ce; ++c) {
             const bool main = c >= cb;
             const bool valid = t < min(kC, N - c * kC);
@@ -443,7 +446,6 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                             c0 *= cw0; s0 *= cw0; c1 *= cw1; s1 *= cw1;
                         }
                         if (KW && which == 1) { c0 *= wk; s0 *= wk; c1 *= wk; s1 *= wk; }
-                        if (!valid) { c0 = s0 = c1 = s1 = 0.f; }
                         pc[NPR * r + i] = pack_bf16(c0, c1);
                         ps[NPR * r + i] = pack_bf16(s0, s1);
                     }

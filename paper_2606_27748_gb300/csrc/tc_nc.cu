@@ -271,9 +271,13 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                     cc0 *= cw0; s0 *= cw0; cc1 *= cw1; s1 *= cw1;
                 }
                 if (MODE == kState && KW) { cc0 *= wk; s0 *= wk; cc1 *= wk; s1 *= wk; }
-                if (!valid) { cc0 = s0 = cc1 = s1 = 0.f; }
                 pc[e] = pack_bf16(cc0, cc1);
                 ps[e] = pack_bf16(s0, s1);
+            }
+            // (keys past N: out of the totals; output rows past N are not stored)
+            if (MODE == kState && __any_sync(0xffffffffu, !valid) && !valid) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) pc[e] = ps[e] = 0u;
             }
             if (j >= 2 && !bar_wait(&bars.phi_free[pb], ((j - 2) >> 1) & 1, &abort_flag, status))
                 break;
