@@ -294,8 +294,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
             __sincosf(a[2 * i], &s0, &c0);
             __sincosf(a[2 * i + 1], &s1, &c1);
             if (NS) {
-                const float cw0 = w[2 * i], cw1 = w[2 * i + 1];
-                c0 *= cw0; s0 *= cw0; c1 *= cw1; s1 *= cw1;
+                mul2x2(c0, c1, s0, s1, w[2 * i], w[2 * i + 1]);
             }
             if (KW) { c0 *= wsc; s0 *= wsc; c1 *= wsc; s1 *= wsc; }
             pc[i] = pack_bf16(c0, c1);

@@ -442,8 +442,7 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
                         __sincosf(xl[e], &s0, &c0);
                         __sincosf(xl[e + 1], &s1, &c1);
                         if (NS) {
-                            const float cw0 = xl[8 + e], cw1 = xl[8 + e + 1];
-                            c0 *= cw0; s0 *= cw0; c1 *= cw1; s1 *= cw1;
+                            mul2x2(c0, c1, s0, s1, xl[8 + e], xl[8 + e + 1]);
                         }
                         if (KW && which == 1) { c0 *= wk; s0 *= wk; c1 *= wk; s1 *= wk; }
                         pc[NPR * r + i] = pack_bf16(c0, c1);

@@ -267,8 +267,7 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
                 __sincosf(a[2 * e], &s0, &cc0);
                 __sincosf(a[2 * e + 1], &s1, &cc1);
                 if (NS) {
-                    const float cw0 = w[2 * e], cw1 = w[2 * e + 1];
-                    cc0 *= cw0; s0 *= cw0; cc1 *= cw1; s1 *= cw1;
+                    mul2x2(cc0, cc1, s0, s1, w[2 * e], w[2 * e + 1]);
                 }
                 if (MODE == kState && KW) { cc0 *= wk; s0 *= wk; cc1 *= wk; s1 *= wk; }
                 pc[e] = pack_bf16(cc0, cc1);
