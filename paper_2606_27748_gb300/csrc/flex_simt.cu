@@ -113,7 +113,7 @@ __global__ void featmap_kernel(Problem p, const T* x, const float* W1, const flo
 // four k 8 float4 loads feed 64 fmas, so the fma pipe and not the shared-memory port is the
 // limit (one output per thread took two loads per fma), and a short sequence spreads over
 // up to 8 SMs instead of one.  Measured on GB300 against one CTA per sequence with
-// one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 23 us, bf16 n B32 H4
+// one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 16 us, bf16 n B32 H4
 // N1024 d32 M16 477 -> 73 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
 // 8.58 -> 0.33 ms (10 of the 78 TFLOP/s fp32 peak: per chunk the products run between
 // barriers with one backward CTA per SM, so load latency and the barriers bound it).

@@ -308,8 +308,8 @@ __global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* part,
 // groups' arithmetic (0.7 us each, overlapping); per CTA about a third of the time is set-up
 // and the chain rule.  Measured, one distillation step n B32 H8 N512 M64: 361 us with all
 // warps in step and thread 0 issuing, 307 us now (mask and side as compile-time cases 357 ->
-// 333, the held block as a tensor-memory operand -> 324, loads by their own warp -> 307).  The rows of
-// dW' are added into this CTA's slot; a reduction sums the slots over the sides, the batch
+// 333, the held block as a tensor-memory operand -> 324, loads by their own warp -> 307); 289 with
+// overlapped launches and the feature pass's 32-byte stores, 196 of them here.  The rows of dW' are added into this CTA's slot; a reduction sums the slots over the sides, the batch
 // and the splits in a fixed order, so the result does not depend on scheduling.  On the
 // key side, with the prefactor, the chain rule takes dphi(k_j) = w_j dphi~(k_j) and dtau
 // gains -(phi~(k_j) . dphi~(k_j)) |k_j|^2 exp(-tau).  Every wait is bounded.

@@ -29,9 +29,9 @@
 // adds 2 exp(-tau) s_j k_j to dk_j (folded into the same row adds) and -ln(w_j) s_j to
 // dtau (per-CTA slots, reduced with dW in a fixed order).
 //
-// Roles: warp 16 (one thread) loads the tiles by TMA and issues every MMA; warp 17 (one
-// thread) tells the partner CTA when its copies have landed; 16 compute warps (four per tensor-memory lane quadrant, each a quarter of the
-// columns) do the CUDA-core work and never meet at a CTA barrier: each hand-off is one
+// Roles: warp 16 (one elected lane per operation) loads the tiles by TMA and issues every MMA;
+// warp 17 tells the partner CTA when its copies have landed; 16 compute warps (four per
+// tensor-memory lane quadrant, each a quarter of the columns) do the CUDA-core work and never meet at a CTA barrier: each hand-off is one
 // arrival per warp on an mbarrier the issuer waits for, and the MMAs' completion, which
 // follows every warp's arrival, releases the compute warps again.  Work that does not depend
 // on a running MMA group (masks, row stores, the next chunk's g tile, the state snapshot)
@@ -45,10 +45,10 @@
 //   kGrad F    [q projection, dphi(q)] / chain rule, next chunk's g / [dq, dW] / dq rows
 //   kGrad R    [k projection, dphi(k)] / phi(k), chain rule / [dv, dk, dW] / dv, dk rows
 // The phases of a chunk depend on one another (an SM holds one CTA's tensor memory), so the
-// length of this chain bounds the kernel, not DRAM (7%) or the tensor pipe: per chunk of
-// s M128 about 6.9 us (F) and 10.4 us (R), from 8.2 and 11.2 with all threads meeting at CTA
-// barriers and thread 0 issuing; measured forward and backward: s B8 H12 N8192 M128 2.16 ->
-// 1.76 ms, n non-causal B32 H8 N4000 M64 1.30 -> 1.10 ms.
+// length of this chain bounds the kernel, not DRAM (7%) or the tensor pipe: a chunk of s M128
+// takes about 15 us in F and R together, from 19.4 with all threads meeting at CTA barriers
+// and thread 0 issuing; measured forward and backward: s B8 H12 N8192 M128 2.16 -> 1.58 ms,
+// n non-causal B32 H8 N4000 M64 1.30 -> 0.91 ms.
 // Every wait is bounded.  Tiles of the following chunks are loaded as soon as the region
 // each one occupies is free (two buffers where the pass leaves room).
 //
@@ -1297,7 +1297,7 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 // (from its low part); n: rows < 64 are dU, rows >= 64 are dV of frequency 64g + row%64.
 // One block per (head, group, column quad): thread (row, lane) sums every fourth slot with
 // eight loads in flight, the four lanes are then added in order.  It is bound by reading the
-// slots (32 KB each) at memory latency: B32 H8 in two ranges 29.5 -> XXX us against one thread
+// slots (32 KB each) at memory latency: B32 H8 in two ranges 29.5 -> 13.3 us against one thread
 // per output.
 constexpr int kReduceThreads = 512;
 __global__ void __launch_bounds__(kReduceThreads)
@@ -1421,7 +1421,7 @@ __global__ void __launch_bounds__(kStateThreads)
 // The count minimises rounds of CTAs on 152 SMs x (set-up + chunks), in causal chunk times
 // (about 8 us; the two extra launches cost about one); short sequences (under 8 chunks) gain
 // nothing.  Forward and backward of n with tau, B2 H8 N2000 M64 (32 CTAs uncut, 128 in four
-// ranges): 248 -> 160 us.
+// ranges): 248 -> 160 us (109 with the later steps).
 int causal_splits(const Problem& p)
 {
     const long long units = (long long)p.B * p.H * (p.M / 64);

@@ -8,7 +8,9 @@
 // thread 0 issues the projections x W^T (s: W1; n: U = (W1+W2)/2 and
 // V = (W1-W2)/2), one group of 64 frequencies per 64 (s) or 128 (n) columns; every thread
 // takes one row and 32 frequencies of each group: arguments reduced by 2 pi, hardware
-// sin/cos, products, bf16 pack, 64-byte stores of its cos and sin runs.
+// sin/cos, products, bf16 pack, 32-byte stores of its cos and sin runs.  Bound by latency (two
+// CTAs an SM, four blocks one after the other: 16.5 us for n B32 H8 N512 M64, whose 50 MB take
+// 7.4; 20 with 16-byte stores).
 //
 // The frequencies enter the projection split into bf16 high and low parts (two MMAs into
 // one fp32 accumulator): x is exactly bf16, so the projection carries the fp32

@@ -63,6 +63,11 @@
 //   [192,352)  two buffers of phi(Q) [S | z] + A [V | 1]: numerator 0-63, denominator 64
 //   [352,432)  [S | z] (lane = feature), z in column 64
 //   [432,496)  phi(Q) as bf16 pairs (column c = features 2c, 2c+1; cos in 0-31, sin 32-63)
+//
+// What bounds it: the chain of a chunk (features of q, phi(Q) freed, A, mask, A V) and the
+// feature warps' instruction issue; the sin/cos unit is busy a third of the time.  n B4 H16
+// N16384 M128 402 -> 351 us, s B8 H12 N4096 M64 86 -> 80 us: warp-wide MMA issue (402 -> 390),
+// 32-byte row stores (370), no zeroing of rows that nothing uses (353), packed products (351).
 #include <cuda.h>
 
 #include "flex_internal.h"

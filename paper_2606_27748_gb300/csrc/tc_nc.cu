@@ -24,6 +24,12 @@
 // shared memory and written by TMA stores).  Projection buffers (TMEM) and feature tiles
 // (shared memory) are double-buffered, so the feature warps compute job j+1 while the
 // tensor core consumes job j.
+//
+// What bounds it: the feature warps' instruction issue beside memory (n M64: 3 sin/cos, of
+// which one on the fma pipe, per 8 bytes read or written).  n B8 H8 N65536 M64: 511 -> 449 us
+// with warp-wide MMA issue, the totals written as the output kernel's operand, contiguous
+// partials, overlapped launches, zeroing in the ragged chunk only and packed products
+// (212 us states, 9 totals, 230 output; 319 us of HBM traffic in all).
 #include <cuda.h>
 
 #include <algorithm>
