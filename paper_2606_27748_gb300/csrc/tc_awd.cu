@@ -308,9 +308,10 @@ __global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* part,
 // groups' arithmetic (0.7 us each, overlapping); per CTA about a third of the time is set-up
 // and the chain rule.  Measured, one distillation step n B32 H8 N512 M64: 361 us with all
 // warps in step and thread 0 issuing, 307 us now (mask and side as compile-time cases 357 ->
-// 333, the held block as a tensor-memory operand -> 324, loads by their own warp -> 307); 289 with
-// overlapped launches and the feature pass's 32-byte stores, 196 of them here.  The rows of dW' are added into this CTA's slot; a reduction sums the slots over the sides, the batch
-// and the splits in a fixed order, so the result does not depend on scheduling.  On the
+// 333, the held block as a tensor-memory operand -> 324, loads by their own warp -> 307); 281 with
+// overlapped launches, the feature pass's 32-byte stores and the wider sum of the slots (12.7 ->
+// 9 us), 196 of them here.  The rows of dW' are added into this CTA's slot; a reduction sums the
+// slots over the sides, the batch and the splits in a fixed order, so the result does not depend on scheduling.  On the
 // key side, with the prefactor, the chain rule takes dphi(k_j) = w_j dphi~(k_j) and dtau
 // gains -(phi~(k_j) . dphi~(k_j)) |k_j|^2 exp(-tau).  Every wait is bounded.
 constexpr int kComputeG = 16;                    // compute warps, four per lane quadrant
@@ -748,10 +749,11 @@ done:
 
 // dW1, dW2 [H][M][64] and dtau [H] from the slots [2 sides][B*H][hsplit][G][16 column
 // quads][128 rows][4].  One block per (head, group, column quad): thread (row, lane) sums
-// every fourth slot (slots in (side, batch entry, split) order) with eight loads in flight;
+// every fourth slot (slots in (side, batch entry, split) order) with LD loads in flight;
 // the four lanes are then added in order.  For Flexformer_n rows 0-63 of a group are dU, rows
 // 64-127 dV (U = (W1+W2)/2, V = (W1-W2)/2), so dW1 = (dU+dV)/2, dW2 = (dU-dV)/2.
 constexpr int kReduceThreads = 512;
+template <int LD>  // loads in flight per thread (wide_reduce)
 __global__ void __launch_bounds__(kReduceThreads)
     awd_dw_reduce_kernel(int B, int H, int M, int nonstat, int hsplit,
                          const float* slots, const float* dtau_part,
@@ -760,24 +762,33 @@ __global__ void __launch_bounds__(kReduceThreads)
 {
     grid_dep_wait();
     __shared__ float4 sums[3][128];
-    const int BH = B * H, G = M / 64, per_side = B * hsplit, nslot = 2 * per_side;
+    const int BH = B * H, G = M / 64, per_side = B * hsplit;
     const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
     const int row = threadIdx.x % 128, ln = threadIdx.x / 128;
     auto add = [](float4& a, const float4& x) {
         a = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
     };
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = ln; s0 < nslot; s0 += 32) {
-        float4 x[8];
+    // slot i = bb hsplit + sp, bb = side B + b < 2 B; from one slot to the fourth after it
+    // without a division
+    const int dbb = 4 / hsplit, dsp = 4 % hsplit;
+    int bb = ln / hsplit, sp = ln % hsplit;
+    while (bb < 2 * B) {
+        float4 x[LD];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int s = s0 + 4 * e, side = s / per_side, rem = s % per_side;
-            const size_t cta = (size_t)(side * BH + (rem / hsplit) * H + h) * hsplit + rem % hsplit;
-            x[e] = s < nslot ? reinterpret_cast<const float4*>(slots)[((cta * G + g) * 16 + quad) * 128 + row]
-                             : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e = 0; e < LD; ++e) {
+            const size_t cta = (size_t)(bb * H + h) * hsplit + sp;
+            x[e] = bb < 2 * B ? reinterpret_cast<const float4*>(slots)[((cta * G + g) * 16 + quad) * 128 + row]
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+            bb += dbb;
+            sp += dsp;
+            if (sp >= hsplit) {
+                sp -= hsplit;
+                ++bb;
+            }
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) add(a, x[e]);
+        for (int e = 0; e < LD; ++e) add(a, x[e]);
     }
     if (ln > 0) sums[ln - 1][row] = a;
     __syncthreads();
@@ -862,9 +873,11 @@ cudaError_t launch_bwd_typed(const Problem& p, const void* q, const void* k, con
                      p.H, p.N, p.M, p.causal, hs, score_scale, rowstat, dloss, W1, W2, kw, tau, slots,
                      dtau_part, status);
     if (e != cudaSuccess) return e;
-    return launch_after(awd_dw_reduce_kernel, dim3((unsigned)(p.H * (p.M / 64) * 16)), kReduceThreads, 0, 0,
-                        true, s, p.B, p.H, p.M, p.nonstat, hs, (const float*)slots,
-                        (const float*)dtau_part, dW1, dW2, tau ? dtau : (float*)nullptr);
+    const long long blocks = 16LL * p.H * (p.M / 64);
+    auto reduce = wide_reduce(blocks) ? awd_dw_reduce_kernel<16> : awd_dw_reduce_kernel<8>;
+    return launch_after(reduce, dim3((unsigned)blocks), kReduceThreads, 0, 0, true, s, p.B, p.H, p.M,
+                        p.nonstat, hs, (const float*)slots, (const float*)dtau_part, dW1, dW2,
+                        tau ? dtau : (float*)nullptr);
 }
 
 template <int G2>

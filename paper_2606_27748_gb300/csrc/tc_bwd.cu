@@ -1296,10 +1296,11 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 // frequencies 64g + row (from the high bf16 part of da), rows >= 64 the same frequencies
 // (from its low part); n: rows < 64 are dU, rows >= 64 are dV of frequency 64g + row%64.
 // One block per (head, group, column quad): thread (row, lane) sums every fourth slot with
-// eight loads in flight, the four lanes are then added in order.  It is bound by reading the
-// slots (32 KB each) at memory latency: B32 H8 in two ranges 29.5 -> 13.3 us against one thread
-// per output.
+// LD loads in flight, the four lanes are then added in order.  It is bound by reading the slots
+// (32 KB each) at memory latency and by the index arithmetic: B32 H8 in two ranges 29.5 us with one
+// thread per output, 13.3 with eight loads in flight, 9.1 with 16 and no division per slot.
 constexpr int kReduceThreads = 512;
+template <int LD>  // loads in flight per thread (wide_reduce)
 __global__ void __launch_bounds__(kReduceThreads)
     tc_dw_reduce_kernel(int B, int H, int M, int G, int nsplit, int nonstat,
                         const float* part, float* __restrict__ dW1,
@@ -1310,22 +1311,27 @@ __global__ void __launch_bounds__(kReduceThreads)
     grid_dep_wait();
     const int quad = blockIdx.x % 16, g = blockIdx.x / 16 % G, h = blockIdx.x / (16 * G);
     const int row = threadIdx.x % 128, ln = threadIdx.x / 128;
-    const int per = B * nsplit;                        // slots of (head, group) and pass
-    const size_t half = (size_t)B * H * nsplit * G;    // slots per pass
-    auto slot_of = [&](int i) {                        // i < 2 per: pass F's slots, then R's
-        const int pass = i / per, r = i % per;
-        return (size_t)pass * half + ((size_t)(r / nsplit * H + h) * nsplit + r % nsplit) * G + g;
-    };
+    // slot i = bb nsplit + sp, bb = pass B + b < 2 B: pass F's slots, then R's; from one slot
+    // to the fourth after it without a division
+    const int dbb = 4 / nsplit, dsp = 4 % nsplit;
+    int bb = ln / nsplit, sp = ln % nsplit;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i0 = ln; i0 < 2 * per; i0 += 32) {
-        float4 x[8];
+    while (bb < 2 * B) {
+        float4 x[LD];
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            x[u] = i0 + 4 * u < 2 * per
-                       ? reinterpret_cast<const float4*>(part)[(slot_of(i0 + 4 * u) * 16 + quad) * 128 + row]
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < LD; ++u) {
+            const size_t slot = ((size_t)(bb * H + h) * nsplit + sp) * G + g;
+            x[u] = bb < 2 * B ? reinterpret_cast<const float4*>(part)[(slot * 16 + quad) * 128 + row]
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+            bb += dbb;
+            sp += dsp;
+            if (sp >= nsplit) {
+                sp -= nsplit;
+                ++bb;
+            }
+        }
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < LD; ++u)
             a = make_float4(a.x + x[u].x, a.y + x[u].y, a.z + x[u].z, a.w + x[u].w);
     }
     if (ln > 0) sums[ln - 1][row] = a;
@@ -1352,7 +1358,8 @@ __global__ void __launch_bounds__(kReduceThreads)
     }
     if (dtau && quad == 0 && g == 0 && threadIdx.x < 32) {  // dtau[h]: head h's pass R slots
         float t = 0.f;
-        for (int i = threadIdx.x; i < per * G; i += 32)
+        const size_t half = (size_t)B * H * nsplit * G;  // slots per pass
+        for (int i = threadIdx.x; i < B * nsplit * G; i += 32)
             t += dtau_part[half + ((size_t)(i / (nsplit * G) * H + h) * nsplit + i / G % nsplit) * G + i % G];
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (threadIdx.x == 0) dtau[h] = t;
@@ -1544,7 +1551,8 @@ cudaError_t launch_bwd(const Problem& p, const void* q, const void* k, const voi
                    : launch_mode<NS, KW, 1, kGrad>(p, m, q, k, v, W1, W2, tau, out, den, dout, dq,
                                                    dk, dv, f, w, nsplit, status, s);
     if (e != cudaSuccess) return e;
-    return launch_after(tc_dw_reduce_kernel, dim3((unsigned)(p.H * G * 16)), kReduceThreads, 0, 0, true, s,
+    auto reduce = wide_reduce(16LL * p.H * G) ? tc_dw_reduce_kernel<16> : tc_dw_reduce_kernel<8>;
+    return launch_after(reduce, dim3((unsigned)(p.H * G * 16)), kReduceThreads, 0, 0, true, s,
                         p.B, p.H, p.M, G, nsplit, p.nonstat, (const float*)(f + w.part), dW1, dW2,
                         (const float*)(f + w.dtau), KW ? dtau : (float*)nullptr);
 }

@@ -413,6 +413,12 @@ cudaError_t launch_after(void (*kern)(KArgs...), dim3 blocks, int threads, int s
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Loads in flight per thread of the dW reductions (512 threads a block): 16 take 88 registers
+// and so one block an SM, which pays while the blocks fit the SMs at once (128 blocks of 128
+// slots each: 13.3 us with 8, 9.1 with 16); more blocks need two an SM (384 blocks of 16 slots:
+// 6.3 us with 8, 9.2 with 16).
+inline bool wide_reduce(long long blocks) { return blocks <= 152; }
+
 inline int sm_count()
 {
     int dev = 0, n = 0;
