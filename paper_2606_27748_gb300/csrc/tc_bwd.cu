@@ -47,8 +47,8 @@
 // The phases of a chunk depend on one another (an SM holds one CTA's tensor memory), so the
 // length of this chain bounds the kernel, not DRAM (7%) or the tensor pipe: a chunk of s M128
 // takes about 15 us in F and R together, from 19.4 with all threads meeting at CTA barriers
-// and thread 0 issuing; measured forward and backward: s B8 H12 N8192 M128 2.16 -> 1.58 ms,
-// n non-causal B32 H8 N4000 M64 1.30 -> 0.91 ms.
+// and thread 0 issuing; measured forward and backward: s B8 H12 N8192 M128 2.16 -> 1.57 ms,
+// n non-causal B32 H8 N4000 M64 1.30 -> 0.89 ms.
 // Every wait is bounded.  Tiles of the following chunks are loaded as soon as the region
 // each one occupies is free (two buffers where the pass leaves room).
 //
