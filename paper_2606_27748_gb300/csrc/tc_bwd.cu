@@ -94,10 +94,13 @@ struct BwCfg {
     static constexpr uint32_t SN = PK + 32768;     // state snapshot [feature][64 dcol], bf16
     static constexpr uint32_t ZR = SN + 16384;     // z or r [2 chunk parities][128] fp32
     static constexpr uint32_t CROW = ZR + 1024;    // c_t [2 chunk parities][128] fp32
-    static constexpr uint32_t SPART = CROW + 1024; // s_t partials [4 column quarters][128] fp32
-    // s: a receive block for dk (its W rows take half the space); n has no room for one
+    // s_t partials [4 column quarters][128] fp32; kGrad has a second set behind them, by chunk
+    // parity
+    static constexpr uint32_t SPART = CROW + 1024;
+    // s: a receive block for dk (its W rows take half the space; causal only, so the second
+    // set of partials shares its place); n has no room for one
     static constexpr uint32_t XR = NS ? PK : SPART + 2048;
-    static constexpr uint32_t BYTES = SPART + 2048 + (NS ? 0 : 16384);
+    static constexpr uint32_t BYTES = SPART + 2048 + (NS ? 2048 : 16384);
     static constexpr uint32_t T_P = 0, T_A = 128, T_D = 256, T_S = 384;
     static_assert(BYTES + 1024 <= 232448, "shared memory budget");
 };
@@ -613,8 +616,8 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
             }
         }
     };
-    // this thread's share of row t's s_t partials, in order
-    auto row_sum = [&](int r) { return (spart[r] + spart[128 + r]) + (spart[256 + r] + spart[384 + r]); };
+    // row t's s_t partials in `sp`, in order
+    auto row_sum = [&](const float* sp) { return (sp[t] + sp[128 + t]) + (sp[256 + t] + sp[384 + t]); };
     // TMA of one tile of chunk cn into shared memory, and of a chunk's rows into L2
     auto load_tile = [&](uint32_t dst, const CUtensorMap* map, int cn, uint64_t* bar) {
         wtma_load_3d(sb + dst, map, 0, cn * kC, bh, bar);
@@ -909,7 +912,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                     if (!take_rows(dv, T_DV, t0, valid, 0.f, 0, 0, sb + L::PQ, sb + L::DA2)) goto done;
                     snapshot(zr + 128 * ((it + 1) & 1));
                     if (!wwait(&m0, p_m0)) goto done;  // dk, dW
-                    if (!take_rows(dk, T_X, t0, valid, KW ? 2.f * itau * row_sum(t) : 0.f, L::K, 1,
+                    if (!take_rows(dk, T_X, t0, valid, KW ? 2.f * itau * row_sum(spart) : 0.f, L::K, 1,
                                    sb + (kLate ? L::PK : L::PQ + 16384), sb + L::XR))
                         goto done;
                     if (KW) arrive(&srdy);
@@ -1214,8 +1217,12 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                     if (!wwait(&m0, p_m0)) goto done;
                     const float sp = feature_backward(std::false_type{}, zr, sb + L::PK, sb + L::GT, da1, 1.0f,
                                                       valid, wk);
+                    // Two sets of partials: with two tile buffers a warp may be here while another
+                    // still reads the row sums of chunk i - 1 below.  None may be a chunk further
+                    // ahead: m0 of chunk i + 1 follows every warp's srdy of chunk i - 1.
+                    float* sp_ = spart + 512 * (i & 1);
                     if (KW) {
-                        spart[128 * wg + t] = sp;
+                        sp_[128 * wg + t] = sp;
                         dtau_acc = fmaf(lw0 - logf(wk), sp, dtau_acc);  // centred, as above
                     }
                     if (i > 0 && !finalize(t0 - kC, kC)) goto done;
@@ -1223,7 +1230,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                     if (!wwait(&m1, p_m1)) goto done;
                     if (i > 0 && (!staging_free(0) || !staging_free(1))) goto done;
                     if (!take_rows(dv, T_DV, t0, valid, 0.f, 0, 0, sb + L::Q, sb + L::DO) ||
-                        !take_rows(dk, T_X, t0, valid, KW ? 2.f * itau * row_sum(t) : 0.f, kb[i % NB],
+                        !take_rows(dk, T_X, t0, valid, KW ? 2.f * itau * row_sum(sp_) : 0.f, kb[i % NB],
                                    1, sb + L::DA2, sb + L::O))
                         goto done;
                     arrive(&srdy);
