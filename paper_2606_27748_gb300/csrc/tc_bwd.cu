@@ -651,10 +651,14 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
                 mbar_arrive_cluster(mapa(smem_u32(&xdone[xi]), partner));
             }
     };
-    // A compute warp, before it rewrites the staging region of exchange xi.
+    // A compute warp, before it rewrites the staging region of exchange xi.  Every warp that waits
+    // has to gate the next exchange, or that one may complete first and the parity wait miss its
+    // phase: in kGrad, where the staging regions hold nothing else, only the warps that send wait
+    // (the partner's next landing takes their rows); in the causal passes all wait, before the
+    // arrival that gates the MMAs whose rows are sent.
     uint32_t ph_xdone[2] = {0, 0};
     auto staging_free = [&](int xi) -> bool {
-        if (CS == 1) return true;
+        if (CS == 1 || (MODE == kGrad && (t >> 6) == rank)) return true;  // uniform over a warp
         const bool ok = __all_sync(0xffffffffu,
                                    bar_wait_cluster(&xdone[xi], ph_xdone[xi], &abort_flag, status));
         ph_xdone[xi] ^= 1;

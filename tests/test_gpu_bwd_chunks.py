@@ -52,3 +52,10 @@ def check(variant, M, N, tau):
     ("s", 513, True), ("s", 700, False), ("n", 640, True), ("n", 770, True), ("n", 600, False)])
 def test_chunks_of_one_cta(variant, N, tau):
     check(variant, 64, N, tau)
+
+
+@pytest.mark.parametrize("variant,N,tau", [
+    ("s", 513, True), ("s", 700, False), ("n", 640, True), ("n", 770, False)])
+def test_chunks_of_one_cluster(variant, N, tau):
+    """M = 128: the two CTAs of a sequence exchange rows chunk after chunk."""
+    check(variant, 128, N, tau)
