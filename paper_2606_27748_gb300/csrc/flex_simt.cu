@@ -209,6 +209,51 @@ __device__ __forceinline__ void mm_tn(const float* a, int pa, const float* b, in
     }
 }
 
+// Products with a masked T x T block M (M[i][j] = 0 for j > i) end at the diagonal: half the
+// work, and a masked key or query is left out, not multiplied by zero, so an infinite or NaN
+// value (or a key weight that overflows) reaches no row that does not see it.
+// Rows 4y..4y+3 of M B: acc[r][c] += sum_{j <= 4y + r} M[4y + r][j] b[j pb + c].
+__device__ __forceinline__ void mm_masked(const float* M, int pm, int y, const float* b, int pb,
+                                          float (&acc)[4][4])
+{
+    mm_nn(M + 4 * y * pm, pm, b, pb, 2 * pb, 3 * pb, 4 * pb, 4 * y, acc);
+    float4 x[4];  // the diagonal block
+#pragma unroll
+    for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(M + (4 * y + r) * pm + 4 * y);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 v = *reinterpret_cast<const float4*>(b + (4 * y + k) * pb);
+#pragma unroll
+        for (int r = k; r < 4; ++r) {
+            const float m = k == 0 ? x[r].x : k == 1 ? x[r].y : k == 2 ? x[r].z : x[r].w;
+            acc[r][0] = fmaf(m, v.x, acc[r][0]);
+            acc[r][1] = fmaf(m, v.y, acc[r][1]);
+            acc[r][2] = fmaf(m, v.z, acc[r][2]);
+            acc[r][3] = fmaf(m, v.w, acc[r][3]);
+        }
+    }
+}
+// Rows 4y..4y+3 of M^T B over T rows: acc[r][c] += sum_{i >= 4y + r} M[i][4y + r] b[i pb + c].
+__device__ __forceinline__ void mm_masked_t(const float* M, int pm, int y, const float* b, int pb,
+                                            int T, float (&acc)[4][4])
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // the diagonal block
+        const float4 x = *reinterpret_cast<const float4*>(M + (4 * y + k) * pm + 4 * y);
+        const float4 v = *reinterpret_cast<const float4*>(b + (4 * y + k) * pb);
+        const float xr[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int r = 0; r <= k; ++r) {
+            acc[r][0] = fmaf(xr[r], v.x, acc[r][0]);
+            acc[r][1] = fmaf(xr[r], v.y, acc[r][1]);
+            acc[r][2] = fmaf(xr[r], v.z, acc[r][2]);
+            acc[r][3] = fmaf(xr[r], v.w, acc[r][3]);
+        }
+    }
+    const int i = 4 * y + 4;
+    mm_tn(M + i * pm + 4 * y, pm, b + i * pb, pb, T - i, acc);
+}
+
 template <int R, int C>
 __device__ __forceinline__ void zero(float (&acc)[R][C])
 {
@@ -624,12 +669,10 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
             for (int n = 0; n < ND; ++n) {
                 const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
-                if (y < TT)
-                    mm_nn(A + 4 * y * L.pa, L.pa, V + e, L.pd, 2 * L.pd, 3 * L.pd, 4 * L.pd, L.T,
-                          num[n]);
+                if (y < TT) mm_masked(A, L.pa, y, V + e, L.pd, num[n]);
             }
             if (tid < lpr * L.T)
-                for (int j = part; j < L.T; j += lpr)
+                for (int j = part; j <= row; j += lpr)
                     dsum = fmaf(A[row * L.pa + j], V[j * L.pd + d], dsum);
         }
         if (tid < lpr * L.T) {
@@ -889,9 +932,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncthreads();
             if (f.on) {
                 zero(dp);
-                if (p.causal)
-                    mm_nn(dA + 4 * f.y * L.pa, L.pa, Pk + 4 * f.x, L.pp, 2 * L.pp, 3 * L.pp,
-                          4 * L.pp, L.T, dp);
+                if (p.causal) mm_masked(dA, L.pa, f.y, Pk + 4 * f.x, L.pp, dp);
                 mm_nt<4>(G + 4 * f.y * L.pd, L.pd, Sg + f.x * L.pd, L.CT * L.pd, d, dp);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
@@ -960,7 +1001,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (f.on) {
                 zero(dp);
-                if (p.causal) mm_tn(dA + 4 * f.y, L.pa, Pq + 4 * f.x, L.pp, L.T, dp);
+                if (p.causal) mm_masked_t(dA, L.pa, f.y, Pq + 4 * f.x, L.pp, L.T, dp);
                 mm_nt<4>(V + 4 * f.y * L.pd, L.pd, Rg + f.x * L.pd, L.CT * L.pd, d, dp);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
@@ -1004,7 +1045,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int n = 0; n < ND; ++n) {
             const int id = tid + n * kThreads, y = id / d4, e = 4 * (id % d4);
             if (y < TT) {
-                if (p.causal) mm_tn(A + 4 * y, L.pa, G + e, L.pd, L.T, dvt[n]);
+                if (p.causal) mm_masked_t(A, L.pa, y, G + e, L.pd, L.T, dvt[n]);
                 if (tau)
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
