@@ -34,6 +34,7 @@ using namespace tc;
 
 constexpr int kC = 128;
 constexpr int kThreadsA = 256;
+constexpr int kOnePerSm = 116 * 1024;  // more than half of an SM's 228 KB
 
 template <int G2>  // 64-feature blocks of phi: 2M / 64
 struct AwdCfg {
@@ -828,7 +829,12 @@ cudaError_t launch_typed(const Problem& p, const void* q, const void* k, const v
     if (!make_act_map(&mq, q, BH, p.N) || !make_act_map(&mk, k, BH, p.N) ||
         !make_feat_map(&mpq, pq, BH, p.N, 2 * p.M) || !make_feat_map(&mpk, pk, BH, p.N, 2 * p.M))
         return cudaErrorInvalidValue;
-    const int smem = (int)AwdCfg<G2>::BYTES + 1024;
+    // A grid of at most one block an SM asks for so much shared memory that an SM takes one
+    // (M = 64 would fit two): it starts while the feature map's blocks still leave, on whatever
+    // SMs are free by then, and pairs on some of them leave others idle.  Loss of one sequence, n,
+    // N 16384 M 64 (128 blocks): 375 us, 248 with one block an SM.
+    int smem = (int)AwdCfg<G2>::BYTES + 1024;
+    if ((long long)BH * nqb <= sm_count()) smem = std::max(smem, kOnePerSm);
     auto kern = tc_awd_kernel<G2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
