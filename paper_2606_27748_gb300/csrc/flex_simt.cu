@@ -31,7 +31,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxCluster = 8;   // CTAs that share one sequence
 constexpr int kMaxT = 128;       // tokens per chunk (over 64: the non-causal forward only)
-constexpr int kMaxMG = 32;       // frequencies per group (64 features)
+constexpr int kMaxMG = 32;       // frequencies per group (64 features) of chunks over 32 tokens
 
 __device__ __forceinline__ float load_act(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ float load_act(const __nv_bfloat16* p, size_t i)
@@ -128,7 +128,15 @@ struct Plan {
     int wres;           // every group's projection rows stay in shared memory
     int CL;             // CTAs per sequence
     int S, W, dW, Xq, Xk, V, G, Pq, Pk, A, red, total;  // offsets (floats)
+    int nt;             // threads per CTA
+    int any;            // a plan of the kernels with NT = 0
 };
+
+// NT: threads of the CTA, kThreads or (0) Plan::nt.  Kernels with NT = 0 take the plans of short
+// sequences and of many small ones: any thread count, groups of any size, no products with a
+// state that is still zero and none that nothing reads.  (One kernel for every plan was 1-3%
+// slower on long sequences; so is the count by a function instead of this expression.)
+#define FLEX_THREADS (NT ? NT : (int)blockDim.x)
 
 // Row of column tile x, column c in arrays whose rows are read four at a time by
 // neighbouring x (projection rows, state rows): c CT + x, so that 16 lanes with
@@ -266,16 +274,16 @@ __device__ __forceinline__ void zero(float (&acc)[R][C])
 // Projection rows of group g of one head.  s: column c (0, 1) of tile x is frequency
 // 2x + c; n: columns 0..3 are u, w of frequency 2x, then u, w of 2x + 1, with
 // U = (W1+W2)/2, V = (W1-W2)/2.  Rows past M are zero.
-template <bool NS>
+template <bool NS, int NT>
 __device__ void stage_projection(const Problem& p, const Plan& L, const float* W1,
                                  const float* W2, int h, int g, float* W)
 {
     const int d = p.d, dq = d / 4, total = L.KP * dq;
-    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * kThreads) {  // four loads in flight
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * FLEX_THREADS) {  // four loads in flight
         float4 w[4], w2[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int idx = i0 + u * kThreads, row = idx / dq, c = row / L.CT, x = row % L.CT;
+            const int idx = i0 + u * FLEX_THREADS, row = idx / dq, c = row / L.CT, x = row % L.CT;
             const int f = g * L.MG + 2 * x + (NS ? c >> 1 : c);
             w[u] = w2[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (idx < total && f < p.M) {
@@ -286,7 +294,7 @@ __device__ void stage_projection(const Problem& p, const Plan& L, const float* W
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int idx = i0 + u * kThreads, row = idx / dq;
+            const int idx = i0 + u * FLEX_THREADS, row = idx / dq;
             if (idx >= total) break;
             if (NS) {
                 const float sg = (row / L.CT & 1) ? -1.f : 1.f;
@@ -300,16 +308,16 @@ __device__ void stage_projection(const Problem& p, const Plan& L, const float* W
 
 // Rows of a chunk from one tensor, or from two (src2 non-null), zero from row `rows` on; the
 // loads of a thread (up to eight) are issued before its stores.
-template <typename T>
+template <int NT, typename T>
 __device__ void load_rows(const T* src, const T* src2, size_t base, int rows, int d, float* dst,
                           float* dst2, int pitch, int nrows)
 {
     const int dq = d / 4, total = nrows * dq;
-    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * kThreads) {
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * FLEX_THREADS) {
         float4 x[4], y[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int idx = i0 + u * kThreads, t = idx / dq, e = 4 * (idx % dq);
+            const int idx = i0 + u * FLEX_THREADS, t = idx / dq, e = 4 * (idx % dq);
             x[u] = y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (t < rows) {
                 x[u] = load_act4(src, base + (size_t)t * d + e);
@@ -318,7 +326,7 @@ __device__ void load_rows(const T* src, const T* src2, size_t base, int rows, in
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int idx = i0 + u * kThreads, t = idx / dq, e = 4 * (idx % dq);
+            const int idx = i0 + u * FLEX_THREADS, t = idx / dq, e = 4 * (idx % dq);
             if (idx >= total) break;
             *reinterpret_cast<float4*>(dst + t * pitch + e) = x[u];
             if (src2) *reinterpret_cast<float4*>(dst2 + t * pitch + e) = y[u];
@@ -466,13 +474,14 @@ __device__ __forceinline__ void mm_tn_split(const float* a, int pa, const float*
 
 // State of one group: S[prow(f)][e] += sum_j P[j][f] Y[j][e] and, in column d, the sum
 // weighted by Y[j][d] (z, or r from G = [g | c]).
+template <int NT>
 __device__ __forceinline__ void state_update(const Plan& L, int d, const float* P, const float* Y,
                                              float* S)
 {
     const int dq = d / 4, tiles = L.CT * dq;
     // over long chunks, lanes without a tile of their own share one
-    const int ks = L.T <= 64 ? 1 : 4 * tiles <= kThreads ? 4 : 2 * tiles <= kThreads ? 2 : 1;
-    for (int i0 = threadIdx.x & ~31; i0 < tiles * ks; i0 += kThreads) {
+    const int ks = L.T <= 64 ? 1 : 4 * tiles <= FLEX_THREADS ? 4 : 2 * tiles <= FLEX_THREADS ? 2 : 1;
+    for (int i0 = threadIdx.x & ~31; i0 < tiles * ks; i0 += FLEX_THREADS) {
         // (whole warps take part in the exchange: lanes past the end repeat the last tile)
         const int at = i0 + (threadIdx.x & 31), id = min(at / ks, tiles - 1);
         const int x = id / dq, e = 4 * (id % dq);
@@ -487,13 +496,25 @@ __device__ __forceinline__ void state_update(const Plan& L, int d, const float* 
                              s->w + acc[r][3]);
         }
     }
-    if (threadIdx.x < 4 * L.F) {  // four lanes per feature (4 F is a multiple of 32)
-        const int f = threadIdx.x >> 2;
-        float z = 0.f;
-        for (int j = threadIdx.x & 3; j < L.T; j += 4) z = fmaf(P[j * L.pp + f], Y[j * L.pd + d], z);
-        z += __shfl_xor_sync(0xffffffffu, z, 1);
-        z += __shfl_xor_sync(0xffffffffu, z, 2);
-        if ((threadIdx.x & 3) == 0) S[prow(L, f) * L.pd + d] += z;
+    // column d: four lanes per feature (4 F is a multiple of 32)
+    if constexpr (NT == kThreads) {
+        if (threadIdx.x < 4 * L.F) {
+            const int f = threadIdx.x >> 2;
+            float z = 0.f;
+            for (int j = threadIdx.x & 3; j < L.T; j += 4) z = fmaf(P[j * L.pp + f], Y[j * L.pd + d], z);
+            z += __shfl_xor_sync(0xffffffffu, z, 1);
+            z += __shfl_xor_sync(0xffffffffu, z, 2);
+            if ((threadIdx.x & 3) == 0) S[prow(L, f) * L.pd + d] += z;
+        }
+    } else {
+        for (int i = threadIdx.x; i < 4 * L.F; i += FLEX_THREADS) {
+            const int f = i >> 2;
+            float z = 0.f;
+            for (int j = i & 3; j < L.T; j += 4) z = fmaf(P[j * L.pp + f], Y[j * L.pd + d], z);
+            z += __shfl_xor_sync(0xffffffffu, z, 1);
+            z += __shfl_xor_sync(0xffffffffu, z, 2);
+            if ((i & 3) == 0) S[prow(L, f) * L.pd + d] += z;
+        }
     }
 }
 
@@ -501,12 +522,13 @@ __device__ __forceinline__ void state_update(const Plan& L, int d, const float* 
 // total, or the sum over the lower (prefix) or higher (suffix) ranks.  Each CTA owns a slice
 // of the state: it alone reads and rewrites that slice in all CTAs, so it works in place.
 enum { kTotal, kPrefix, kSuffix };
+template <int NT>
 __device__ void exchange_state(float* S, int n, int CL, int mode)
 {
     tc::cluster_sync();
     const uint32_t base = tc::smem_u32(S);
     const int rank = (int)tc::cluster_rank();
-    for (int i = rank * kThreads + threadIdx.x; i < n / 4; i += CL * kThreads) {
+    for (int i = rank * FLEX_THREADS + threadIdx.x; i < n / 4; i += CL * FLEX_THREADS) {
         float4 v[kMaxCluster];
 #pragma unroll
         for (int r = 0; r < kMaxCluster; ++r)
@@ -548,7 +570,7 @@ __device__ __forceinline__ void chunk_range(const Plan& L, int N, int rank, int*
 // ------------------------------------------------------------------------------------
 // Forward.
 // ------------------------------------------------------------------------------------
-template <typename T, bool NS, int ND>
+template <typename T, bool NS, int ND, int NT>
 __global__ void __launch_bounds__(kThreads, 2)
     simt_fwd_kernel(Problem p, Plan L, const T* q, const T* k, const T* v, const float* W1,
                     const float* W2, const float* tau, T* out, float* den)
@@ -572,20 +594,20 @@ __global__ void __launch_bounds__(kThreads, 2)
 
     if (L.wres)
         for (int g = 0; g < L.ng; ++g)
-            stage_projection<NS>(p, L, W1, W2, h, g, sm + L.W + g * gW);
-    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
+            stage_projection<NS, NT>(p, L, W1, W2, h, g, sm + L.W + g * gW);
+    for (int i = tid; i < L.ng * gS; i += FLEX_THREADS) S[i] = 0.f;
 
     if (!p.causal || L.CL > 1) {  // this range's sums
         for (int c = cb; c < ce; ++c) {
             const int t0 = c * L.T, rows = min(L.T, N - t0);
-            load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
+            load_rows<NT>(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
             unit_weights(L, d, rows, V);
             __syncthreads();
             if (tau) weight_keys(L, Xk, rows, d, itau, V, red);
             for (int g = 0; g < L.ng; ++g) {
                 float* W = sm + L.W + g * gW;
                 if (!L.wres) {
-                    stage_projection<NS>(p, L, W1, W2, h, g, W);
+                    stage_projection<NS, NT>(p, L, W1, W2, h, g, W);
                     __syncthreads();
                 }
                 if (f.on) {
@@ -594,19 +616,20 @@ __global__ void __launch_bounds__(kThreads, 2)
                     store_tile(Pk, L.pp, f, pf);
                 }
                 __syncthreads();
-                state_update(L, d, Pk, V, S + g * gS);
+                state_update<NT>(L, d, Pk, V, S + g * gS);
                 __syncthreads();
             }
         }
-        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
+        if (L.CL > 1) exchange_state<NT>(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
     }
     __syncthreads();
 
     for (int c = cb; c < ce; ++c) {
         const int t0 = c * L.T, rows = min(L.T, N - t0);
-        load_rows(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
+        const bool seen = NT || !p.causal || L.CL > 1 || c > cb;  // (else the state is still zero)
+        load_rows<NT>(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
         if (p.causal) {
-            load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
+            load_rows<NT>(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
             unit_weights(L, d, rows, V);
         }
         __syncthreads();
@@ -619,7 +642,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             float* W = sm + L.W + g * gW;
             float* Sg = S + g * gS;
             if (!L.wres) {
-                stage_projection<NS>(p, L, W1, W2, h, g, W);
+                stage_projection<NS, NT>(p, L, W1, W2, h, g, W);
                 __syncthreads();
             }
             if (f.on) {
@@ -636,12 +659,12 @@ __global__ void __launch_bounds__(kThreads, 2)
                 mm_nt<4>(Pq + 4 * ay * L.pp, L.pp, Pk + ax * L.pp, TT * L.pp, L.F, aa);
 #pragma unroll
             for (int n = 0; n < ND; ++n) {
-                const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
-                if (y < TT)
+                const int id = tid + n * FLEX_THREADS, y = id / dq, e = 4 * (id % dq);
+                if (seen && y < TT)
                     mm_nn(Pq + 4 * y * L.pp, L.pp, Sg + e, L.CT * L.pd, 2 * L.CT * L.pd,
                           3 * L.CT * L.pd, L.pd, L.F, num[n]);
             }
-            if (tid < lpr * L.T)  // denominator
+            if (seen && tid < lpr * L.T)  // denominator
                 for (int i = part; i < L.CT; i += lpr) {
                     const float4 x = *reinterpret_cast<const float4*>(Pq + row * L.pp + 4 * i);
                     const float* z = Sg + i * L.pd + d;
@@ -652,7 +675,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 }
             __syncthreads();
             if (p.causal) {
-                state_update(L, d, Pk, V, Sg);
+                if (NT || c + 1 < ce) state_update<NT>(L, d, Pk, V, Sg);  // (else nothing reads it)
                 if (g + 1 < L.ng) __syncthreads();
             }
         }
@@ -668,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             __syncthreads();
 #pragma unroll
             for (int n = 0; n < ND; ++n) {
-                const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
+                const int id = tid + n * FLEX_THREADS, y = id / dq, e = 4 * (id % dq);
                 if (y < TT) mm_masked(A, L.pa, y, V + e, L.pd, num[n]);
             }
             if (tid < lpr * L.T)
@@ -686,7 +709,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         __syncthreads();
 #pragma unroll
         for (int n = 0; n < ND; ++n) {
-            const int id = tid + n * kThreads, y = id / dq, e = 4 * (id % dq);
+            const int id = tid + n * FLEX_THREADS, y = id / dq, e = 4 * (id % dq);
             if (y < TT)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
@@ -755,14 +778,14 @@ __device__ __forceinline__ void store_chain(const Plan& L, const Place& f, const
 }
 
 // dx tiles += da W and dW += da^T X of one group.
-template <bool NS, int ND>
+template <bool NS, int ND, int NT>
 __device__ __forceinline__ void project_back(const Plan& L, int d, const float* D, const float* W,
                                              const float* X, float* dW, float (&dx)[ND][4][4])
 {
     const int dq = d / 4, TT = L.T / 4, o = L.CT * L.pd;
 #pragma unroll
     for (int n = 0; n < ND; ++n) {
-        const int id = threadIdx.x + n * kThreads, y = id / dq, e = 4 * (id % dq);
+        const int id = threadIdx.x + n * FLEX_THREADS, y = id / dq, e = 4 * (id % dq);
         if (y < TT) {
             if (NS)
                 mm_nn(D + 4 * y * L.pp, L.pp, W + e, o, 2 * o, 3 * o, L.pd, L.KP, dx[n]);
@@ -770,7 +793,7 @@ __device__ __forceinline__ void project_back(const Plan& L, int d, const float* 
                 mm_nn(D + 4 * y * L.pp, L.pp, W + e, o, L.pd, o + L.pd, 2 * L.pd, L.KP, dx[n]);
         }
     }
-    for (int id = threadIdx.x; id < L.KP / 4 * dq; id += kThreads) {
+    for (int id = threadIdx.x; id < L.KP / 4 * dq; id += FLEX_THREADS) {
         const int x = id / dq, e = 4 * (id % dq);
         float acc[4][4];
         zero(acc);
@@ -784,14 +807,14 @@ __device__ __forceinline__ void project_back(const Plan& L, int d, const float* 
     }
 }
 
-template <typename T, int ND>
+template <typename T, int ND, int NT>
 __device__ __forceinline__ void store_rows(const Plan& L, int d, const float (&x)[ND][4][4],
                                            T* dst, size_t base, int rows)
 {
     const int dq = d / 4;
 #pragma unroll
     for (int n = 0; n < ND; ++n) {
-        const int id = threadIdx.x + n * kThreads, y = id / dq, e = 4 * (id % dq);
+        const int id = threadIdx.x + n * FLEX_THREADS, y = id / dq, e = 4 * (id % dq);
         if (y < L.T / 4)
 #pragma unroll
             for (int r = 0; r < 4; ++r)
@@ -801,7 +824,7 @@ __device__ __forceinline__ void store_rows(const Plan& L, int d, const float (&x
     }
 }
 
-template <typename T, bool NS, int ND>
+template <typename T, bool NS, int ND, int NT>
 __global__ void __launch_bounds__(kThreads, 1)
     simt_bwd_kernel(Problem p, Plan L, const T* q, const T* k, const T* v, const float* W1,
                     const float* W2, const float* tau, const T* out, const float* den,
@@ -835,22 +858,22 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (L.wres)
         for (int g = 0; g < L.ng; ++g)
-            stage_projection<NS>(p, L, W1, W2, h, g, sm + L.W + g * gW);
-    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
-    for (int i = tid; i < L.ng * gD; i += kThreads) dW[i] = 0.f;
+            stage_projection<NS, NT>(p, L, W1, W2, h, g, sm + L.W + g * gW);
+    for (int i = tid; i < L.ng * gS; i += FLEX_THREADS) S[i] = 0.f;
+    for (int i = tid; i < L.ng * gD; i += FLEX_THREADS) dW[i] = 0.f;
 
     auto load_kv = [&](int t0, int rows) {
-        load_rows(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
+        load_rows<NT>(k, v, base + (size_t)t0 * d, rows, d, Xk, V, L.pd, L.T);
         unit_weights(L, d, rows, V);
     };
     auto load_qg = [&](int t0, int rows) {
-        load_rows(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
+        load_rows<NT>(q, (const T*)nullptr, base + (size_t)t0 * d, rows, d, Xq, (float*)nullptr, L.pd, L.T);
         load_upstream(p, L, dout, out, den, base + (size_t)t0 * d, den_base + t0, rows, G);
     };
     auto group_W = [&](int g) {  // the group's projection rows, staged now unless resident
         float* W = sm + L.W + g * gW;
         if (!L.wres) {
-            stage_projection<NS>(p, L, W1, W2, h, g, W);
+            stage_projection<NS, NT>(p, L, W1, W2, h, g, W);
             __syncthreads();
         }
         return W;
@@ -890,7 +913,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     store_tile(keys ? Pk : Pq, L.pp, f, pf);
                 }
                 __syncthreads();
-                state_update(L, d, keys ? Pk : Pq, keys ? V : G, S + g * gS);
+                state_update<NT>(L, d, keys ? Pk : Pq, keys ? V : G, S + g * gS);
                 __syncthreads();
             }
         }
@@ -900,11 +923,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!p.causal || L.CL > 1) {
         __syncthreads();
         range_state(true);
-        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
+        if (L.CL > 1) exchange_state<NT>(S, L.ng * gS, L.CL, p.causal ? kPrefix : kTotal);
     }
     __syncthreads();
     for (int c = cb; c < ce; ++c) {
         const int t0 = c * L.T, rows = min(L.T, N - t0);
+        const bool seen = NT || !p.causal || L.CL > 1 || c > cb;  // (else the state is still zero)
         load_qg(t0, rows);
         if (p.causal) load_kv(t0, rows);
         __syncthreads();
@@ -933,7 +957,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (f.on) {
                 zero(dp);
                 if (p.causal) mm_masked(dA, L.pa, f.y, Pk + 4 * f.x, L.pp, dp);
-                mm_nt<4>(G + 4 * f.y * L.pd, L.pd, Sg + f.x * L.pd, L.CT * L.pd, d, dp);
+                if (seen) mm_nt<4>(G + 4 * f.y * L.pd, L.pd, Sg + f.x * L.pd, L.CT * L.pd, d, dp);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const float ci = G[(4 * f.y + r) * L.pd + d];
@@ -944,24 +968,25 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             __syncthreads();
             if (f.on) store_chain<NS>(L, f, dp, pf, qf, Pq);
-            if (p.causal) state_update(L, d, Pk, V, Sg);
+            if (p.causal && (NT || c + 1 < ce)) state_update<NT>(L, d, Pk, V, Sg);
             __syncthreads();
-            project_back<NS, ND>(L, d, Pq, W, Xq, dW + g * gD, dx);
+            project_back<NS, ND, NT>(L, d, Pq, W, Xq, dW + g * gD, dx);
             __syncthreads();
         }
-        store_rows<T, ND>(L, d, dx, dq, base + (size_t)t0 * d, rows);
+        store_rows<T, ND, NT>(L, d, dx, dq, base + (size_t)t0 * d, rows);
     }
 
     // ---- dk, dv: reverse direction with R_j, r_j (S's buffer is reused for R) ----
-    for (int i = tid; i < L.ng * gS; i += kThreads) S[i] = 0.f;
+    for (int i = tid; i < L.ng * gS; i += FLEX_THREADS) S[i] = 0.f;
     __syncthreads();
     if (!p.causal || L.CL > 1) {
         range_state(false);
-        if (L.CL > 1) exchange_state(S, L.ng * gS, L.CL, p.causal ? kSuffix : kTotal);
+        if (L.CL > 1) exchange_state<NT>(S, L.ng * gS, L.CL, p.causal ? kSuffix : kTotal);
         __syncthreads();
     }
     for (int c = ce - 1; c >= cb; --c) {
         const int t0 = c * L.T, rows = min(L.T, N - t0);
+        const bool seen = NT || !p.causal || L.CL > 1 || c < ce - 1;  // (else the state is still zero)
         load_kv(t0, rows);
         if (p.causal) load_qg(t0, rows);
         __syncthreads();
@@ -994,15 +1019,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mm_nt<4>(Pq + 4 * ay * L.pp, L.pp, Pk + ax * L.pp, TT * L.pp, L.F, aa);
 #pragma unroll
             for (int n = 0; n < ND; ++n) {
-                const int id = tid + n * kThreads, y = id / d4, e = 4 * (id % d4);
-                if (y < TT)
+                const int id = tid + n * FLEX_THREADS, y = id / d4, e = 4 * (id % d4);
+                if (seen && y < TT)
                     mm_nn(Pk + 4 * y * L.pp, L.pp, Rg + e, L.CT * L.pd, 2 * L.CT * L.pd,
                           3 * L.CT * L.pd, L.pd, L.F, dvt[n]);
             }
             if (f.on) {
                 zero(dp);
                 if (p.causal) mm_masked_t(dA, L.pa, f.y, Pq + 4 * f.x, L.pp, L.T, dp);
-                mm_nt<4>(V + 4 * f.y * L.pd, L.pd, Rg + f.x * L.pd, L.CT * L.pd, d, dp);
+                if (seen) mm_nt<4>(V + 4 * f.y * L.pd, L.pd, Rg + f.x * L.pd, L.CT * L.pd, d, dp);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const float wj = V[(4 * f.y + r) * L.pd + d];
@@ -1015,9 +1040,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             __syncthreads();
             if (f.on) store_chain<NS>(L, f, dp, pf, qf, Pk);
-            if (p.causal) state_update(L, d, Pq, G, Rg);
+            if (p.causal && (NT || c > cb)) state_update<NT>(L, d, Pq, G, Rg);
             __syncthreads();
-            project_back<NS, ND>(L, d, Pk, W, Xk, dW + g * gD, dx);
+            project_back<NS, ND, NT>(L, d, Pk, W, Xk, dW + g * gD, dx);
             __syncthreads();
         }
         if (p.causal && a_on)
@@ -1043,7 +1068,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll
         for (int n = 0; n < ND; ++n) {
-            const int id = tid + n * kThreads, y = id / d4, e = 4 * (id % d4);
+            const int id = tid + n * FLEX_THREADS, y = id / d4, e = 4 * (id % d4);
             if (y < TT) {
                 if (p.causal) mm_masked_t(A, L.pa, y, G + e, L.pd, L.T, dvt[n]);
                 if (tau)
@@ -1059,8 +1084,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
             }
         }
-        store_rows<T, ND>(L, d, dvt, dv, base + (size_t)t0 * d, rows);
-        store_rows<T, ND>(L, d, dx, dk, base + (size_t)t0 * d, rows);
+        store_rows<T, ND, NT>(L, d, dvt, dv, base + (size_t)t0 * d, rows);
+        store_rows<T, ND, NT>(L, d, dx, dk, base + (size_t)t0 * d, rows);
         __syncthreads();
     }
 
@@ -1071,7 +1096,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();
         if (tid == 0) {
             float t = 0.f;
-            for (int w = 0; w < kThreads / 32; ++w) t += red[w];
+            for (int w = 0; w < FLEX_THREADS / 32; ++w) t += red[w];
             red[kMaxT] = t;
         }
     }
@@ -1082,7 +1107,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int Mc = NS ? 2 * p.M : p.M;
     float* part = dw_part + (size_t)bh * Mc * d;
     const uint32_t dw_addr = tc::smem_u32(dW);
-    for (int i = rank * kThreads + tid; i < L.ng * gD / 4; i += L.CL * kThreads) {
+    for (int i = rank * FLEX_THREADS + tid; i < L.ng * gD / 4; i += L.CL * FLEX_THREADS) {
         const int row = 4 * i / d, e = 4 * i % d, g = row / L.KP, kk = row % L.KP;
         const int fr = g * L.MG + (NS ? 2 * (kk >> 2) + ((kk >> 1) & 1) : kk);
         if (fr >= p.M) continue;
@@ -1231,11 +1256,12 @@ bool fits_bwd(const Problem& p)
 
 // The plan for groups of at most mg frequencies and T tokens per chunk, with or without
 // resident projection rows.
-Plan layout(const Problem& p, bool bwd, int mg, int T, bool wres)
+Plan layout(const Problem& p, bool bwd, int mg, int T, bool wres, int nt = kThreads)
 {
     Plan L = {};
     L.T = T;
     L.lpr = T > 64 ? 2 : 4;
+    L.nt = nt;
     L.wres = wres;
     L.CL = 1;
     L.ng = (p.M + mg - 1) / mg;
@@ -1245,7 +1271,7 @@ Plan layout(const Problem& p, bool bwd, int mg, int T, bool wres)
     L.KP = p.nonstat ? 2 * L.MG : L.MG;
     L.pd = p.d + 4;
     L.pp = L.F + 4;
-    L.pa = std::max(T, 16) + 4;
+    L.pa = (std::max(T, L.CT) + 3) / 4 * 4 + 4;  // (also the backward's s_j partials, CT a row)
     int o = 0;
     auto take = [&](int n) {
         const int at = o;
@@ -1289,6 +1315,29 @@ bool make_plan(const Problem& p, bool bwd, Plan* plan)
         *plan = layout(p, bwd, kMaxMG, 128, true);
         found = 2 * ((size_t)plan->total * 4 + 1024) <= 228 * 1024;
     }
+    // Short sequences: a chunk no longer than needed and groups as large as its threads take (the
+    // groups run one after the other); more sequences than run at once (two CTAs an SM) take no
+    // more threads than have a tile.  The kernels before these (one output a thread), chunks of
+    // 64, this: forward n non-causal N16 d64 M64, 64 sequences 41, 31, 19 us, 2048 sequences 519,
+    // 391, 154; d16 M256, 64 sequences 47, 60, 29.  At N 1 still up to 1.5 times the kernels before
+    // (d16 M256: 19, 60, 28; d32 M32, 2048 sequences: 33, 107, 41), backwards at most even.
+    const bool many = p.d <= 64 && (long long)p.B * p.H > 2 * 152;
+    if (!found && p.N <= 32) {
+        const int T = p.N <= 16 ? 16 : 32, mg = 8 * kThreads / T;
+        const int ct = layout(p, bwd, mg, T, true).CT;
+        int nt = 4 * T;
+        while (nt < kThreads && (!many || nt < T / 4 * std::max(ct, p.d / 4))) nt *= 2;
+        *plan = layout(p, bwd, mg, T, true, nt);
+        found = (size_t)plan->total <= kSmemFloats;
+    }
+    // Many sequences of small heads: half the threads of a 64-token chunk would have no tile.
+    // Forward n, N65 d16 M16, 1024 sequences, the same three: causal 76, 97, 58 us, not 58, 72, 54.
+    // (d4 M4, N200, 2048 sequences, not causal: 91, 193, 179.)
+    if (!found && many && tiles <= kThreads / 2) {
+        *plan = layout(p, bwd, kMaxMG, 32, true, 128);
+        found = true;  // (a 64-token chunk fits)
+    }
+    plan->any = found && plan->T < 64;
     for (int mg = kMaxMG; mg >= 4 && !found; mg /= 2)  // smaller groups: the largest shapes only
         for (int T = 64; T >= 8 && !found; T /= 2)
             for (int wres = 1; wres >= 0 && !found; --wres) {
@@ -1330,7 +1379,7 @@ cudaError_t launch_plan(void (*kern)(KArgs...), const Problem& p, const Plan& L,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((long long)p.B * p.H * L.CL));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)L.nt);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1348,7 +1397,9 @@ cudaError_t launch_fwd_t(const Problem& p, const Plan& L, const void* q, const v
                          const void* v, const float* W1, const float* W2, const float* tau,
                          void* out, float* den, cudaStream_t s)
 {
-    auto kern = p.d > 64 ? simt_fwd_kernel<T, NS, 2> : simt_fwd_kernel<T, NS, 1>;
+    auto kern = L.any ? simt_fwd_kernel<T, NS, 2, 0>
+                : p.d > 64 ? simt_fwd_kernel<T, NS, 2, kThreads>
+                           : simt_fwd_kernel<T, NS, 1, kThreads>;
     return launch_plan(kern, p, L, s, (const T*)q, (const T*)k, (const T*)v, W1, W2, tau, (T*)out,
                        den);
 }
@@ -1359,7 +1410,9 @@ cudaError_t launch_bwd_t(const Problem& p, const Plan& L, const void* q, const v
                          const void* out, const float* den, const void* dout, void* dq, void* dk,
                          void* dv, float* part, float* tpart, cudaStream_t s)
 {
-    auto kern = p.d > 64 ? simt_bwd_kernel<T, NS, 2> : simt_bwd_kernel<T, NS, 1>;
+    auto kern = L.any ? simt_bwd_kernel<T, NS, 2, 0>
+                : p.d > 64 ? simt_bwd_kernel<T, NS, 2, kThreads>
+                           : simt_bwd_kernel<T, NS, 1, kThreads>;
     return launch_plan(kern, p, L, s, (const T*)q, (const T*)k, (const T*)v, W1, W2, tau,
                        (const T*)out, den, (const T*)dout, (T*)dq, (T*)dk, (T*)dv, part, tpart);
 }

@@ -8,8 +8,9 @@ from paper_2606_27748_gb300 import build, flexattn
 
 pytestmark = pytest.mark.gpu
 
-# (dtype, B, H, N, d, M): one CTA and several ranges a sequence, one and two frequency groups
-SHAPES = [("f32", 1, 2, 50, 32, 32), ("f32", 1, 2, 300, 32, 16), ("f32", 1, 1, 200, 64, 64),
+# (dtype, B, H, N, d, M): one CTA and several ranges a sequence, one and two frequency groups, the
+# plans of short sequences and of many small ones
+SHAPES = [("f32", 1, 2, 50, 32, 32), ("f32", 1, 2, 20, 32, 100), ("f32", 39, 8, 70, 16, 16), ("f32", 1, 2, 300, 32, 16), ("f32", 1, 1, 200, 64, 64),
           ("f32", 1, 1, 90, 128, 24), ("bf16", 1, 2, 150, 32, 16)]
 
 
