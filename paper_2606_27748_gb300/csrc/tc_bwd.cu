@@ -124,7 +124,7 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
 template <bool NS, bool KW, int CS, int MODE, int PASS>
 __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUtensorMap& tmap_k,
     const CUtensorMap& tmap_v, const CUtensorMap& tmap_do, const CUtensorMap& tmap_o, int H,
-    int N, int M, int G, int causal, const __nv_bfloat16* __restrict__ q,
+    int N, int M, int G, const __nv_bfloat16* __restrict__ q,
     const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
     const float* __restrict__ W1, const float* __restrict__ W2,
     const __nv_bfloat16* __restrict__ outp, const float* __restrict__ den,
@@ -137,7 +137,7 @@ __device__ __forceinline__ void tc_bwd_body(const CUtensorMap& tmap_q, const CUt
     using L = BwCfg<NS>;
     // blocks [0, half): pass R, [half, 2 half): pass F, half = units * nsplit; within a pass
     // idx = (sequence * nsplit + split) * G + group (the groups of a cluster adjacent); the
-    // chunks are split into nsplit ranges (non-causal modes; 1 for the causal scans).
+    // chunks are split into nsplit ranges (causal scans: 1 unless a small batch is cut).
     // Partial slots are indexed by slot = pass * half + idx.
     const int half_grid = units * nsplit;
     const int idx = (int)blockIdx.x % half_grid;
@@ -1277,7 +1277,7 @@ __global__ void __launch_bounds__(kThreadsB, 1)
                   const __grid_constant__ CUtensorMap tmap_k,
                   const __grid_constant__ CUtensorMap tmap_v,
                   const __grid_constant__ CUtensorMap tmap_do,
-                  const __grid_constant__ CUtensorMap tmap_o, int H, int N, int M, int G, int causal,
+                  const __grid_constant__ CUtensorMap tmap_o, int H, int N, int M, int G,
                   const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                   const float* __restrict__ W1, const float* __restrict__ W2,
@@ -1292,12 +1292,12 @@ __global__ void __launch_bounds__(kThreadsB, 1)
 {
     if ((int)blockIdx.x < units * nsplit)
         tc_bwd_body<NS, KW, CS, MODE, kPassR>(
-            tmap_q, tmap_k, tmap_v, tmap_do, tmap_o, H, N, M, G, causal, q, k, v, W1, W2,
+            tmap_q, tmap_k, tmap_v, tmap_do, tmap_o, H, N, M, G, q, k, v, W1, W2,
             outp, den, dout, dq, dk, dv, dw_part, kw, tau, dtau_part, units, nsplit,
             state_part, state_total, status);
     else
         tc_bwd_body<NS, KW, CS, MODE, kPassF>(
-            tmap_q, tmap_k, tmap_v, tmap_do, tmap_o, H, N, M, G, causal, q, k, v, W1, W2,
+            tmap_q, tmap_k, tmap_v, tmap_do, tmap_o, H, N, M, G, q, k, v, W1, W2,
             outp, den, dout, dq, dk, dv, dw_part, kw, tau, dtau_part, units, nsplit,
             state_part, state_total, status);
 }
@@ -1516,7 +1516,7 @@ cudaError_t launch_mode(const Problem& p, const BwdArgs& m, const void* q, const
     // (the first kernel of a call, without key weights, starts in stream order)
     const bool after = KW || MODE == kGrad || (MODE == kCausal && nsplit > 1);
     return launch_after(kb, dim3((unsigned)(2 * units * nsplit)), kThreadsB, smem, CS, after, s, m.mq, m.mk,
-                        m.mv, m.mdo, m.mo, p.H, p.N, p.M, p.M / 64, p.causal, (CB)q, (CB)k, (CB)v, W1,
+                        m.mv, m.mdo, m.mo, p.H, p.N, p.M, p.M / 64, (CB)q, (CB)k, (CB)v, W1,
                         W2, (CB)out, den, (CB)dout, (B16)dq, (B16)dk, (B16)dv, f + w.part,
                         KW ? (const float*)(f + w.kw) : (const float*)nullptr, tau, f + w.dtau, units,
                         nsplit, f + w.state_part, (const float*)(f + w.state_total), status);

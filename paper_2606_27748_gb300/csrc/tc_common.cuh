@@ -108,20 +108,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint6
         : "memory");
 }
 
-// D[tmem] (+)= A[tmem] x B[smem]: A (M rows = lanes, bf16 packed two K elements per
-// 32-bit column, low half = even K index) read from tensor memory.
-__device__ __forceinline__ void mma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem,
-                                                uint64_t b_desc, uint32_t idesc,
-                                                uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // Arrive once on the mbarrier when every tcgen05 operation issued so far by this thread
 // has completed.
 __device__ __forceinline__ void mma_commit(void* mbar)
@@ -160,6 +146,8 @@ __device__ __forceinline__ void wmma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
         : "memory");
 }
 
+// A (M rows = lanes, bf16 packed two K elements per 32-bit column, low half = even K index) read
+// from tensor memory.
 __device__ __forceinline__ void wmma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                                  uint32_t idesc, uint32_t accumulate)
 {
