@@ -307,7 +307,10 @@ __global__ void __launch_bounds__(256)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 0) tmem_dealloc(tm, P);
+    if (warp == 0) {
+        drain_after_abort(!ok);
+        tmem_dealloc(tm, P);
+    }
 }
 
 template <typename T>

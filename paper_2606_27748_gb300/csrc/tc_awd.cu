@@ -271,7 +271,10 @@ __global__ void __launch_bounds__(kThreadsA, 1)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 0) tmem_dealloc(tm, 256);
+    if (warp == 0) {
+        drain_after_abort(!ok);
+        tmem_dealloc(tm, 256);
+    }
 }
 
 __global__ void awd_reduce_kernel(int BH, int nqb, int N, const float* part,
@@ -728,11 +731,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
 
 done:
     __syncthreads();
-    if (abort_flag && tid == 0) {  // gave up: let copies into this CTA's shared memory land
-        const long long t0 = clock64();
-        while (clock64() - t0 < kDrainCycles) {
-        }
-    }
+    if (tid == 0) drain_after_abort(abort_flag != 0);
     // dtau partial of this CTA, summed in a fixed order
     float dsum = dtau_acc;
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);

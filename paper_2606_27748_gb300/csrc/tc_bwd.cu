@@ -1258,11 +1258,7 @@ done:
             dtau_part[slot] = sum;
         }
     }
-    if (abort_flag && tid == 0) {  // gave up: let copies into this CTA's shared memory land
-        const long long t0 = clock64();
-        while (clock64() - t0 < kDrainCycles) {
-        }
-    }
+    if (tid == 0) drain_after_abort(abort_flag != 0);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();

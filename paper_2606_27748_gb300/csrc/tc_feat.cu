@@ -160,7 +160,10 @@ __global__ void __launch_bounds__(kThreadsF)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 0) tmem_dealloc(tm, NCOLS);
+    if (warp == 0) {
+        drain_after_abort(!ok);
+        tmem_dealloc(tm, NCOLS);
+    }
     if (!rowscale) grid_dep_wait();  // so that a kernel that waits for this one has both
 }
 

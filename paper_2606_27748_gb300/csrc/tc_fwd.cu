@@ -725,7 +725,10 @@ __global__ void __launch_bounds__(Cfg<NS, CS>::THREADS, 1)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == kWarpMMA) tmem_dealloc(tm, 512);
+    if (warp == kWarpMMA) {
+        drain_after_abort(abort_flag != 0);
+        tmem_dealloc(tm, 512);
+    }
     if (CS > 1) cluster_sync();  // no CTA leaves while its partner may still write to it
 }
 

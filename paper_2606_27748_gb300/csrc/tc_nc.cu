@@ -397,7 +397,10 @@ __global__ void __launch_bounds__(kThreadsNC, 1)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == kWarpMMA) tmem_dealloc(tm, 512);
+    if (warp == kWarpMMA) {
+        drain_after_abort(abort_flag != 0);
+        tmem_dealloc(tm, 512);
+    }
 }
 
 // Sums of a sequence's partials in split order, rounded to bf16 and laid out as the output

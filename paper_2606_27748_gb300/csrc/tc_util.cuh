@@ -183,9 +183,16 @@ __device__ __forceinline__ void diagnostic_stall(uint64_t* bar, volatile int* ab
     if (cycles > 0) bar_wait(bar, 0, abort_flag, status, cycles);
 }
 
-// On the way out after an abort: clocks that a CTA waits so that no copy into its shared memory is
-// still in flight when it exits.
+// On the way out after an abort (and a CTA barrier): waits so that no copy into the CTA's shared
+// memory is still in flight when it exits.
 constexpr long long kDrainCycles = 20000000LL;  // ~10 ms
+__device__ __forceinline__ void drain_after_abort(bool aborted)
+{
+    if (!aborted) return;
+    const long long t0 = clock64();
+    while (clock64() - t0 < kDrainCycles) {
+    }
+}
 
 // bar_wait for a barrier that other CTAs of the cluster arrive on (acquire at cluster scope).
 __device__ __forceinline__ bool bar_wait_cluster(uint64_t* bar, uint32_t parity,
