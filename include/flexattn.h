@@ -72,13 +72,14 @@ const char* flex_strerror(int status);
 /* Workspace bytes of flex_linattn_fwd (backward = 0) or flex_linattn_bwd (backward = 1) for
  * this shape; 0 if the shape is invalid or unsupported.  (The causal backward of a small
  * batch uses part of it to run each sequence in ranges; it accepts a smaller workspace that
- * holds the uncut form's scratch and is slower with it.) */
+ * holds the uncut form's scratch, is slower with it, and adds up in another order: results
+ * repeat bit for bit with workspaces of one size, not between the two forms.) */
 size_t flex_workspace_bytes(const flex_shape* shape, int causal, int backward);
 
 /* Feature map phi of Eq. phi_n (W2 == NULL) or Eq. phi_non (W2 != NULL), written out.
  * x: [B][H][N][d], phi: [B][H][N][2M], both in shape->dtype, scaled by M^{-1/2}.  bf16
- * with d = 64 and M in {64, 128} projects on the tensor cores (frequencies rounded to
- * bf16); other shapes use fp32 CUDA-core arithmetic.  This and flex_awd_loss are the only
+ * with d = 64 and M in {64, 128} projects on the tensor cores (frequencies as bf16 high
+ * and low parts); other shapes use fp32 CUDA-core arithmetic.  This and flex_awd_loss are the only
  * entry points that write phi to memory; the attention entry points keep it on chip. */
 int flex_featmap(const flex_shape* shape, const void* x, const float* W1, const float* W2,
                  void* phi, void* stream);

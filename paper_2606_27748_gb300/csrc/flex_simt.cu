@@ -115,8 +115,9 @@ __global__ void featmap_kernel(Problem p, const T* x, const float* W1, const flo
 // up to 8 SMs instead of one.  Measured on GB300 against one CTA per sequence with
 // one output per thread: forward f32 s B1 H1 N256 d32 M32 132 -> 16 us, bf16 n B32 H4
 // N1024 d32 M16 477 -> 73 us; forward and backward f32 n tau B4 H4 N1000 d64 M64
-// 8.58 -> 0.33 ms (10 of the 78 TFLOP/s fp32 peak: per chunk the products run between
-// barriers with one backward CTA per SM, so load latency and the barriers bound it).
+// 8.58 -> 0.33 ms (10 of the 78 TFLOP/s fp32 peak: 96 of 152 SMs, and there per chunk the
+// products run between barriers, one backward CTA per SM: issue slots 43% and the fma pipe
+// 32% busy over all SMs, the rest shared-memory latency, barriers and instruction fetch).
 struct Plan {
     int T;              // tokens per chunk (a multiple of 8, at most kMaxT)
     int lpr;            // lanes per row in row-wise sums: 4, or 2 with 128 tokens
@@ -375,7 +376,8 @@ struct Place {
 // (Cody and Waite: the fp32 values of pi/2 and of the two remainders, each step one fma), then
 // polynomials on [-pi/4, pi/4], sin r = r + r y (s0 + s1 y + s2 y^2) and
 // cos r = 1 + y (-1/2 + y (c0 + c1 y + c2 y^2)) with y = r^2, fitted here by least squares on
-// 4000 Chebyshev nodes refined by Lawson's iteration (approximation error 2e-9 and 1e-10).
+// 4000 Chebyshev nodes refined by Lawson's iteration (approximation error of these, in fp32,
+// 2.3e-9 and 5.1e-10).
 // Max error against fp64 over |x| <= 10^4: 7.1e-8 (rms 1.7e-8; rounding the exact value:
 // 1.5e-8), as the CUDA library's sincosf, which larger arguments take.  About 15 instructions
 // an argument instead of 45; inlined library calls also overflowed the instruction cache.

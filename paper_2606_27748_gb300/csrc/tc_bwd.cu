@@ -45,7 +45,7 @@
 //   kGrad F    [q projection, dphi(q)] / chain rule, next chunk's g / [dq, dW] / dq rows
 //   kGrad R    [k projection, dphi(k)] / phi(k), chain rule / [dv, dk, dW] / dv, dk rows
 // The phases of a chunk depend on one another (an SM holds one CTA's tensor memory), so the
-// length of this chain bounds the kernel, not DRAM (7%) or the tensor pipe: a chunk of s M128
+// length of this chain bounds the kernel, not DRAM (14%) or the tensor pipe (18%): a chunk of s M128
 // takes about 15 us in F and R together, from 19.4 with all threads meeting at CTA barriers
 // and thread 0 issuing; measured forward and backward: s B8 H12 N8192 M128 2.16 -> 1.57 ms,
 // n non-causal B32 H8 N4000 M64 1.30 -> 0.89 ms.
